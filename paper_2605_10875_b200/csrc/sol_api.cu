@@ -290,6 +290,7 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
   dn.t = cs.t_op;
   dn.t_f32 = cs.t;
   dn.keep = cs.keep;
+  dn.p_permille = p_permille;
   dn.w = w_down;
   dn.live = cs.live;
   dn.M = B;

@@ -440,11 +440,12 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_down_kernel(const DownDev 
 // At batch <= 8 the union of the channels that some token keeps is well below d_ff when tokens are pruned, and a
 // 64-channel block is almost never dead as a whole: this kernel reads W_down channel by channel and skips
 // every channel that no token keeps, so the bytes follow the union of kept rows.  CTA = (128 output columns,
-// range of channels) as in umma_down; a warp takes groups of 32 channels of the range, finds the kept ones with
-// one ballot, reads each kept channel's 256 bytes of the slab (two 128-byte pieces of the packed layout, one per
-// column half) and multiplies them into float32 accumulators (<= 8 tokens x 4 columns per lane) on the FMA
-// pipes; the warps are merged through shared memory.
-constexpr int DR_WARPS = 8;
+// range of channels) as in umma_down.
+//
+// Bound by the bytes in flight.  A warp takes groups of 32 channels of the range, finds the kept ones with one
+// ballot and packs their numbers and t values into a table of its own; then it requests them sixteen at a time, two
+// channels per 16-byte load of the warp (lanes 0-15 and 16-31; eight lanes per 128-byte half of a channel's 256
+// XX of a warp and then the warps are added up in a fixed order.
 constexpr int DR_MAXB = 8;
 
 struct DownRowsDev {
@@ -452,35 +453,59 @@ struct DownRowsDev {
   const unsigned char* w;     // packed W_down_t
   const float* t;             // [M][ff] silu(g) u before masking
   const unsigned char* keep;  // [M][ff] 1 = kept
+  const int32_t* p_permille;  // [M] prune rates
   float* partial;             // [chunks][Mpad][d]
 };
 
-__global__ void __launch_bounds__(DR_WARPS * 32) down_rows_kernel(const DownRowsDev p) {
-  __shared__ float red[DR_WARPS][DR_MAXB][128];
+// MB: tokens the registers are laid out for (>= M).  Few tokens leave room for 32 warps, more need 16.
+template <int MB>
+struct DownRowsCfg {
+  static constexpr int WARPS = MB <= 2 ? 32 : 16;
+  static constexpr int TAB_WORDS = 32 * (1 + MB);  // per warp: kept channels of the group, their t of every token
+  static constexpr int SMEM = WARPS * (TAB_WORDS + MB * 128) * 4;
+};
+
+template <int MB>
+__global__ void __launch_bounds__(DownRowsCfg<MB>::WARPS * 32, 1) down_rows_kernel(const DownRowsDev p) {
+  using C = DownRowsCfg<MB>;
+  extern __shared__ __align__(16) unsigned char dr_smem[];
   const int slab = blockIdx.x, chunk = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* red = reinterpret_cast<float*>(dr_smem);  // [WARPS][MB][128]
+  int* tab = reinterpret_cast<int*>(dr_smem + C::WARPS * MB * 512) + warp * C::TAB_WORDS;
+  float* tab_t = reinterpret_cast<float*>(tab + 32);  // [32][MB]
   const int jblocks = (p.ff + 63) / 64;
   const int j0 = (int)(((long long)p.ff * chunk) / p.chunks), j1 = (int)(((long long)p.ff * (chunk + 1)) / p.chunks);
+  const int sub = lane >> 4, half = (lane >> 3) & 1, q = lane & 7;  // channel of a pair, 64-column half, 16-byte piece
+  const unsigned char* w_slab = p.w + (size_t)slab * jblocks * UM_TILE_SPAN + half * 8192;
   pdl_trigger();
+  // A token that prunes nothing needs every channel, whatever the selection says: the weights of this warp's
+  // first group then start towards L2 while the kernels before are still running.
+  bool dense = false;
+#pragma unroll
+  for (int m = 0; m < MB; ++m)
+    if (m < p.M) dense = dense || p.p_permille[m] <= 0;
+  if (dense) {
+    const int j = j0 + warp * 32 + lane;
+    if (j < j1) {
+      const unsigned char* row = p.w + ((size_t)slab * jblocks + (j >> 6)) * UM_TILE_SPAN + (j & 63) * 128;
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(row));
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(row + 8192));
+    }
+  }
   pdl_wait();
-  float acc[DR_MAXB][4];
+  uint64_t acc[MB][4];  // pairs of columns
 #pragma unroll
-  for (int m = 0; m < DR_MAXB; ++m)
+  for (int m = 0; m < MB; ++m)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[m][c] = 0.f;
-  // A warp takes groups of 32 consecutive channels of the CTA's range.  Lane l first looks channel l of the group
-  // up in the tokens' keep masks and fetches the tokens' t for it (one round trip, all loads independent); the
-  // channels that some token keeps are then taken eight at a time: their weight pieces are requested together
-  // (256 bytes per channel, coalesced), the tokens' t come from the owning lane by a shuffle.  Looking one
-  // channel up after the other put three dependent round trips in front of every four channels (66 us for
-  // the whole matrix at batch 1).
+    for (int c = 0; c < 4; ++c) acc[m][c] = 0ull;
 #pragma unroll 1
-  for (int g0 = j0 + warp * 32; g0 < j1; g0 += DR_WARPS * 32) {
+  for (int g0 = j0 + warp * 32; g0 < j1; g0 += C::WARPS * 32) {
     const int jl = g0 + lane;
-    float tl[DR_MAXB];
+    float tl[MB];
     bool mine = false;
 #pragma unroll
-    for (int m = 0; m < DR_MAXB; ++m) {
+    for (int m = 0; m < MB; ++m) {
       tl[m] = 0.f;
       if (jl < j1 && m < p.M) {
         const bool k = p.keep[(size_t)m * p.ff + jl] != 0;
@@ -489,56 +514,74 @@ __global__ void __launch_bounds__(DR_WARPS * 32) down_rows_kernel(const DownRows
         mine = mine || k;
       }
     }
-    unsigned todo = __ballot_sync(0xffffffffu, mine);
-    while (todo) {  // warp-uniform
-      int ch[8];
-      uint32_t wv[8][2];
+    const unsigned todo = __ballot_sync(0xffffffffu, mine);
+    const int n = __popc(todo);
+    __syncwarp();  // the table of the group before is not read any more
+    if (mine) {
+      const int at = __popc(todo & ((1u << lane) - 1u));
+      tab[at] = jl;
+#pragma unroll
+      for (int m = 0; m < MB; ++m) tab_t[at * MB + m] = tl[m];
+    }
+    __syncwarp();
+#pragma unroll 1
+    for (int u0 = 0; u0 < n; u0 += 16) {  // warp-uniform
+      uint4 wv[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        ch[u] = -1;
-        wv[u][0] = wv[u][1] = 0u;
-        if (todo) {
-          ch[u] = __ffs(todo) - 1;
-          todo &= todo - 1;
-          // channel j of the slab: block j / 64, row c = j % 64; lane l holds columns 2 l, 2 l + 1 of each 64-column half
-          const int j = g0 + ch[u], c = j & 63;
-          const unsigned char* base = p.w + ((size_t)slab * jblocks + (j >> 6)) * UM_TILE_SPAN + c * 128 +
-                                      (((lane >> 2) ^ (c & 7)) * 16) + (lane & 3) * 4;
-          wv[u][0] = *reinterpret_cast<const uint32_t*>(base);
-          wv[u][1] = *reinterpret_cast<const uint32_t*>(base + 8192);
+        const int at = u0 + 2 * u + sub;
+        wv[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (at < n) {
+          const int j = tab[at], c = j & 63;
+          wv[u] = *reinterpret_cast<const uint4*>(w_slab + (size_t)(j >> 6) * UM_TILE_SPAN + c * 128 + ((q ^ (c & 7)) * 16));
         }
       }
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
-        if (ch[u] < 0) continue;  // warp-uniform
-        const float w0 = bf16_lo(wv[u][0]), w1 = bf16_hi(wv[u][0]), w2 = bf16_lo(wv[u][1]), w3 = bf16_hi(wv[u][1]);
+        if (u0 + 2 * u >= n) break;  // warp-uniform
+        const int at = min(u0 + 2 * u + sub, n - 1);  // an absent second channel has zero weights
+        const uint64_t w[4] = {f32x2(bf16_lo(wv[u].x), bf16_hi(wv[u].x)), f32x2(bf16_lo(wv[u].y), bf16_hi(wv[u].y)),
+                               f32x2(bf16_lo(wv[u].z), bf16_hi(wv[u].z)), f32x2(bf16_lo(wv[u].w), bf16_hi(wv[u].w))};
 #pragma unroll
-        for (int m = 0; m < DR_MAXB; ++m) {
-          const float tv = __shfl_sync(0xffffffffu, tl[m], ch[u]);
-          acc[m][0] = fmaf(tv, w0, acc[m][0]);
-          acc[m][1] = fmaf(tv, w1, acc[m][1]);
-          acc[m][2] = fmaf(tv, w2, acc[m][2]);
-          acc[m][3] = fmaf(tv, w3, acc[m][3]);
+        for (int m = 0; m < MB; ++m) {
+          const float tv = tab_t[at * MB + m];
+          const uint64_t tt = f32x2(tv, tv);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[m][c] = fma_f32x2(tt, w[c], acc[m][c]);
         }
       }
     }
   }
-  // columns of the slab held by lane l: 2 l, 2 l + 1 (first half), 64 + 2 l, 64 + 2 l + 1 (second half)
+  // the two channels of a pair, then the warps: columns half * 64 + 8 q ..
 #pragma unroll
-  for (int m = 0; m < DR_MAXB; ++m) {
-    red[warp][m][2 * lane] = acc[m][0];
-    red[warp][m][2 * lane + 1] = acc[m][1];
-    red[warp][m][64 + 2 * lane] = acc[m][2];
-    red[warp][m][64 + 2 * lane + 1] = acc[m][3];
+  for (int m = 0; m < MB; ++m) {
+    float a[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+      a[c] = __uint_as_float((uint32_t)(acc[m][c >> 1] >> (32 * (c & 1))));
+      a[c] += __shfl_xor_sync(0xffffffffu, a[c], 16);
+    }
+    if (sub == 0) {
+      float4* dst = reinterpret_cast<float4*>(red + (warp * MB + m) * 128 + half * 64 + q * 8);
+      dst[0] = make_float4(a[0], a[1], a[2], a[3]);
+      dst[1] = make_float4(a[4], a[5], a[6], a[7]);
+    }
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < p.M * 128; i += DR_WARPS * 32) {
+  for (int i = threadIdx.x; i < p.M * 128; i += C::WARPS * 32) {
     const int m = i >> 7, c = i & 127;
     float a = 0.f;
 #pragma unroll
-    for (int w = 0; w < DR_WARPS; ++w) a += red[w][m][c];
+    for (int w = 0; w < C::WARPS; ++w) a += red[w * MB * 128 + i];
     p.partial[((size_t)chunk * p.Mpad + m) * p.d + slab * 128 + c] = a;
   }
+}
+
+template <int MB>
+static void launch_down_rows(const DownRowsDev& r, cudaStream_t st) {
+  using C = DownRowsCfg<MB>;
+  ensure_dynamic_smem(reinterpret_cast<const void*>(&down_rows_kernel<MB>), C::SMEM);
+  SOL_LAUNCH("gemm_down_gathered", down_rows_kernel<MB>, dim3(r.d / 128, r.chunks), dim3(C::WARPS * 32), C::SMEM, st, r);
 }
 
 // ============================================================================
@@ -680,8 +723,12 @@ void launch_gemm_down(const GemmDown& g, cudaStream_t st) {
   if (g.M <= DR_MAXB && g.t_f32 != nullptr && g.keep != nullptr) {  // small batch: channel by channel, only kept rows
     DownRowsDev r;
     r.M = g.M; r.Mpad = pad_rows(g.M); r.ff = g.ff; r.d = g.d; r.chunks = g.chunks;
-    r.w = static_cast<const unsigned char*>(g.w); r.t = g.t_f32; r.keep = g.keep; r.partial = g.partial;
-    SOL_LAUNCH("gemm_down_gathered", down_rows_kernel, dim3(g.d / 128, g.chunks), dim3(DR_WARPS * 32), 0, st, r);
+    r.w = static_cast<const unsigned char*>(g.w); r.t = g.t_f32; r.keep = g.keep; r.p_permille = g.p_permille; r.partial = g.partial;
+    if (g.M == 1) launch_down_rows<1>(r, st);
+    else if (g.M == 2) launch_down_rows<2>(r, st);
+    else if (g.M == 3) launch_down_rows<3>(r, st);
+    else if (g.M == 4) launch_down_rows<4>(r, st);
+    else launch_down_rows<8>(r, st);
     return;
   }
   DownDev d;
