@@ -195,22 +195,16 @@ void launch_reduce_out(const float* partial, int chunks, int M, int Mpad, int d,
 void launch_pack_weights(const sol_shape_t& s, int kind, const void* src0, const void* src1, void* dst, cudaStream_t st);
 
 // ---- attention (sol_attn.cu) ------------------------------------------------
-// Kept tokens per pass-2 chunk: 32 KB of V rows.
+// Tokens of a row per slot of the partial results.
 inline int attn_split_len(int head_dim) { return head_dim == 64 ? 256 : 128; }
 inline int attn_splits(int head_dim, int max_pages, int page_size) {
   const int len = attn_split_len(head_dim);
   const int s = (max_pages * page_size + len - 1) / len;
   return s < 1 ? 1 : s;
 }
-// CTAs per row of the token selection: one per 2048 tokens.
-inline int attn_select_segs(int max_pages, int page_size) {
-  const int s = (max_pages * page_size + 2047) / 2048;
-  return s < 1 ? 1 : s;
-}
-constexpr int ATTN_ITEM_CHUNKS = 64;  // chunks of attn_split_len kept tokens per pass-2 work item at most
 constexpr int PAGE = 64;  // tokens of a cache page
 // words of AttnArgs::work_ctr
-enum : int { WC_ITEMS = 0, WC_NEXT = 1, WC_CPI = 2, WC_DONE = 4 };
+enum : int { WC_NEXT = 1, WC_CPI = 2, WC_DONE = 4 };
 
 struct AttnArgs {
   sol_shape_t shape;
@@ -232,20 +226,15 @@ struct AttnArgs {
   float* sigma;         // [B][Hkv][Tmax]
   uint32_t* row_hist;   // [B][Hkv][4096] histogram of a row's scores (rows that span several selection CTAs)
   uint32_t* row_ctl;    // [B][Hkv][8] selection state of a row
-  uint32_t* seg_pub;    // [B][Hkv][segments] kept count of each 2048-token segment of the row (| ready bit)
-  int32_t* cand_idx;    // [B][Hkv][1024] tokens between the selection's edges
-  float* cand_val;      // [B][Hkv][1024] their scores
-  int32_t* list_idx;    // [B][Hkv][Tmax] token index of every kept token, in the order pass 2 reads them
+  int32_t* list_idx;    // Quest mode: [B][Hkv][Tmax] token index of every listed token
   int32_t* kept_idx_out; // optional: the caller's [B][Hkv][Tmax] array for the ascending index list
   int32_t* kept_cnt;    // [B][Hkv]
-  uint32_t* kept_row;   // same layout as kept_idx: cache row (page table applied) of every kept token,
-                        // 0xffffffff: bad page
+  uint32_t* kept_row;   // Quest mode: same layout, cache row (page table applied) of every listed token, 0xffffffff: bad page
   float* part;          // [B][Hkv][S][G][hd + 2]
   int splits;           // S = ceil(Tmax / attn_split_len(hd))
-  int32_t* plan;        // [3][132] cumulative page / segment counts over the batch: the flat work lists of pass 1 and
-                        // of the selection, written by the query preparation
-  int32_t* work_items;  // [B*Hkv*S][2] pass-2 work list (item code, kept count), filled by the selection
-  int32_t* work_ctr;    // [4 + B*Hkv]: items emitted, next item to claim, chunks per item, unused; then the finished
+  int32_t* plan;        // [2][132] cumulative segment / item counts over the batch: the flat work lists of the selection
+                        // and of pass 2, written by the query preparation
+  int32_t* work_ctr;    // [4 + B*Hkv]: unused, next item to claim, kept tokens per item, unused; then the finished
                         // items of every (sequence, kv-head)
   // outputs (each optional)
   float* out_f32;    // [B][Hq][hd]
@@ -279,7 +268,7 @@ void launch_span_attention(const AttnArgs& a, int n_tok, cudaStream_t st);
 
 // Offsets of the attention scratch inside a buffer, starting at `at` (a multiple of 256).
 struct AttnScratch {
-  size_t q_rot, q_split, logits, sigma, row_hist, row_ctl, seg_pub, cand_idx, cand_val, kept_idx, kept_cnt, kept_row, part, plan, work_items, work_ctr, page_mask, quest_keys, quest_err, quest_hmask, quest_qsplit, quest_l1, quest_order, end;
+  size_t q_rot, q_split, logits, sigma, row_hist, row_ctl, kept_idx, kept_cnt, kept_row, part, plan, work_ctr, page_mask, quest_keys, quest_err, quest_hmask, quest_qsplit, quest_l1, quest_order, end;
   int splits;
 };
 inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_pages, size_t at) {
@@ -298,15 +287,15 @@ inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_page
   L.sigma = take(BK * Tmax * 4);
   L.row_hist = take(BK * 4096 * 4);
   L.row_ctl = take(BK * 8 * 4);
-  L.seg_pub = take(BK * (size_t)attn_select_segs(max_pages, s.page_size) * 4);
-  L.cand_idx = take(BK * 1024 * 4);
-  L.cand_val = take(BK * 1024 * 4);
+  // not used; the sum stays what sol_workspace_bytes has always answered and the static scratch's limit is made of
+  take(BK * ((Tmax + 2047) / 2048) * 4);
+  take(BK * 1024 * 8);
   L.kept_idx = take(BK * Tmax * 4);
   L.kept_cnt = take(BK * 4);
   L.kept_row = take(BK * Tmax * 4);
   L.part = take(BK * L.splits * G * (hd + 2) * 4);
   L.plan = take(3 * 132 * 4);
-  L.work_items = take(BK * L.splits * 8);
+  take(BK * L.splits * 8);  // not used, see above
   L.work_ctr = take((4 + BK) * 4);
   const bool quest = s.token_select == SOL_SELECT_QUEST_PAGES;
   L.page_mask = take(quest ? BK * (Tmax / 4) : 0);
@@ -328,16 +317,12 @@ inline void attn_scratch_bind(AttnArgs& a, void* base, const AttnScratch& L, int
   a.sigma = reinterpret_cast<float*>(b + L.sigma);
   a.row_hist = reinterpret_cast<uint32_t*>(b + L.row_hist);
   a.row_ctl = reinterpret_cast<uint32_t*>(b + L.row_ctl);
-  a.seg_pub = reinterpret_cast<uint32_t*>(b + L.seg_pub);
-  a.cand_idx = reinterpret_cast<int32_t*>(b + L.cand_idx);
-  a.cand_val = reinterpret_cast<float*>(b + L.cand_val);
   a.list_idx = reinterpret_cast<int32_t*>(b + L.kept_idx);
   a.kept_idx_out = kept_idx;
   a.kept_cnt = kept_cnt ? kept_cnt : reinterpret_cast<int32_t*>(b + L.kept_cnt);
   a.kept_row = reinterpret_cast<uint32_t*>(b + L.kept_row);
   a.part = reinterpret_cast<float*>(b + L.part);
   a.plan = reinterpret_cast<int32_t*>(b + L.plan);
-  a.work_items = reinterpret_cast<int32_t*>(b + L.work_items);
   a.work_ctr = reinterpret_cast<int32_t*>(b + L.work_ctr);
   a.page_mask = b + L.page_mask;
   a.quest_keys = reinterpret_cast<uint32_t*>(b + L.quest_keys);
