@@ -60,6 +60,9 @@ __device__ __forceinline__ RowPlan row_plan(const sol_shape_t& sh, const sol_kv_
   return r;
 }
 
+// Warps of a pass-2 CTA (one CTA per SM).
+constexpr int gather_warps(int hd, int gmax) { return hd == 64 ? (gmax == 4 ? 16 : 12) : 8; }
+
 // Tokens of a row per pass-2 item, for items of about c kept tokens each; min_len (the token count of a slot of the
 // partial results) at least.  A multiple of 128, so that the scores of an item start on a full line.
 __device__ __forceinline__ int gather_item_tokens(const RowPlan& rp, int c, int min_len) {
@@ -102,6 +105,8 @@ struct PrepDev {
 };
 
 constexpr int PREP_THREADS = 128;
+constexpr int ITEM_FILL = 256;  // measured: 64 to 192 cut long rows into too many items (290 -> 365 us where all of
+                                // 128 ragged sequences' tokens are kept), 512 gave up balance (32 equal sequences 98 -> 122)
 // words of AttnArgs::row_ctl, per (sequence, kv-head): segments whose scores are in the histogram, largest |score|,
 // keep edge (float bits)
 enum : int { RC_DONE = 0, RC_MAX, RC_EDGE, RC_WORDS = 8 };
@@ -121,10 +126,10 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
   pdl_wait();
 
   // The first CTA lays out the work of the kernels that follow: cumulative segment and item counts over the
-  // batch, and the kept tokens of a pass-2 item: the smallest power of two (64 to 1024) that gives every resident
-  // warp of pass 2 at most one item, so that there is no second, partly filled round of items; when even the
-  // longest runs leave more items than warps there is work for many rounds, and runs of 1024 tokens (32
-  // batches, enough to amortise filling a warp's ring of row copies), claimed one by one, balance it.
+  // batch, and the kept tokens c of a pass-2 item, a power of two from 64 to 1024: the one with the least time by the
+  // rounds its items take on the resident warps, each round as long as an item and the ITEM_FILL tokens that filling
+  // a warp's ring of row copies is worth.  (Long items alone left the chip half empty in a second round: 134 MB of
+  // values of 32 sequences in 55 us.)
   if (kvh == 0 && b == 0) {
     constexpr int C0 = 64, NC = 5;
     __shared__ int wsum[PLAN_LISTS][PREP_THREADS / 32];
@@ -149,10 +154,17 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
       if (l == 0) atomicAdd(&n_items[q], n);
     }
     __syncthreads();
-    int pick = NC - 1;
+    int pick = 0;
+    long long best = 0x7fffffffffffffffLL;
 #pragma unroll
-    for (int q = NC - 2; q >= 0; --q)
-      if ((long long)n_items[q] * Hkv <= p.target_items) pick = q;
+    for (int q = 0; q < NC; ++q) {
+      const long long rounds = ((long long)n_items[q] * Hkv + p.target_items - 1) / p.target_items;
+      const long long cost = rounds * ((C0 << q) + ITEM_FILL);
+      if (cost <= best) {
+        best = cost;
+        pick = q;
+      }
+    }
 #pragma unroll
     for (int q = 0; q < NC; ++q)
       if (q == pick) cnt[PLAN_ITEMS] = per_seq[q];
@@ -178,6 +190,7 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
     if (tid == 0) {
       p.work_ctr[WC_CPI] = C0 << pick;
       p.work_ctr[WC_NEXT] = 0;
+      p.work_ctr[WC_SELECT] = 0;
     }
   }
 
@@ -414,88 +427,61 @@ struct ScoreDev {
 
 constexpr int SC_WARPS = 4;  // pages per CTA
 static_assert(SC_WARPS * PAGE == PLAN_GROUP_TOKENS, "a unit of attn_score is one page per warp");
-constexpr int SC_MAX_GRID = 32768;  // CTAs launched at most; beyond that a CTA takes several units
+constexpr int SC_PER_SM = 12;  // CTAs per SM of the grid: twice what is resident (6 and 24 measured the same within 1 %)
 
-template <int HD, int HG, bool FLAT>
+template <int HD, int HG>
 __global__ void __launch_bounds__(SC_WARPS * 32) attn_score_kernel(const ScoreDev p) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int PAGE_BYTES = PAGE * HD * 2;
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SC_WARPS * PAGE_BYTES);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   pdl_trigger();
-  // Two ways to give the CTAs their unit (sequence, kv-head, group of four pages).  Direct (FLAT = false): a
-  // 3-D grid over the longest row the page table allows; CTAs beyond their sequence's length leave at once.
-  // That is the cheapest mapping, but an empty CTA costs ~0.5 ns of CTA issue: 70 us for the 131072 CTAs of
-  // 128 ragged sequences, four in five of them empty.  Flat (FLAT = true, chosen by the host when the direct
-  // grid would exceed SC_MAX_GRID): the units that exist are numbered along the batch; every CTA adds up the
-  // sequences' group counts itself from the lengths (an input of the step, so before the wait for the
-  // earlier kernels) and takes every gridDim.x-th unit.  The flat mapping costs each CTA two block
-  // barriers and a block-wide count, which made uniform batches 6-15 % slower, hence both.
-  // A row that keeps every token has no units: pass 2 reads its keys with its values.  A launch may then have no
-  // work at all; its first CTA still waits for the kernels before, so that the kernels after can rely on them.
-  const bool first_cta = blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0;
+  // The units (sequence, kv-head, group of four pages) that exist are numbered along the batch: every CTA adds up the
+  // sequences' group counts itself from the lengths and keep-rates (inputs of the step, so before the wait for the
+  // earlier kernels) and takes every gridDim.x-th unit.  A row that keeps every token has no units: pass 2 reads its
+  // keys with its values.  (A 3-D grid over the longest row the page table allows spends ~0.5 ns of CTA issue on every
+  // empty CTA, and a CTA per unit its set-up: 64 sequences of 16384 tokens 352 us, this 341; 128 ragged sequences 161
+  // and 147.)
   __shared__ int s_cum[SC_WARPS * 32 + 1], s_len[SC_WARPS * 32], s_wsum[SC_WARPS];
-  int my_incl = 0, n_units = 1;
-  if (FLAT) {
-    const int tid = threadIdx.x;
-    int Tt = 0;
-    if (tid < p.B) {
-      const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
-      Tt = rp.dense() ? 0 : max(rp.T, 0);
-    }
-    my_incl = (Tt + PLAN_GROUP_TOKENS - 1) / PLAN_GROUP_TOKENS;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const int x = __shfl_up_sync(0xffffffffu, my_incl, o);
-      if (lane >= o) my_incl += x;
-    }
-    if (lane == 31) s_wsum[warp] = my_incl;
-    if (tid == 0) s_cum[0] = 0;
-    __syncthreads();
-    for (int w = 0; w < warp; ++w) my_incl += s_wsum[w];
-    s_cum[tid + 1] = my_incl;
-    s_len[tid] = Tt;
-    __syncthreads();
-    n_units = s_cum[p.B] * p.Hkv;
-    if ((int)blockIdx.x >= n_units) {
-      if (first_cta) pdl_wait();
-      return;
-    }
-  } else {
-    if ((int)blockIdx.x * SC_WARPS * PAGE >= p.kv.seq_lens[blockIdx.z] ||
-        row_plan(p.sh, p.kv, p.r_permille, blockIdx.z).dense()) {
-      if (first_cta) pdl_wait();
-      return;
-    }
+  int Tt = 0;
+  if (tid < p.B) {
+    const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
+    Tt = rp.dense() ? 0 : max(rp.T, 0);  // never indexes past the page table
   }
-  if (threadIdx.x == 0) {
+  int my_incl = (Tt + PLAN_GROUP_TOKENS - 1) / PLAN_GROUP_TOKENS;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, my_incl, o);
+    if (lane >= o) my_incl += x;
+  }
+  if (lane == 31) s_wsum[warp] = my_incl;
+  if (tid == 0) {
+    s_cum[0] = 0;
     for (int i = 0; i < SC_WARPS; ++i) mbar_init(&bars[i], 1);
     fence_mbar_init();
   }
   __syncthreads();
+  for (int w = 0; w < warp; ++w) my_incl += s_wsum[w];
+  s_cum[tid + 1] = my_incl;
+  s_len[tid] = Tt;
+  __syncthreads();
+  const int n_units = s_cum[p.B] * p.Hkv;
+  // a launch may have no work at all; its first CTA still waits for the kernels before, on which the ones after rely
+  if ((int)blockIdx.x >= max(n_units, 1)) return;
   pdl_wait();
   const int g = lane >> 2, t = lane & 3;
   constexpr int KS = HD / 32;  // pair steps (two MMAs of k=16 each)
   uint32_t phase = 0;
   bool dead = false;  // a wait ran out: no more work, but the block-wide counts below still need this warp
 #pragma unroll 1
-  for (int u = FLAT ? blockIdx.x : 0; u < n_units; u += gridDim.x) {
-    int b, kvh, grp, T;
-    if (FLAT) {
-      // sequence of unit u: how many cumulative counts lie at or below u / Hkv
-      const int key = u / p.Hkv;
-      b = __syncthreads_count((int)threadIdx.x < p.B && my_incl <= key);
-      const int first = s_cum[b], n_groups = s_cum[b + 1] - first;
-      const int rem = u - first * p.Hkv;
-      kvh = rem / n_groups;
-      grp = rem - kvh * n_groups;
-      T = s_len[b];
-    } else {
-      b = blockIdx.z;
-      kvh = blockIdx.y;
-      grp = blockIdx.x;
-      T = min(p.kv.seq_lens[b], p.kv.max_pages_per_seq * PAGE);  // never index past the page table
-    }
+  for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
+    // sequence of unit u: how many cumulative counts lie at or below u / Hkv
+    const int key = u / p.Hkv;
+    const int b = __syncthreads_count(tid < p.B && my_incl <= key);
+    const int first = s_cum[b], n_groups = s_cum[b + 1] - first;
+    const int rem = u - first * p.Hkv;
+    const int kvh = rem / n_groups, grp = rem - kvh * n_groups;
+    const int T = s_len[b];
     const int lp = grp * SC_WARPS + warp;  // logical page
     if (dead || lp * PAGE >= T || lp >= p.kv.max_pages_per_seq) continue;
     const int page = p.kv.page_table[(size_t)b * p.kv.max_pages_per_seq + lp];
@@ -594,8 +580,11 @@ __global__ void __launch_bounds__(SC_WARPS * 32) attn_score_kernel(const ScoreDe
 // (A list of the kept tokens in memory, written by kernels of its own over 2048-token segments and read back by
 // pass 2, cost 16 bytes of traffic per kept token and, with the settling, two more latency-bound launches: 24 + 35 +
 // 21 us per layer on 128 ragged sequences.)
-constexpr int TS_THREADS = 256;
-constexpr int TS_PER_SM = 4;  // CTAs per SM of the persistent grid
+// Latency-bound: a chain of barriers and L2 round trips per row.  Hence one bulk copy for a segment's scores and short
+// rolled loops over them in shared memory (unrolled over registers, the code of a unit was fetched cold for 14 us even
+// where a launch has one unit of 2000 scores), and 512 threads.
+constexpr int TS_THREADS = 512;
+constexpr int TS_PER_SM = 3;  // CTAs per SM of the persistent grid: 53 KB of shared memory and 48 warps
 constexpr float TS_FLT_MAX = 3.402823466e+38f;
 
 struct SelectDev {
@@ -609,6 +598,7 @@ struct SelectDev {
   uint32_t* row_hist;    // [B*Hkv][SEL_BINS], zero on entry (rows of several segments)
   uint32_t* row_ctl;     // [B*Hkv][RC_WORDS], zero on entry
   int32_t* kept_cnt;
+  int32_t* work_ctr;
   int* status;
 };
 
@@ -636,10 +626,12 @@ __device__ __forceinline__ int ts_block_scan(int v, int& total, int* warp_tot) {
 }
 
 struct SelSmem {
-  SelectSmemOverlay sm;  // the candidates are listed when the histogram is no longer read
+  alignas(128) float score[TH_SEG];  // the segment's scores
+  alignas(16) SelectSmemOverlay sm;  // the candidates are listed when the histogram is no longer read
+  uint64_t bar;
   double qsum[128];
   float fmax_w[TS_THREADS / 32];
-  int s_flag;
+  int s_flag, s_next;
   int cum[PLAN_STRIDE];
 };
 
@@ -712,16 +704,17 @@ __device__ __forceinline__ void settle_row(const SelectDev& p, SelectSmemOverlay
   } else if (need_s > 0) {
     const int ns = ns_all;
     const float* sup_val = sm.f32;
-    // float32 rank inside the list: the element of rank need_s - 1 carries the k-th value
-    for (int c = tid; c < ns; c += TS_THREADS) {
+    // float32 rank inside the list: the element of rank need_s - 1 carries the k-th value.  A warp per candidate: a
+    // thread per candidate walked the list alone, a chain of up to some hundred shared-memory reads.
+    for (int c = warp; c < ns; c += WARPS) {
       const float v = sup_val[c];
       const int j = sm.cand_idx[c];
       int rank = 0;
-      for (int o = 0; o < ns; ++o) {
+      for (int o = lane; o < ns; o += 32) {
         const float vo = sup_val[o];
         rank += (vo > v) || (vo == v && sm.cand_idx[o] < j);
       }
-      if (rank == need_s - 1) sm.pick[1] = __float_as_int(v);
+      if (__reduce_add_sync(0xffffffffu, rank) == need_s - 1) sm.pick[1] = __float_as_int(v);
     }
     __syncthreads();
     const float thr32 = __int_as_float(sm.pick[1]);
@@ -770,17 +763,23 @@ __device__ __forceinline__ void settle_row(const SelectDev& p, SelectSmemOverlay
       }
       __syncthreads();
     }
-    rank_candidates<TS_THREADS>(ns, need_s, sm);  // cand_keep[c] = 1 for the need_s best of the list
-    __syncthreads();
-    for (int c = tid; c < ns; c += TS_THREADS)
-      if (sm.cand_keep[c]) sig[sm.cand_idx[c]] = INFINITY;
+    for (int c = warp; c < ns; c += WARPS) {  // the need_s best of the list are kept
+      const double v = sm.cand_val[c];
+      const int j = sm.cand_idx[c];
+      int rank = 0;
+      for (int o = lane; o < ns; o += 32) {
+        const double vo = sm.cand_val[o];
+        rank += (vo > v) || (vo == v && sm.cand_idx[o] < j);
+      }
+      if (__reduce_add_sync(0xffffffffu, rank) < need_s && lane == 0) sig[j] = INFINITY;
+    }
     n_list += need_s;
   }
   if (tid == 0) p.kept_cnt[bk] = n_list;
 }
 
-// One (sequence, kv-head, 8192-token segment) of a row that needs a selection.
-__device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& hs, int b, int kvh, int seg) {
+// One (sequence, kv-head, 8192-token segment) of a row that needs a selection; the phase of hs.bar is the caller's.
+__device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& hs, int b, int kvh, int seg, uint32_t& phase) {
   SelectSmemOverlay& sm = hs.sm;
   uint32_t* hist = sm.hist;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -792,28 +791,25 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   uint32_t* ctl = p.row_ctl + (size_t)bk * RC_WORDS;
   uint32_t* gh = p.row_hist + (size_t)bk * SEL_BINS;
   const int nseg = (T + TH_SEG - 1) / TH_SEG;
-  for (int i = tid; i < SEL_BINS; i += TS_THREADS) hist[i] = 0;
+  const int j_first = seg * TH_SEG, n_here = min(T - j_first, TH_SEG);
+  if (tid == 0) {  // a row's space ends on a full page, so whole groups of four may be read
+    const uint32_t bytes = (uint32_t)((n_here + 3) & ~3) * 4;
+    mbar_expect_tx(&hs.bar, bytes);
+    bulk_g2s(hs.score, sig + j_first, bytes, &hs.bar);
+  }
+  for (int i = tid; i < SEL_BINS / 4; i += TS_THREADS) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
+  mbar_wait(&hs.bar, phase, p.status);  // a wait that gives up is reported; what follows stays in bounds
+  phase ^= 1;
 
-  // ---- this CTA's scores: 32 per thread, all loads issued before the first use ----
-  constexpr int VPT = TH_SEG / TS_THREADS / 4;  // float4 loads per thread
-  float4 v[VPT];
-  auto load_segment = [&](int base) {
-#pragma unroll
-    for (int q = 0; q < VPT; ++q) {
-      const int j = base + (q * TS_THREADS + tid) * 4;
-      v[q] = j < T ? *reinterpret_cast<const float4*>(sig + j) : make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-  };
-  load_segment(seg * TH_SEG);
   float mx = 0.f;
-#pragma unroll
-  for (int q = 0; q < VPT; ++q) {
-    const int j0 = seg * TH_SEG + (q * TS_THREADS + tid) * 4;
-    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll 1
+  for (int i = tid * 4; i < n_here; i += TS_THREADS * 4) {
+    const float4 v = *reinterpret_cast<const float4*>(hs.score + i);
+    const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-      const int j = j0 + e;
+      const int j = j_first + i + e;
       if (j < T && !rp.forced(j)) {
         atomicAdd(&hist[key_value_bin(float_key(vv[e]))], 1u);
         mx = fmaxf(mx, fabsf(vv[e]));
@@ -823,9 +819,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   mx = warp_max(mx);
   if (lane == 0) hs.fmax_w[warp] = mx;
   __syncthreads();
-  mx = 0.f;
-#pragma unroll
-  for (int w = 0; w < TS_THREADS / 32; ++w) mx = fmaxf(mx, hs.fmax_w[w]);
+  mx = warp_max(lane < TS_THREADS / 32 ? hs.fmax_w[lane] : 0.f);
   if (nseg > 1) {  // only the CTA that arrives last goes on
     for (int i = tid; i < SEL_BINS; i += TS_THREADS) {
       const uint32_t c = hist[i];
@@ -838,28 +832,35 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
     __syncthreads();
     if (!hs.s_flag) return;
     __threadfence();
-    for (int i = tid; i < SEL_BINS; i += TS_THREADS) hist[i] = __ldcg(gh + i);
+    for (int i = tid; i < SEL_BINS / 4; i += TS_THREADS)
+      reinterpret_cast<uint4*>(hist)[i] = __ldcg(reinterpret_cast<const uint4*>(gh) + i);
     mx = __uint_as_float(__ldcg(ctl + RC_MAX));
     __syncthreads();
   }
 
-  // ---- the bin that holds the `want`-th largest of the histogrammed scores, and how many lie above it:
-  //      thread t owns bins 4095 - 16 t .. 4080 - 16 t
+  // ---- the bin that holds the `want`-th largest of the histogrammed scores, how many lie above it, how many in it:
+  //      thread t owns a run of bins, the first thread the highest
   auto rank_bin = [&](int want) {
     constexpr int BPT = SEL_BINS / TS_THREADS;
+    const uint4* own = reinterpret_cast<const uint4*>(hist + SEL_BINS - BPT * (tid + 1));
     int mine = 0;
 #pragma unroll
-    for (int q = 0; q < BPT; ++q) mine += (int)hist[SEL_BINS - 1 - tid * BPT - q];
+    for (int q = 0; q < BPT / 4; ++q) {
+      const uint4 x = own[q];
+      mine += (int)(x.x + x.y + x.z + x.w);
+    }
     int total;
     const int before = ts_block_scan(mine, total, sm.scan[0]);
     if (before < want && want <= before + mine) {
       int a = before;
+#pragma unroll 1
       for (int q = 0; q < BPT; ++q) {
         const int bin = SEL_BINS - 1 - tid * BPT - q;
         const int c = (int)hist[bin];
         if (want <= a + c) {
           sm.pick[0] = bin;
           sm.pick[1] = a;
+          sm.pick[2] = c;
           break;
         }
         a += c;
@@ -869,15 +870,15 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   };
   const int need_total = rp.k - rp.nf;
   rank_bin(need_total);
-  const int vbin = sm.pick[0], above_bin = sm.pick[1];
-  const int pop = (int)hist[vbin];
+  const int vbin = sm.pick[0];
+  int above = sm.pick[1];  // scores above the bin
   uint32_t klo, khi;
   value_bin_key_range(vbin, klo, khi);
-  __syncthreads();
   const bool prefix_bin = vbin != 0 && vbin != SEL_BINS / 2 - 1 && vbin != SEL_BINS / 2 && vbin != SEL_BINS - 1;
-  if (pop > SEL_CAND_CAP / 2 && prefix_bin) {
+  if (sm.pick[2] > SEL_CAND_CAP / 2 && prefix_bin) {
     // A crowded bin (many nearly equal scores): histogram the next 12 key bits of the bin's keys (they share
     // their upper 15 bits) and take the sub-bin of the k-th score, so that the candidate list stays short.
+    __syncthreads();
     for (int i = tid; i < SEL_BINS; i += TS_THREADS) hist[i] = 0;
     __syncthreads();
 #pragma unroll 4
@@ -887,63 +888,86 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
       if (kk >= klo && kk <= khi) atomicAdd(&hist[(kk >> 5) & 0xfffu], 1u);
     }
     __syncthreads();
-    rank_bin(need_total - above_bin);
+    rank_bin(need_total - above);
+    above += sm.pick[1];
     klo = (klo & 0xfffe0000u) | ((uint32_t)sm.pick[0] << 5);
     khi = klo | 31u;
   }
   // window: 2^-16 of the largest score, far above the float32 accumulation error of a head_dim-long dot product
   const float delta = mx * 1.52587890625e-05f;
+  const float bin_hi = key_to_float(khi);
   const float lo = key_to_float(klo) - delta;
-  const float edge = fminf(key_to_float(khi) + delta, TS_FLT_MAX);
+  const float edge = fminf(bin_hi + delta, TS_FLT_MAX);
   if (tid == 0) {
     ctl[RC_EDGE] = __float_as_uint(edge);  // for pass 2 and token_list
     sm.counts[0] = 0;
   }
   __syncthreads();  // the histogram is not read any more: the candidates take its space
 
-  // ---- what lies above the edge is counted, what lies between the edges is listed ----
-  int n_above = 0;
-#pragma unroll 1
-  for (int base = 0; base < T; base += TH_SEG) {
-    if (nseg > 1) load_segment(base);  // a row of one segment still has its scores
+  // ---- what lies between the edges is listed; `above` loses those of the list that lie above the bin ----
+  int in_window = 0;
+  auto list_candidates = [&](float4 v, int j0) {
+    const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-    for (int q = 0; q < VPT; ++q) {
-      const int j0 = base + (q * TS_THREADS + tid) * 4;
-      const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
+    for (int e = 0; e < 4; ++e) {
+      if (vv[e] >= lo && vv[e] <= edge) {
         const int j = j0 + e;
-        if (vv[e] >= lo && j < T && !rp.forced(j)) {
-          if (vv[e] > edge) {
-            ++n_above;
-          } else {
-            const int slot = atomicAdd(&sm.counts[0], 1);
-            if (slot < SEL_CAND_CAP) {
-              sm.cand_idx[slot] = j;
-              sm.f32[slot] = vv[e];
-            }
+        if (j < T && !rp.forced(j)) {
+          if (vv[e] > bin_hi) ++in_window;
+          const int slot = atomicAdd(&sm.counts[0], 1);
+          if (slot < SEL_CAND_CAP) {
+            sm.cand_idx[slot] = j;
+            sm.f32[slot] = vv[e];
           }
         }
       }
     }
+  };
+  if (nseg == 1) {
+#pragma unroll 1
+    for (int i = tid * 4; i < n_here; i += TS_THREADS * 4) list_candidates(*reinterpret_cast<const float4*>(hs.score + i), i);
+  } else {
+#pragma unroll 1
+    for (int j0 = tid * 4; j0 < T; j0 += TS_THREADS * 16) {  // four loads in flight
+      float4 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int j = j0 + q * TS_THREADS * 4;
+        v[q] = *reinterpret_cast<const float4*>(sig + (j < T ? j : 0));
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (j0 + q * TS_THREADS * 4 < T) list_candidates(v[q], j0 + q * TS_THREADS * 4);
+    }
   }
-  n_above = block_count<TS_THREADS>(n_above, 0, sm);  // the barrier inside also publishes the candidates
-  settle_row(p, sm, hs.qsum, rp, b, kvh, n_above + rp.nf, edge, lo, delta, sm.counts[0]);
+  in_window = block_count<TS_THREADS>(in_window, 0, sm);  // the barrier inside also publishes the candidates
+  settle_row(p, sm, hs.qsum, rp, b, kvh, above - in_window + rp.nf, edge, lo, delta, sm.counts[0]);
 }
 
 // Persistent CTAs over the flat list of (sequence, kv-head, segment) units of the rows that need a selection.
 __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(const SelectDev p) {
-  __shared__ SelSmem hs;
+  extern __shared__ __align__(128) unsigned char ts_smem[];
+  SelSmem& hs = *reinterpret_cast<SelSmem*>(ts_smem);
   pdl_trigger();
+  if (threadIdx.x == 0) {
+    mbar_init(&hs.bar, 1);
+    fence_mbar_init();
+  }
   pdl_wait();
   for (int i = threadIdx.x; i <= p.B; i += TS_THREADS) hs.cum[i] = p.plan[PLAN_HSEG * PLAN_STRIDE + i];
   __syncthreads();
   const int Hkv = p.sh.n_kv_heads;
   const int n_units = hs.cum[p.B] * Hkv;
-  for (int u = blockIdx.x; u < n_units; u += gridDim.x) {
+  uint32_t phase = 0;
+  // a CTA's first unit is its index, the later ones are claimed (while the unit before is worked on): the CTA that
+  // comes last on a row has the whole of it to settle, and units dealt by index left some CTAs with several such rows
+  for (int u = blockIdx.x; u < n_units;) {
+    if (threadIdx.x == 0) hs.s_next = (int)gridDim.x + atomicAdd(p.work_ctr + WC_SELECT, 1);
     const int b = plan_find(hs.cum, p.B, u / Hkv);
     const int n = hs.cum[b + 1] - hs.cum[b], rem = u - hs.cum[b] * Hkv;
-    token_select_item(p, hs, b, rem / n, rem % n);
+    token_select_item(p, hs, b, rem / n, rem % n, phase);
+    __syncthreads();
+    u = hs.s_next;
     __syncthreads();
   }
 }
@@ -1042,10 +1066,13 @@ constexpr int GA_DENSE = 16;   // tokens per warp step of a row that keeps every
 // sum) is written and the warp that finishes the last item of a (sequence, kv-head) merges the partials.
 // The pipeline's fill, steady state and drain are one rolled loop: a launch that gives every warp one item of a few
 // batches runs its code cold.
+// Sixteen warps with rings of three batches, where shared memory allows it: a warp's steps are chains of dependent
+// instructions, so more warps beat deeper rings (12 warps with four batches: 118 against 79 us at r = 0.25 on 128 ragged
+// sequences, 139 against 129 at r = 0.5, the same where every token is kept).
 template <int HD, int GMAX>
 struct GatherCfg {
-  static constexpr int WARPS = HD == 64 ? 12 : 8;
-  static constexpr int NST = HD == 64 && GMAX == 4 ? 4 : 3;  // batches of rows per warp ring
+  static constexpr int WARPS = gather_warps(HD, GMAX);
+  static constexpr int NST = 3;                              // batches of rows per warp ring
   static constexpr int STAGE_BYTES = GA_BATCH * HD * 2;      // 4 KB / 8 KB
   static constexpr int THREADS = WARPS * 32;
   static constexpr int RING_BYTES = WARPS * NST * STAGE_BYTES;  // 192 KB (hd 64, G > 4: 144 KB)
@@ -1242,54 +1269,56 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
       const float* lgrow = p.logits + row * G;
       const float edge = rp.mode == 2 ? __uint_as_float(p.row_ctl[(size_t)bk * RC_WORDS + RC_EDGE]) : INFINITY;
 
-      // ---- the queue of kept tokens: offsets from n0, in order; the scores of the next two chunks wait in registers ----
+      // ---- the queue of kept tokens' offsets from n0; the scores of the next two chunks wait in registers: lane l holds
+      //      tokens 4 l .. 4 l + 3 of both halves of a chunk ----
       int q_head = 0, q_tail = 0, c_at = n0;
       float4 sv[2], sw[2];
       auto fetch_scores = [&](int base, float4 (&v)[2]) {
-        const int j = base + lane * 8;
-        v[0] = v[1] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        if (j < n1 && rp.mode == 2) {  // a row's space ends on a full page: a group of eight never passes it
-          v[0] = *reinterpret_cast<const float4*>(sig + j);
-          v[1] = *reinterpret_cast<const float4*>(sig + j + 4);
+#pragma unroll
+        for (int x = 0; x < 2; ++x) {
+          const int j = base + x * (GA_CHUNK / 2) + lane * 4;
+          v[x] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+          if (j < n1 && rp.mode == 2) v[x] = *reinterpret_cast<const float4*>(sig + j);  // a row's space ends on a full page
         }
       };
       fetch_scores(c_at, sv);
       fetch_scores(c_at + GA_CHUNK, sw);
+      const uint32_t below = (1u << lane) - 1u;
       // the next (up to) 32 kept tokens, one per lane: (cache row or -1, token)
       auto pop = [&]() {
 #pragma unroll 1
         while (q_tail - q_head < GA_BATCH && c_at < n1) {  // warp-uniform
-          const int left = q_tail - q_head, j0 = c_at + lane * 8;
+          const int left = q_tail - q_head;
           const uint16_t moved = lane < left ? my_q[q_head + lane] : (uint16_t)0;
-          const float vv[8] = {sv[0].x, sv[0].y, sv[0].z, sv[0].w, sv[1].x, sv[1].y, sv[1].z, sv[1].w};
           uint32_t keep = 0;
-#pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if (vv[e] > edge) keep |= 1u << e;
-          if (j0 < rp.n_sink || j0 + 8 > rp.T - rp.n_win) {
+          {
+            const float vv[8] = {sv[0].x, sv[0].y, sv[0].z, sv[0].w, sv[1].x, sv[1].y, sv[1].z, sv[1].w};
 #pragma unroll
             for (int e = 0; e < 8; ++e)
-              if (rp.forced(j0 + e)) keep |= 1u << e;
+              if (vv[e] > edge) keep |= 1u << e;
           }
-          if (j0 + 8 > n1) keep &= j0 < n1 ? (1u << (n1 - j0)) - 1u : 0u;
           sv[0] = sw[0];
           sv[1] = sw[1];
           fetch_scores(c_at + 2 * GA_CHUNK, sw);
-          int incl = __popc(keep);
-          const int mine = incl;
+          if (c_at < rp.n_sink || c_at + GA_CHUNK > min(n1, rp.T - rp.n_win)) {  // warp-uniform: forced tokens, the run's end
 #pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += y;
+            for (int e = 0; e < 8; ++e) {
+              const int j = c_at + (e >> 2) * (GA_CHUNK / 2) + lane * 4 + (e & 3);
+              if (rp.forced(j)) keep |= 1u << e;
+              if (j >= n1) keep &= ~(1u << e);
+            }
           }
           __syncwarp();
           if (lane < left) my_q[lane] = moved;
-          int pos = left + incl - mine;
+          q_tail = left;
 #pragma unroll
-          for (int e = 0; e < 8; ++e)
-            if ((keep >> e) & 1u) my_q[pos++] = (uint16_t)(j0 + e - n0);
+          for (int e = 0; e < 8; ++e) {
+            const bool k = (keep >> e) & 1u;
+            const uint32_t all = __ballot_sync(0xffffffffu, k);
+            if (k) my_q[q_tail + __popc(all & below)] = (uint16_t)(c_at - n0 + (e >> 2) * (GA_CHUNK / 2) + lane * 4 + (e & 3));
+            q_tail += __popc(all);
+          }
           q_head = 0;
-          q_tail = left + __shfl_sync(0xffffffffu, incl, 31);
           c_at += GA_CHUNK;
           __syncwarp();
         }
@@ -1302,11 +1331,11 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         return e;
       };
 
-      float mh[GMAX], ls[GMAX];
+      float mt[HG], lt[HG];  // head 4 hg + t: running maximum, this lane's share of the sum
 #pragma unroll
-      for (int h = 0; h < GMAX; ++h) {
-        mh[h] = -INFINITY;
-        ls[h] = 0.f;
+      for (int hg = 0; hg < HG; ++hg) {
+        mt[hg] = -INFINITY;
+        lt[hg] = 0.f;
       }
       int2 e_cur = pop();
       int nb = q_tail > q_head ? 0x7fffffff : 0;  // batches of the item: known once a pop comes back empty
@@ -1348,19 +1377,39 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         if (s - (NST - 1) < 0) continue;
         // ---- the batch that was requested NST - 1 steps ago, in the slot that is written next ----
         cp_async_wait<NST - 1>();
+        __syncwarp();  // every lane's pieces of the batch have landed
+        // softmax weights relative to the running maximum, in the logits' place: lane (g, t) takes head t of tokens g,
+        // g + 8, g + 16, g + 24, so that a maximum over the batch is three exchanges
         float* wt = my_w + slot_w * GA_BATCH * GMAX;  // [32][GMAX]
         float sc0 = 0.f, sc1 = 0.f;                   // rescaling of this lane's accumulator columns
 #pragma unroll
-        for (int h = 0; h < GMAX; ++h) {  // softmax weights relative to the running maximum, in the logits' place
-          const float x = h < G ? wt[lane * GMAX + h] * p.scale_log2 : -INFINITY;
-          const float nm = fmaxf(mh[h], warp_max(x));
-          const float sc = mh[h] == -INFINITY ? 0.f : exp2f(mh[h] - nm);
-          const float pw = x == -INFINITY ? 0.f : exp2f(x - nm);
-          mh[h] = nm;
-          ls[h] = ls[h] * sc + pw;
-          if (h == ((2 * t) & (GMAX - 1))) sc0 = sc;
-          if (h == ((2 * t + 1) & (GMAX - 1))) sc1 = sc;
-          wt[lane * GMAX + h] = pw;
+        for (int hg = 0; hg < HG; ++hg) {
+          float x[4], mx = -INFINITY;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            x[q] = hg * 4 + t < G ? wt[(g + 8 * q) * GMAX + hg * 4 + t] * p.scale_log2 : -INFINITY;
+            mx = fmaxf(mx, x[q]);
+          }
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+          mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+          const float nm = fmaxf(mt[hg], mx);
+          const float sc = mt[hg] == -INFINITY ? 0.f : exp2f(mt[hg] - nm);
+          mt[hg] = nm;
+          float l = 0.f;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float w = x[q] == -INFINITY ? 0.f : exp2f(x[q] - nm);
+            l += w;
+            wt[(g + 8 * q) * GMAX + hg * 4 + t] = w;
+          }
+          lt[hg] = lt[hg] * sc + l;
+          // this lane's accumulator columns: heads 2t, 2t + 1 (modulo 4 where the columns are high and low parts)
+          const float y0 = __shfl_sync(0xffffffffu, sc, (2 * t) & 3), y1 = __shfl_sync(0xffffffffu, sc, (2 * t + 1) & 3);
+          if (HG == 1 || (t >> 1) == hg) {
+            sc0 = y0;
+            sc1 = y1;
+          }
         }
 #pragma unroll
         for (int j = 0; j < HD / 16; ++j) {
@@ -1369,7 +1418,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
           acc[j][2] *= sc0;
           acc[j][3] *= sc1;
         }
-        __syncwarp();  // every lane's pieces of the batch have landed and the weights are in place
+        __syncwarp();  // the weights are in place
         const uint32_t st = smem_u32(my_ring + slot_w * C::STAGE_BYTES);
 #pragma unroll
         for (int ks = 0; ks < GA_BATCH / 16; ++ks) {
@@ -1388,11 +1437,14 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
       }
       __syncwarp();  // the queue is not read any more
 #pragma unroll
-      for (int h = 0; h < GMAX; ++h) {
-        const float l = warp_sum(ls[h]);
-        if (lane == 0) {
-          ml[h] = mh[h];
-          ml[GMAX + h] = l;
+      for (int hg = 0; hg < HG; ++hg) {
+        float l = lt[hg];
+        l += __shfl_xor_sync(0xffffffffu, l, 4);
+        l += __shfl_xor_sync(0xffffffffu, l, 8);
+        l += __shfl_xor_sync(0xffffffffu, l, 16);
+        if (g == 0) {
+          ml[hg * 4 + t] = mt[hg];
+          ml[GMAX + hg * 4 + t] = l;
         }
       }
     }
@@ -1443,25 +1495,12 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
 // ============================================================================
 // host side
 // ============================================================================
-template <int HD, int HG, bool FLAT>
-static void launch_score_as(const ScoreDev& d, dim3 grid, cudaStream_t st) {
+template <int HD, int HG>
+static void launch_score(const ScoreDev& d, int groups_per_row, cudaStream_t st) {
   const int smem = SC_WARPS * PAGE * HD * 2 + SC_WARPS * 8 + 32;
-  ensure_dynamic_smem(reinterpret_cast<const void*>(&attn_score_kernel<HD, HG, FLAT>), smem);
-  SOL_LAUNCH("attn_score", (attn_score_kernel<HD, HG, FLAT>), grid, dim3(SC_WARPS * 32), smem, st, d);
-}
-// Direct 3-D grid while it stays within SC_MAX_GRID CTAs, else the flat numbering of the units that exist.
-template <int HD>
-static void launch_score(const ScoreDev& d, int HG, int groups_per_row, cudaStream_t st) {
-  const long long direct = (long long)groups_per_row * d.Hkv * d.B;
-  if (direct <= SC_MAX_GRID) {
-    const dim3 grid(groups_per_row, d.Hkv, d.B);
-    if (HG == 1) launch_score_as<HD, 1, false>(d, grid, st);
-    else launch_score_as<HD, 2, false>(d, grid, st);
-  } else {
-    const dim3 grid(SC_MAX_GRID);
-    if (HG == 1) launch_score_as<HD, 1, true>(d, grid, st);
-    else launch_score_as<HD, 2, true>(d, grid, st);
-  }
+  ensure_dynamic_smem(reinterpret_cast<const void*>(&attn_score_kernel<HD, HG>), smem);
+  const long long units = (long long)groups_per_row * d.Hkv * d.B, ctas = (long long)SC_PER_SM * sm_count();
+  SOL_LAUNCH("attn_score", (attn_score_kernel<HD, HG>), dim3((unsigned)(units < ctas ? units : ctas)), dim3(SC_WARPS * 32), smem, st, d);
 }
 
 // Persistent: one CTA per SM.
@@ -1486,7 +1525,7 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   pd.q_rot = a.q_rot; pd.q_split = static_cast<uint16_t*>(a.q_split); pd.work_ctr = a.work_ctr; pd.status = a.status;
   pd.row_hist = a.row_hist; pd.row_ctl = a.row_ctl; pd.kept_cnt = a.kept_cnt;
   pd.plan = a.plan; pd.r_permille = a.r_permille; pd.min_len = attn_split_len(hd);
-  pd.target_items = sm_count() * (hd == 64 ? 12 : 8);  // the pass-2 warps resident at once
+  pd.target_items = sm_count() * gather_warps(hd, 4 * HG);  // the pass-2 warps resident at once
   SOL_LAUNCH("attn_prep_rope_append", attn_prep_kernel, dim3(Hkv, a.B), dim3(PREP_THREADS), 0, st, pd);
 
   if (a.span_tokens > 0) {  // KV refresh: the rows are spans of one sequence's tokens, every token before a row's own is kept
@@ -1511,17 +1550,23 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   sd.q_split = static_cast<const uint16_t*>(a.q_split);
   sd.logits = a.logits; sd.sigma = a.sigma; sd.status = a.status; sd.B = a.B;
   const int groups_per_row = (a.kv.max_pages_per_seq + SC_WARPS - 1) / SC_WARPS;
-  if (hd == 64) launch_score<64>(sd, HG, groups_per_row, st);
-  else launch_score<128>(sd, HG, groups_per_row, st);
+  if (hd == 64) {
+    if (HG == 1) launch_score<64, 1>(sd, groups_per_row, st);
+    else launch_score<64, 2>(sd, groups_per_row, st);
+  } else {
+    if (HG == 1) launch_score<128, 1>(sd, groups_per_row, st);
+    else launch_score<128, 2>(sd, groups_per_row, st);
+  }
 
   SelectDev se;
   se.sh = sh; se.kv = a.kv; se.r_permille = a.r_permille; se.Tmax = Tmax; se.q_rot = a.q_rot; se.B = a.B;
   se.sigma = a.sigma; se.row_hist = a.row_hist; se.row_ctl = a.row_ctl; se.kept_cnt = a.kept_cnt;
-  se.status = a.status; se.plan = a.plan;
+  se.status = a.status; se.plan = a.plan; se.work_ctr = a.work_ctr;
   // persistent grid: a few CTAs per SM, never more than there can be units
   const long long sel_units = (long long)a.B * Hkv * ((Tmax + TH_SEG - 1) / TH_SEG), sel_res = (long long)sm_count() * TS_PER_SM;
+  ensure_dynamic_smem(reinterpret_cast<const void*>(&token_select_kernel), (int)sizeof(SelSmem));
   SOL_LAUNCH("token_select", token_select_kernel, dim3((unsigned)(sel_units < sel_res ? sel_units : sel_res)),
-             dim3(TS_THREADS), 0, st, se);
+             dim3(TS_THREADS), sizeof(SelSmem), st, se);
   if (a.kept_idx_out != nullptr) {
     ListDev ld;
     ld.sh = sh; ld.kv = a.kv; ld.r_permille = a.r_permille; ld.Tmax = Tmax; ld.sigma = a.sigma; ld.row_ctl = a.row_ctl;

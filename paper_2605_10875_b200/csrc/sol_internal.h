@@ -204,7 +204,7 @@ inline int attn_splits(int head_dim, int max_pages, int page_size) {
 }
 constexpr int PAGE = 64;  // tokens of a cache page
 // words of AttnArgs::work_ctr
-enum : int { WC_NEXT = 1, WC_CPI = 2, WC_DONE = 4 };
+enum : int { WC_SELECT = 0, WC_NEXT = 1, WC_CPI = 2, WC_DONE = 4 };
 
 struct AttnArgs {
   sol_shape_t shape;
@@ -234,7 +234,7 @@ struct AttnArgs {
   int splits;           // S = ceil(Tmax / attn_split_len(hd))
   int32_t* plan;        // [2][132] cumulative segment / item counts over the batch: the flat work lists of the selection
                         // and of pass 2, written by the query preparation
-  int32_t* work_ctr;    // [4 + B*Hkv]: unused, next item to claim, kept tokens per item, unused; then the finished
+  int32_t* work_ctr;    // [4 + B*Hkv]: next unit of the selection to claim, next pass-2 item to claim, kept tokens per item, unused; then the finished
                         // items of every (sequence, kv-head)
   // outputs (each optional)
   float* out_f32;    // [B][Hq][hd]

@@ -2,7 +2,7 @@
 import numpy as np
 import pytest
 
-from tests.test_gpu_parity import TINY, _mlp_case
+from tests.test_gpu_parity import TINY, _attention_case, _mlp_case
 
 pytestmark = pytest.mark.gpu
 
@@ -15,3 +15,21 @@ def test_down_rows_tiles(B, ff):
     rates = [1000, 999, 960, 500, 37, 0, 750, 875]
     _mlp_case(cfg, B, rates[:B], seed=ff + B)
     _mlp_case(cfg, B, rates[::-1][:B], seed=ff + B + 1)
+
+
+# The attention's passes at the edges of their tiles: 16-token steps and 64-token pages of the rows that keep every token,
+# 256-token chunks of the scores, rows around one selection segment (8192), runs of several items, forced sets wider than a
+# chunk, in every register layout (head_dim, heads per kv-head).
+@pytest.mark.parametrize("hd,hq,hkv", [(64, 4, 2), (64, 12, 4), (64, 8, 1), (128, 4, 2), (128, 8, 1), (128, 6, 2)])
+@pytest.mark.parametrize("sink,window", [(0, 1), (5, 300)])
+def test_attention_pass_edges(hd, hq, hkv, sink, window):
+    cfg = dict(TINY, head_dim=hd, n_q_heads=hq, n_kv_heads=hkv, d_model=768)
+    lens = [1, 15, 16, 17, 63, 65, 255, 257, 511, 769, 1025, 2049]
+    for seed, rates in ((1, [1000]), (2, [1000, 500, 125]), (3, [250, 1, 999])):
+        _attention_case(cfg, lens, np.resize(rates, len(lens)), seed=seed, n_sink=sink, n_window=window)
+
+
+@pytest.mark.parametrize("hd", [64, 128])
+def test_attention_rows_around_a_selection_segment(hd):
+    cfg = dict(TINY, head_dim=hd, n_q_heads=4, n_kv_heads=1, d_model=256)
+    _attention_case(cfg, [8191, 8192, 8193, 16385, 40], [125, 500, 250, 1000, 300], seed=hd)
