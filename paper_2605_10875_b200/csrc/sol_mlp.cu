@@ -8,9 +8,10 @@
 // the largest |g|, |u|.  channel_select_multi spreads every token over
 // ff/1024 CTAs: each finds the histogram bin that holds the m-th largest |t|,
 // keeps what lies above that bin (by more than the float32 error bound of t),
-// drops what lies below, and recomputes the few channels in between exactly
-// from the weight rows; the last CTA of a token ranks those candidates and
-// patches the kept ones in.  Outputs: the masked activations as two bf16
+// drops what lies below, and lists the channels in between; the last CTA of a
+// token ranks those candidates within their error bounds, recomputes the few
+// that the bounds leave open exactly from the weight rows, and patches the
+// kept ones in.  Outputs: the masked activations as two bf16
 // parts (hi + lo) for the tensor-core down projection, a keep mask, and the
 // "granule is live" flags that let the down projection skip weight rows
 // nobody keeps.  A token with more candidates than the list holds (massive
@@ -250,18 +251,109 @@ __global__ void __launch_bounds__(THREADS) channel_select_kernel(const ChanDev p
 // channel_select_multi
 // ============================================================================
 constexpr int CM_THREADS = 256;
-constexpr int CM_MAX_GROUPS = 2;  // groups of four channels per thread at most (template parameter of the kernel)
 
+constexpr int CM_EXACT = 32;
 struct ChanMultiSmem {
   int scan[CM_THREADS / 32];
-  int pick[2];
-  int n_local;
+  int pick;
+  int n_open;
   int flag;
-  int local_idx[CM_THREADS * 4 * CM_MAX_GROUPS];
-  __align__(16) uint16_t x[8192];  // the token's operand row (d_model <= 8192)
-  double val[CH_CAND_CAP];
+  float thr_hi, thr_lo;
   int idx[CH_CAND_CAP];
+  float2 av[CH_CAND_CAP];          // a candidate's float32 |t| and the bound of its error
+  double val[CH_CAND_CAP];         // its exact |t|; +-1e300 where the bounds settle it
+  int open[CH_CAND_CAP];           // the candidates to recompute
+  size_t row_off[CM_EXACT];        // of up to CM_EXACT of them: where their weight rows start, the rows' swizzle,
+  int row_swz[CM_EXACT];
+  double2 part[CM_EXACT][CM_THREADS / 32];  // the warps' sums of g and u
 };
+
+// The two bf16 numbers of a word as float64, by bits (a conversion instruction runs at a small fraction of this rate).  Zeros
+// and denormals come out as numbers of magnitude 2^-127 or less, which is nothing beside the sums' other terms.
+__device__ __forceinline__ double bf16_bits_to_f64(uint32_t high_half) {
+  const uint32_t hi = ((high_half >> 3) & 0x0fffe000u) + 0x38000000u;
+  return __hiloint2double((int)(hi | (high_half & 0x80000000u)), 0);
+}
+
+// Exact |t| of up to CM_EXACT open candidates, by the whole CTA: g_j = scale * sum_e x_e w_je with x the quantizer codes (or
+// the bf16 row), in float64.  A thread owns elements 8 tid .. + 7 of every 2048; the rows are on their way to L2 before the
+// first is read, and the next candidate's pieces travel while one is worked on.  One short rolled loop, because this
+// code runs cold: four candidates side by side, in float64 or in float pairs, gained at d_model 4096 what their code cost
+// at the other sizes (24 us here, 26 and 23 for 16 candidates of a Llama-8B layer; 2.0, 3.2 and 3.8 for one at d_model 256).
+__device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem& sm, int b, int i0, int n) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = p.d;
+  const uint32_t chunk_bytes = (uint32_t)p.R * 128;
+  if (tid < n) {  // where the candidate's gate row starts (its up row follows 128 bytes later)
+    const int row = 2 * sm.idx[sm.open[i0 + tid]], tile = row / p.R, r = row - tile * p.R;
+    sm.row_off[tid] = ((size_t)tile * p.chunks * p.R + r) * 128;
+    sm.row_swz[tid] = r & 7;
+  }
+  for (int i = tid; i < n * (CM_THREADS / 32); i += CM_THREADS) (&sm.part[0][0])[i] = make_double2(0.0, 0.0);
+  __syncthreads();
+  for (int q = tid; q < n * (d / 64); q += CM_THREADS) {  // 256 bytes of both rows per 64 elements
+    const int i = q / (d / 64), chunk = q - i * (d / 64);
+    const unsigned char* src = p.w_gu + sm.row_off[i] + (size_t)chunk * chunk_bytes;
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(src));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(src + 128));
+  }
+#pragma unroll 1
+  for (int base = 0; base < d; base += CM_THREADS * 8) {
+    const int e0 = base + tid * 8, piece = (e0 >> 3) & 7;
+    const bool in = e0 < d;
+    double x[8];
+    {
+      uint4 xv = make_uint4(0u, 0u, 0u, 0u);
+      if (in) xv = *reinterpret_cast<const uint4*>(p.a_op + act_piece_offset(p.Mpad, b, e0 >> 3));
+      const uint32_t xa[4] = {xv.x, xv.y, xv.z, xv.w};
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        x[2 * q] = in ? bf16_bits_to_f64(xa[q] << 16) : 0.0;
+        x[2 * q + 1] = in ? bf16_bits_to_f64(xa[q]) : 0.0;
+      }
+    }
+    const unsigned char* chunk_src = p.w_gu + (size_t)(e0 >> 6) * chunk_bytes;
+    uint4 g_next = make_uint4(0u, 0u, 0u, 0u), u_next = g_next;
+    auto load = [&](int i) {
+      if (in && i < n) {
+        const int swz = sm.row_swz[i];  // even: a gate row is an even row
+        g_next = *reinterpret_cast<const uint4*>(chunk_src + sm.row_off[i] + ((piece ^ swz) * 16));
+        u_next = *reinterpret_cast<const uint4*>(chunk_src + sm.row_off[i] + 128 + ((piece ^ (swz + 1)) * 16));
+      }
+    };
+    load(0);
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const uint32_t ga[4] = {g_next.x, g_next.y, g_next.z, g_next.w}, ua[4] = {u_next.x, u_next.y, u_next.z, u_next.w};
+      load(i + 1);
+      double g = 0.0, u = 0.0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        g = fma(x[2 * q], bf16_bits_to_f64(ga[q] << 16), g);
+        u = fma(x[2 * q], bf16_bits_to_f64(ua[q] << 16), u);
+        g = fma(x[2 * q + 1], bf16_bits_to_f64(ga[q]), g);
+        u = fma(x[2 * q + 1], bf16_bits_to_f64(ua[q]), u);
+      }
+      g = warp_sum_d(g);
+      u = warp_sum_d(u);
+      if (lane == 0) {
+        sm.part[i][warp].x += g;
+        sm.part[i][warp].y += u;
+      }
+    }
+  }
+  __syncthreads();
+  if (tid < n) {
+    double g = 0.0, u = 0.0;
+#pragma unroll
+    for (int w = 0; w < CM_THREADS / 32; ++w) {
+      g += sm.part[tid][w].x;
+      u += sm.part[tid][w].y;
+    }
+    const double sc = (double)p.scale[b], ag = g * sc, au = u * sc;
+    sm.val[sm.open[i0 + tid]] = fabs(ag / (1.0 + exp(-ag)) * au);
+  }
+  __syncthreads();
+}
 
 // CM_GROUPS: groups of four channels per thread, so CM_THREADS * 4 * CM_GROUPS channels per CTA: the launch takes
 // two groups when one group per thread would need more CTAs than are resident at once (a second, partly filled
@@ -272,16 +364,13 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
   __shared__ ChanMultiSmem sm;
   const int slice = blockIdx.x, b = blockIdx.y, S = gridDim.x;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int WARPS = CM_THREADS / 32;
   const int ff = p.ff, d = p.d;
   pdl_trigger();
   pdl_wait();
   uint32_t* sel = p.sel + (size_t)b * CH_SEL_WORDS;
   const int m = (int)(((long long)(1000 - p.p_permille[b]) * ff + 999) / 1000);
-  if (tid == 0) sm.n_local = 0;
   // What the later steps read is requested now, so that it arrives while the histogram is scanned: this CTA's
-  // channels of t (and of g, u when there is a selection to make) and the token's operand row for the exact
-  // re-scoring (into shared memory; a selection almost always leaves a few channels to re-score).
+  // channels of t (and of g, u when there is a selection to make).
   const bool selecting = m > 0 && m < ff;
   float4 v[CM_GROUPS], gq[CM_GROUPS], uq[CM_GROUPS];
 #pragma unroll
@@ -296,12 +385,9 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
       }
     }
   }
-  if (selecting)
-    for (int e = tid * 8; e < d; e += CM_THREADS * 8)
-      *reinterpret_cast<uint4*>(sm.x + e) = *reinterpret_cast<const uint4*>(p.a_op + act_piece_offset(p.Mpad, b, e >> 3));
 
   // ---- the histogram bin of the m-th largest |t| (every CTA of the token finds the same one) ----
-  // keep at or above hi_edge + e_j, drop below lo_edge - e_j, exact in between; e_j = eps * (1.1 |u_j| + |g_j|)
+  // keep at or above hi_edge + e_j, drop below lo_edge - e_j, listed in between; e_j = eps * (1.1 |u_j| + |g_j|)
   // bounds the error of this channel's own float32 |t|
   float hi_edge = 0.f, lo_edge = 0.f, eps = 0.f;
   if (m >= ff) {
@@ -312,14 +398,19 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
     lo_edge = INFINITY;
   } else {
     constexpr int BPT = CH_BINS / CM_THREADS;  // bins per thread, descending
+    static_assert(BPT == 16, "four 16-byte reads per thread");
+    const uint4* own = reinterpret_cast<const uint4*>(sel + CH_BINS - (tid + 1) * BPT);
+    const uint4 h0 = own[0], h1 = own[1], h2 = own[2], h3 = own[3];
+    const float gmax = __uint_as_float(sel[CH_GMAX]), umax = __uint_as_float(sel[CH_UMAX]);
+    const uint32_t hh[BPT] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w, h2.x, h2.y, h2.z, h2.w, h3.x, h3.y, h3.z, h3.w};
     int mine = 0;
 #pragma unroll
-    for (int q = 0; q < BPT; ++q) mine += (int)sel[CH_BINS - 1 - tid * BPT - q];
+    for (int q = 0; q < BPT; ++q) mine += (int)hh[q];
     int incl = mine;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o);
-      if (lane >= o) incl += v;
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
     }
     if (lane == 31) sm.scan[warp] = incl;
     __syncthreads();
@@ -327,19 +418,18 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
     for (int w = 0; w < warp; ++w) before += sm.scan[w];
     if (before < m && m <= before + mine) {
       int a = before;
-      for (int q = 0; q < BPT; ++q) {
-        const int bin = CH_BINS - 1 - tid * BPT - q;
-        const int c = (int)sel[bin];
-        if (m <= a + c) {
-          sm.pick[0] = bin;
-          break;
+      bool found = false;
+#pragma unroll
+      for (int q = BPT - 1; q >= 0; --q) {
+        a += (int)hh[q];
+        if (!found && m <= a) {
+          sm.pick = CH_BINS - (tid + 1) * BPT + q;
+          found = true;
         }
-        a += c;
       }
     }
     __syncthreads();
-    const int tb = sm.pick[0];
-    const float gmax = __uint_as_float(sel[CH_GMAX]), umax = __uint_as_float(sel[CH_UMAX]);
+    const int tb = sm.pick;
     const float bin_lo = chan_bin_lo(tb), bin_hi = tb >= CH_BINS - 1 ? INFINITY : chan_bin_lo(tb + 1);
     // error taken for g_j, u_j: the tensor cores add each 16-long slice of the dot product to the running
     // float32 sum with truncation, so the error grows with the d/16 steps: (d/16) * 2^-24 of the largest
@@ -376,7 +466,11 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
         ++n_above;
         any = true;
       } else if (a >= lo_edge - ej) {
-        sm.local_idx[atomicAdd(&sm.n_local, 1)] = j0 + e;
+        const uint32_t slot = atomicAdd(sel + CH_N_CAND, 1u);
+        if (slot < (uint32_t)CH_CAND_CAP) {
+          reinterpret_cast<float2*>(p.cand_val)[(size_t)b * CH_CAND_CAP + slot] = make_float2(a, ej + 2e-6f * a);  // and what the fast exponential and division add
+          p.cand_idx[(size_t)b * CH_CAND_CAP + slot] = j0 + e;
+        }
       }
     }
     if (in) {  // four channels: half a piece of the packed operand
@@ -387,72 +481,25 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
       if (any) p.live[j0 >> 5] = 1;
     }
   }
+  if (!selecting) {  // all or nothing: there is no candidate to wait for
+    if (slice == 0 && tid == 0) p.kept_cnt[b] = m >= ff ? ff : 0;
+    return;
+  }
   n_above = __reduce_add_sync(0xffffffffu, n_above);
   if (lane == 0 && n_above) atomicAdd(sel + CH_N_ABOVE, (uint32_t)n_above);
-  __syncthreads();
 
-  // ---- exact |t| of the channels in between, from the weight rows ----
-  // g_j = scale * sum_e x_e w_je with x the quantizer codes (or the bf16 row): every product of two bf16
-  // numbers is an exact float32, so the sums are gathered exactly in float pairs
-  const int n_local = sm.n_local;
-  if (n_local > 0) {
-    const double sc = (double)p.scale[b];
-    // the token's operand row (requested at the start) is in shared memory: the barrier above has passed
-    for (int c = warp; c < n_local; c += WARPS) {
-      const int j = sm.local_idx[c];
-      float gh = 0.f, gl = 0.f, uh = 0.f, ul = 0.f;
-      for (int e0 = lane * 8; e0 < d; e0 += 2048) {  // eight 256-wide slices of both rows per round, loads before uses
-        uint4 gv[8], uv[8];
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int e = e0 + r * 256;
-          if (e < d) {  // the piece of elements e .. e + 7 of the channel's gate row and of its up row
-            gv[r] = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j, e >> 6, (e >> 3) & 7));
-            uv[r] = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j + 1, e >> 6, (e >> 3) & 7));
-          }
-        }
-#pragma unroll
-        for (int r = 0; r < 8; ++r) {
-          const int e = e0 + r * 256;
-          if (e >= d) break;
-          const uint4 xv = *reinterpret_cast<const uint4*>(sm.x + e);
-          const uint32_t xa[4] = {xv.x, xv.y, xv.z, xv.w}, ga[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w},
-                         ua[4] = {uv[r].x, uv[r].y, uv[r].z, uv[r].w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float x0 = bf16_lo(xa[q]), x1 = bf16_hi(xa[q]);
-            pair_add(gh, gl, __fmul_rn(x0, bf16_lo(ga[q])));
-            pair_add(gh, gl, __fmul_rn(x1, bf16_hi(ga[q])));
-            pair_add(uh, ul, __fmul_rn(x0, bf16_lo(ua[q])));
-            pair_add(uh, ul, __fmul_rn(x1, bf16_hi(ua[q])));
-          }
-        }
-      }
-      const double ag = warp_sum_d((double)gh + (double)gl) * sc;
-      const double au = warp_sum_d((double)uh + (double)ul) * sc;
-      if (lane == 0) {
-        const uint32_t slot = atomicAdd(sel + CH_N_CAND, 1u);
-        if (slot < (uint32_t)CH_CAND_CAP) {
-          p.cand_val[(size_t)b * CH_CAND_CAP + slot] = fabs(ag / (1.0 + exp(-ag)) * au);
-          p.cand_idx[(size_t)b * CH_CAND_CAP + slot] = j;
-        }
-      }
-    }
-  }
-
-  // ---- the last CTA of the token ranks the candidates and patches the kept ones in ----
+  // ---- the last CTA of the token settles the candidates ----
   __threadfence();
   __syncthreads();
-  if (tid == 0) sm.flag = atomicAdd(sel + CH_DONE, 1u) == (uint32_t)(S - 1) ? 1 : 0;
+  if (tid == 0) {
+    sm.flag = atomicAdd(sel + CH_DONE, 1u) == (uint32_t)(S - 1) ? 1 : 0;
+    sm.n_open = 0;
+  }
   __syncthreads();
   if (!sm.flag) return;
   __threadfence();
   const int n_cand = (int)__ldcg(sel + CH_N_CAND);
   const int need = m - (int)__ldcg(sel + CH_N_ABOVE);
-  if (m >= ff || m <= 0) {
-    if (tid == 0) p.kept_cnt[b] = m >= ff ? ff : 0;
-    return;
-  }
   if (n_cand > CH_CAND_CAP || need < 0 || need > n_cand) {  // more candidates than the list holds: redo the token
     if (tid == 0) {
       sel[CH_FALLBACK] = 1u;
@@ -461,19 +508,61 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
     return;
   }
   for (int c = tid; c < n_cand; c += CM_THREADS) {
-    sm.val[c] = __ldcg(p.cand_val + (size_t)b * CH_CAND_CAP + c);
+    sm.av[c] = __ldcg(reinterpret_cast<const float2*>(p.cand_val) + (size_t)b * CH_CAND_CAP + c);
     sm.idx[c] = __ldcg(p.cand_idx + (size_t)b * CH_CAND_CAP + c);
+  }
+  if (tid == 0) {
+    sm.thr_hi = -INFINITY;  // need == 0: every candidate lies above "the" threshold's bounds nowhere
+    sm.thr_lo = INFINITY;
+  }
+  __syncthreads();
+  // the need-th largest exact |t| of the list lies between the need-th largest of |t| - e and the need-th largest of
+  // |t| + e (four threads per candidate; equal values rank by position, any of them gives the same number)
+  if (need > 0) {
+    for (int c0 = 0; c0 < n_cand; c0 += CM_THREADS / 4) {
+      const int c = c0 + (tid >> 2);
+      const float2 a = c < n_cand ? sm.av[c] : make_float2(0.f, 0.f);
+      const float lo = a.x - a.y, hi = a.x + a.y;
+      int rank_lo = 0, rank_hi = 0;
+      for (int o = tid & 3; o < n_cand; o += 4) {
+        const float2 x = sm.av[o];
+        rank_lo += (x.x - x.y > lo) || (x.x - x.y == lo && o < c);
+        rank_hi += (x.x + x.y > hi) || (x.x + x.y == hi && o < c);
+      }
+      rank_lo += __shfl_xor_sync(0xffffffffu, rank_lo, 1);
+      rank_hi += __shfl_xor_sync(0xffffffffu, rank_hi, 1);
+      rank_lo += __shfl_xor_sync(0xffffffffu, rank_lo, 2);
+      rank_hi += __shfl_xor_sync(0xffffffffu, rank_hi, 2);
+      if (c < n_cand && rank_lo == need - 1) sm.thr_lo = lo;
+      if (c < n_cand && rank_hi == need - 1) sm.thr_hi = hi;
+    }
+  } else if (tid == 0) {
+    sm.thr_hi = INFINITY;  // nothing is kept: every candidate lies below
   }
   __syncthreads();
   for (int c = tid; c < n_cand; c += CM_THREADS) {
-    const double vc = sm.val[c];
-    const int j = sm.idx[c];
+    const float2 a = sm.av[c];
+    double val = 1e300;                          // surely kept
+    if (a.x + a.y < sm.thr_lo) val = -1e300;     // surely dropped
+    else if (!(a.x - a.y > sm.thr_hi)) sm.open[atomicAdd(&sm.n_open, 1)] = c;
+    sm.val[c] = val;
+  }
+  __syncthreads();
+  const int n_open = sm.n_open;
+#pragma unroll 1
+  for (int i0 = 0; i0 < n_open; i0 += CM_EXACT) exact_candidates(p, sm, b, i0, min(CM_EXACT, n_open - i0));
+  for (int c0 = 0; c0 < n_cand; c0 += CM_THREADS / 4) {
+    const int c = c0 + (tid >> 2);
+    const double vc = c < n_cand ? sm.val[c] : 0.0;
+    const int j = c < n_cand ? sm.idx[c] : 0;
     int rank = 0;
-    for (int o = 0; o < n_cand; ++o) {
+    for (int o = tid & 3; o < n_cand; o += 4) {
       const double vo = sm.val[o];
       rank += (vo > vc) || (vo == vc && sm.idx[o] < j);
     }
-    if (rank < need) {
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if (c < n_cand && rank < need && (tid & 3) == 0) {
       const float tv = p.t[(size_t)b * ff + j];
       const uint16_t hv = f2bf(tv);
       uint16_t* dst = reinterpret_cast<uint16_t*>(p.t_op + act_piece_offset(2 * p.Mpad, b, j >> 3) + (j & 7) * 2);
@@ -485,7 +574,7 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
   }
   if (tid == 0) {
     p.kept_cnt[b] = m;
-    atomicAdd(p.status + ST_CH_REFINED, n_cand);
+    atomicAdd(p.status + ST_CH_REFINED, n_open);
   }
 }
 

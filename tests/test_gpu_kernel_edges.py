@@ -33,3 +33,17 @@ def test_attention_pass_edges(hd, hq, hkv, sink, window):
 def test_attention_rows_around_a_selection_segment(hd):
     cfg = dict(TINY, head_dim=hd, n_q_heads=4, n_kv_heads=1, d_model=256)
     _attention_case(cfg, [8191, 8192, 8193, 16385, 40], [125, 500, 250, 1000, 300], seed=hd)
+
+
+# The exact re-scoring of the channel selection: rows shorter than, equal to and longer than what a CTA takes at once (2048
+# elements), and more open candidates than one pass takes (groups of identical channels around the threshold).
+@pytest.mark.parametrize("d,ff", [(256, 1056), (2048, 512), (2304, 512), (4096, 1024), (8192, 256)])
+def test_channel_selection_exact_rescoring(d, ff):
+    cfg = dict(TINY, d_model=d, d_ff=ff)
+
+    def groups(w):  # channels in runs of 40 equal ones: the threshold falls inside a run
+        w.w_gate[:] = w.w_gate[(np.arange(ff) // 40) * 40]
+        w.w_up[:] = w.w_up[(np.arange(ff) // 40) * 40]
+
+    _mlp_case(cfg, 3, [500, 250, 900], seed=d)
+    _mlp_case(cfg, 2, [500, 730], seed=d + 1, mutate=groups)
