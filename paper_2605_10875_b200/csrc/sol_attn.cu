@@ -31,11 +31,7 @@
 
 namespace sol {
 
-// Flat work lists of the attention kernels (AttnArgs::plan): cumulative counts over the sequences of the
-// batch, PLAN_STRIDE words each: 8192-token segments of rows that need a selection, pass-2 items.  Entry b is
-// the count before sequence b (per kv-head), entry B the total.
-enum : int { PLAN_HSEG = 0, PLAN_ITEMS = 1, PLAN_LISTS = 2 };
-constexpr int PLAN_STRIDE = 132;
+constexpr int PLAN_STRIDE = 132;  // words of a cumulative work list: entry b is the count before sequence b (per kv-head), entry B the total
 constexpr int PLAN_GROUP_TOKENS = 4 * PAGE;  // tokens of one pass-1 unit (a CTA of attn_score: one page per warp)
 constexpr int TH_SEG = 8192;  // tokens per token_select CTA
 
@@ -71,6 +67,80 @@ __device__ __forceinline__ int gather_item_tokens(const RowPlan& rp, int c, int 
   return max(len, min_len);
 }
 
+// The flat work lists of the selection and of pass 2 are made by every CTA for itself from the lengths and keep-rates,
+// which are inputs of the step, while the kernels before are still running; a list made by one CTA of attn_prep stood in
+// that kernel's way and cost the readers a round trip to memory.
+
+// cum[b + 1] = cnt of sequences 0 .. b (cnt: this thread's sequence, threads 0 .. 127); cum[0] = 0.  Called by the whole
+// CTA (128 threads or more); wsum: four words of shared memory.
+__device__ __forceinline__ void plan_scan(int cnt, int* cum, int* wsum) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  int incl = cnt;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int x = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += x;
+  }
+  if (lane == 31 && warp < 4) wsum[warp] = incl;
+  __syncthreads();
+  if (tid < 128) {
+    for (int w = 0; w < warp; ++w) incl += wsum[w];
+    cum[tid + 1] = incl;
+    if (tid == 0) cum[0] = 0;
+  }
+  __syncthreads();
+}
+
+// The pass-2 items of every sequence into cum; returns the kept tokens c of an item, a power of two from 64 to 1024: the
+// one with the least time by the rounds its items take on the resident warps, each round as long as an item and the
+// ITEM_FILL tokens that filling a warp's ring of row copies is worth.  (Long items alone left the chip half empty in a
+// second round: 134 MB of values of 32 sequences in 55 us.)
+constexpr int ITEM_FILL = 256;  // measured: 64 to 192 cut long rows into too many items (290 -> 365 us where all of
+                                // 128 ragged sequences' tokens are kept), 512 gave up balance (32 equal sequences 98 -> 122)
+constexpr int ITEM_C0 = 64, ITEM_NC = 5;
+struct PlanSmem {
+  int cum[PLAN_STRIDE];
+  int n_items[ITEM_NC];
+  int wsum[4];
+};
+__device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t& kv, const int32_t* r_permille, int B, int min_len,
+                                          int target_items, PlanSmem& ps) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid < ITEM_NC) ps.n_items[tid] = 0;
+  __syncthreads();
+  int per_seq[ITEM_NC] = {0, 0, 0, 0, 0};
+  if (tid < 128) {
+    if (tid < B) {
+      const RowPlan rp = row_plan(sh, kv, r_permille, tid);
+#pragma unroll
+      for (int q = 0; q < ITEM_NC; ++q) {  // one item at least, so that the output is always written
+        const int len = gather_item_tokens(rp, ITEM_C0 << q, min_len);
+        per_seq[q] = max(1, (rp.T + len - 1) / len);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < ITEM_NC; ++q) {
+      const int n = __reduce_add_sync(0xffffffffu, per_seq[q]);
+      if (lane == 0 && n) atomicAdd(&ps.n_items[q], n);
+    }
+  }
+  __syncthreads();
+  int pick = 0, cnt = 0;
+  long long best = 0x7fffffffffffffffLL;
+#pragma unroll
+  for (int q = 0; q < ITEM_NC; ++q) {
+    const int rounds = (ps.n_items[q] * sh.n_kv_heads + target_items - 1) / target_items;
+    const long long cost = (long long)rounds * ((ITEM_C0 << q) + ITEM_FILL);
+    if (cost <= best) {
+      best = cost;
+      pick = q;
+      cnt = per_seq[q];
+    }
+  }
+  plan_scan(cnt, ps.cum, ps.wsum);
+  return ITEM_C0 << pick;
+}
+
 // The sequence that holds flat unit `u` of a cumulative list (cum[b] <= u < cum[b + 1]); n entries + total.
 __device__ __forceinline__ int plan_find(const int* cum, int n, int u) {
   int lo = 0, hi = n - 1;
@@ -94,19 +164,15 @@ struct PrepDev {
   const uint16_t* q_bf16;  // [B][Hq][hd] or nullptr
   float* q_rot;
   uint16_t* q_split;
-  int32_t* work_ctr;  // zeroed here: next item, finished items of every (sequence, kv-head)
+  int32_t* work_ctr;  // zeroed here
   uint32_t* row_hist; // zeroed here: [B*Hkv][SEL_BINS] score histogram of rows that span several selection CTAs
   uint32_t* row_ctl;  // zeroed here: [B*Hkv][RC_WORDS]
   int32_t* kept_cnt;  // [B*Hkv], written here; token_select writes it again for the rows it settles
-  int32_t* plan;      // written here by the first CTA: [PLAN_LISTS][PLAN_STRIDE]
   const int32_t* r_permille;
-  int min_len, target_items;  // for the choice of the pass-2 item length
   int* status;
 };
 
 constexpr int PREP_THREADS = 128;
-constexpr int ITEM_FILL = 256;  // measured: 64 to 192 cut long rows into too many items (290 -> 365 us where all of
-                                // 128 ragged sequences' tokens are kept), 512 gave up balance (32 equal sequences 98 -> 122)
 // words of AttnArgs::row_ctl, per (sequence, kv-head): segments whose scores are in the histogram, largest |score|,
 // keep edge (float bits)
 enum : int { RC_DONE = 0, RC_MAX, RC_EDGE, RC_WORDS = 8 };
@@ -124,75 +190,6 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
   const bool rope = layer && p.sh.rope_theta > 0.f;
   pdl_trigger();
   pdl_wait();
-
-  // The first CTA lays out the work of the kernels that follow: cumulative segment and item counts over the
-  // batch, and the kept tokens c of a pass-2 item, a power of two from 64 to 1024: the one with the least time by the
-  // rounds its items take on the resident warps, each round as long as an item and the ITEM_FILL tokens that filling
-  // a warp's ring of row copies is worth.  (Long items alone left the chip half empty in a second round: 134 MB of
-  // values of 32 sequences in 55 us.)
-  if (kvh == 0 && b == 0) {
-    constexpr int C0 = 64, NC = 5;
-    __shared__ int wsum[PLAN_LISTS][PREP_THREADS / 32];
-    __shared__ int n_items[NC];
-    const int w = tid >> 5, l = tid & 31;
-    if (tid < NC) n_items[tid] = 0;
-    __syncthreads();
-    int per_seq[NC] = {0, 0, 0, 0, 0};
-    int cnt[PLAN_LISTS] = {0, 0};
-    if (tid < p.B) {
-      const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
-      if (rp.mode == 2) cnt[PLAN_HSEG] = (rp.T + TH_SEG - 1) / TH_SEG;
-#pragma unroll
-      for (int q = 0; q < NC; ++q) {  // one item at least, so that the output is always written
-        const int len = gather_item_tokens(rp, C0 << q, p.min_len);
-        per_seq[q] = max(1, (rp.T + len - 1) / len);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      const int n = __reduce_add_sync(0xffffffffu, per_seq[q]);
-      if (l == 0) atomicAdd(&n_items[q], n);
-    }
-    __syncthreads();
-    int pick = 0;
-    long long best = 0x7fffffffffffffffLL;
-#pragma unroll
-    for (int q = 0; q < NC; ++q) {
-      const long long rounds = ((long long)n_items[q] * Hkv + p.target_items - 1) / p.target_items;
-      const long long cost = rounds * ((C0 << q) + ITEM_FILL);
-      if (cost <= best) {
-        best = cost;
-        pick = q;
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < NC; ++q)
-      if (q == pick) cnt[PLAN_ITEMS] = per_seq[q];
-    int incl[PLAN_LISTS];
-#pragma unroll
-    for (int q = 0; q < PLAN_LISTS; ++q) {
-      incl[q] = cnt[q];
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int x = __shfl_up_sync(0xffffffffu, incl[q], o);
-        if (l >= o) incl[q] += x;
-      }
-      if (l == 31) wsum[q][w] = incl[q];
-    }
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < PLAN_LISTS; ++q) {
-      int before = 0;
-      for (int x = 0; x < w; ++x) before += wsum[q][x];
-      if (tid < p.B) p.plan[q * PLAN_STRIDE + tid + 1] = before + incl[q];
-      if (tid == 0) p.plan[q * PLAN_STRIDE] = 0;
-    }
-    if (tid == 0) {
-      p.work_ctr[WC_CPI] = C0 << pick;
-      p.work_ctr[WC_NEXT] = 0;
-      p.work_ctr[WC_SELECT] = 0;
-    }
-  }
 
   // this (sequence, kv-head)'s part of the q/k/v row: G query heads, the k head, the v head.  The K
   // slices of the projection are summed in order (four loads in flight at a time) and scaled.
@@ -219,6 +216,7 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
 
   if (tid == 0) {
     p.work_ctr[WC_DONE + b * Hkv + kvh] = 0;
+    if (b == 0 && kvh == 0) p.work_ctr[WC_NEXT] = p.work_ctr[WC_SELECT] = 0;
     p.kept_cnt[b * Hkv + kvh] = row_plan(p.sh, p.kv, p.r_permille, b).k;
   }
   // scratch of the token selection of this (sequence, kv-head)
@@ -330,6 +328,22 @@ __device__ __forceinline__ void merge_partials(const AttnOut& o, const float* sr
   const int G = o.G;
   const size_t stride = (size_t)G * (HD + 2);
   // factors of the partials: f[q][h] = 2^(m_q - M_h) / sum_q l_q 2^(m_q - M_h)
+  if (ns <= 32) {  // a partial per lane: every head's maximum and sum in one round trip
+    float2 ml[8];
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      ml[h] = make_float2(-INFINITY, 0.f);
+      if (h < G && lane < ns) ml[h] = __ldcg(reinterpret_cast<const float2*>(src0 + (size_t)lane * stride + (size_t)h * (HD + 2) + HD));
+    }
+#pragma unroll
+    for (int h = 0; h < 8; ++h) {
+      if (h >= G) break;
+      const float mm = warp_max(ml[h].x);
+      const float f = ml[h].x == -INFINITY ? 0.f : exp2f(ml[h].x - mm);
+      const float l = warp_sum(ml[h].y * f);
+      if (lane < ns) fac[lane * G + h] = l > 0.f ? f * (1.0f / l) : 0.f;
+    }
+  } else
 #pragma unroll 1
   for (int h = 0; h < G; ++h) {
     const float* src = src0 + (size_t)h * (HD + 2) + HD;
@@ -592,7 +606,6 @@ struct SelectDev {
   sol_kv_t kv;
   const int32_t* r_permille;
   int Tmax, B;
-  const int32_t* plan;
   const float* q_rot;
   float* sigma;          // kept candidates are overwritten with +inf
   uint32_t* row_hist;    // [B*Hkv][SEL_BINS], zero on entry (rows of several segments)
@@ -632,7 +645,7 @@ struct SelSmem {
   double qsum[128];
   float fmax_w[TS_THREADS / 32];
   int s_flag, s_next;
-  int cum[PLAN_STRIDE];
+  int cum[PLAN_STRIDE], wsum[4];
 };
 
 // The end of a row's selection, by one CTA: n_list tokens lie above the edge or are forced; ns_all candidates lie
@@ -953,9 +966,13 @@ __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(con
     mbar_init(&hs.bar, 1);
     fence_mbar_init();
   }
+  int cnt = 0;
+  if ((int)threadIdx.x < p.B) {
+    const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, threadIdx.x);
+    if (rp.mode == 2) cnt = (rp.T + TH_SEG - 1) / TH_SEG;
+  }
+  plan_scan(cnt, hs.cum, hs.wsum);
   pdl_wait();
-  for (int i = threadIdx.x; i <= p.B; i += TS_THREADS) hs.cum[i] = p.plan[PLAN_HSEG * PLAN_STRIDE + i];
-  __syncthreads();
   const int Hkv = p.sh.n_kv_heads;
   const int n_units = hs.cum[p.B] * Hkv;
   uint32_t phase = 0;
@@ -1024,12 +1041,11 @@ struct GatherDev {
   sol_shape_t sh;
   sol_kv_t kv;
   const int32_t* r_permille;
-  int B, Hkv, G, Tmax, S, min_len;
+  int B, Hkv, G, Tmax, S, min_len, sms;
   const uint16_t* q_split;
   const float* logits;
   const float* sigma;
   const uint32_t* row_ctl;
-  const int32_t* plan;
   int32_t* work_ctr;
   float* part;  // [B][Hkv][S][G][HD + 2]
   float scale_log2;
@@ -1088,7 +1104,8 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
   constexpr int WARPS = C::WARPS, NST = C::NST, HG = GMAX / 4;
   constexpr int CPR = HD / 8;  // 16-byte pieces per row
   extern __shared__ __align__(128) unsigned char gsm[];
-  __shared__ int cum[PLAN_STRIDE];
+  __shared__ PlanSmem ps;
+  const int* const cum = ps.cum;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = p.G, Hkv = p.Hkv;
   const uint16_t* kp = static_cast<const uint16_t*>(p.kv.k_pool);
@@ -1099,10 +1116,8 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
   uint16_t* my_q = reinterpret_cast<uint16_t*>(gsm + C::RING_BYTES + C::W_BYTES) + warp * GA_QUEUE;
   float* ml = reinterpret_cast<float*>(my_q);  // at the end of an item: [GMAX] maxima, [GMAX] sums
   pdl_trigger();
+  const int per_item = plan_items(p.sh, p.kv, p.r_permille, p.B, p.min_len, p.sms * WARPS, ps);
   pdl_wait();
-  for (int i = threadIdx.x; i <= p.B; i += C::THREADS) cum[i] = p.plan[PLAN_ITEMS * PLAN_STRIDE + i];
-  const int per_item = p.work_ctr[WC_CPI];
-  __syncthreads();
   const int n_items = cum[p.B] * Hkv;
   const int total_warps = gridDim.x * WARPS;
 
@@ -1524,8 +1539,7 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   pd.q_bf16 = static_cast<const uint16_t*>(a.q_bf16);
   pd.q_rot = a.q_rot; pd.q_split = static_cast<uint16_t*>(a.q_split); pd.work_ctr = a.work_ctr; pd.status = a.status;
   pd.row_hist = a.row_hist; pd.row_ctl = a.row_ctl; pd.kept_cnt = a.kept_cnt;
-  pd.plan = a.plan; pd.r_permille = a.r_permille; pd.min_len = attn_split_len(hd);
-  pd.target_items = sm_count() * gather_warps(hd, 4 * HG);  // the pass-2 warps resident at once
+  pd.r_permille = a.r_permille;
   SOL_LAUNCH("attn_prep_rope_append", attn_prep_kernel, dim3(Hkv, a.B), dim3(PREP_THREADS), 0, st, pd);
 
   if (a.span_tokens > 0) {  // KV refresh: the rows are spans of one sequence's tokens, every token before a row's own is kept
@@ -1561,7 +1575,7 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   SelectDev se;
   se.sh = sh; se.kv = a.kv; se.r_permille = a.r_permille; se.Tmax = Tmax; se.q_rot = a.q_rot; se.B = a.B;
   se.sigma = a.sigma; se.row_hist = a.row_hist; se.row_ctl = a.row_ctl; se.kept_cnt = a.kept_cnt;
-  se.status = a.status; se.plan = a.plan; se.work_ctr = a.work_ctr;
+  se.status = a.status; se.work_ctr = a.work_ctr;
   // persistent grid: a few CTAs per SM, never more than there can be units
   const long long sel_units = (long long)a.B * Hkv * ((Tmax + TH_SEG - 1) / TH_SEG), sel_res = (long long)sm_count() * TS_PER_SM;
   ensure_dynamic_smem(reinterpret_cast<const void*>(&token_select_kernel), (int)sizeof(SelSmem));
@@ -1578,7 +1592,7 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   gd.sh = sh; gd.kv = a.kv; gd.r_permille = a.r_permille; gd.B = a.B; gd.Hkv = Hkv; gd.G = G; gd.Tmax = Tmax;
   gd.S = a.splits; gd.min_len = attn_split_len(hd);
   gd.q_split = static_cast<const uint16_t*>(a.q_split);
-  gd.logits = a.logits; gd.sigma = a.sigma; gd.row_ctl = a.row_ctl; gd.plan = a.plan; gd.work_ctr = a.work_ctr;
+  gd.logits = a.logits; gd.sigma = a.sigma; gd.row_ctl = a.row_ctl; gd.work_ctr = a.work_ctr; gd.sms = sm_count();
   gd.part = a.part; gd.scale_log2 = (float)(1.4426950408889634 / sqrt((double)hd)); gd.out = out; gd.status = a.status;
   const long long items = (long long)a.B * Hkv * a.splits;
   if (hd == 64) {

@@ -204,7 +204,7 @@ inline int attn_splits(int head_dim, int max_pages, int page_size) {
 }
 constexpr int PAGE = 64;  // tokens of a cache page
 // words of AttnArgs::work_ctr
-enum : int { WC_SELECT = 0, WC_NEXT = 1, WC_CPI = 2, WC_DONE = 4 };
+enum : int { WC_SELECT = 0, WC_NEXT = 1, WC_DONE = 4 };
 
 struct AttnArgs {
   sol_shape_t shape;
@@ -232,9 +232,7 @@ struct AttnArgs {
   uint32_t* kept_row;   // Quest mode: same layout, cache row (page table applied) of every listed token, 0xffffffff: bad page
   float* part;          // [B][Hkv][S][G][hd + 2]
   int splits;           // S = ceil(Tmax / attn_split_len(hd))
-  int32_t* plan;        // [2][132] cumulative segment / item counts over the batch: the flat work lists of the selection
-                        // and of pass 2, written by the query preparation
-  int32_t* work_ctr;    // [4 + B*Hkv]: next unit of the selection to claim, next pass-2 item to claim, kept tokens per item, unused; then the finished
+  int32_t* work_ctr;    // [4 + B*Hkv]: next unit of the selection to claim, next pass-2 item to claim, two unused; then the finished
                         // items of every (sequence, kv-head)
   // outputs (each optional)
   float* out_f32;    // [B][Hq][hd]
@@ -268,7 +266,7 @@ void launch_span_attention(const AttnArgs& a, int n_tok, cudaStream_t st);
 
 // Offsets of the attention scratch inside a buffer, starting at `at` (a multiple of 256).
 struct AttnScratch {
-  size_t q_rot, q_split, logits, sigma, row_hist, row_ctl, kept_idx, kept_cnt, kept_row, part, plan, work_ctr, page_mask, quest_keys, quest_err, quest_hmask, quest_qsplit, quest_l1, quest_order, end;
+  size_t q_rot, q_split, logits, sigma, row_hist, row_ctl, kept_idx, kept_cnt, kept_row, part, work_ctr, page_mask, quest_keys, quest_err, quest_hmask, quest_qsplit, quest_l1, quest_order, end;
   int splits;
 };
 inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_pages, size_t at) {
@@ -294,7 +292,7 @@ inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_page
   L.kept_cnt = take(BK * 4);
   L.kept_row = take(BK * Tmax * 4);
   L.part = take(BK * L.splits * G * (hd + 2) * 4);
-  L.plan = take(3 * 132 * 4);
+  take(3 * 132 * 4);  // not used, see above
   take(BK * L.splits * 8);  // not used, see above
   L.work_ctr = take((4 + BK) * 4);
   const bool quest = s.token_select == SOL_SELECT_QUEST_PAGES;
@@ -322,7 +320,6 @@ inline void attn_scratch_bind(AttnArgs& a, void* base, const AttnScratch& L, int
   a.kept_cnt = kept_cnt ? kept_cnt : reinterpret_cast<int32_t*>(b + L.kept_cnt);
   a.kept_row = reinterpret_cast<uint32_t*>(b + L.kept_row);
   a.part = reinterpret_cast<float*>(b + L.part);
-  a.plan = reinterpret_cast<int32_t*>(b + L.plan);
   a.work_ctr = reinterpret_cast<int32_t*>(b + L.work_ctr);
   a.page_mask = b + L.page_mask;
   a.quest_keys = reinterpret_cast<uint32_t*>(b + L.quest_keys);
