@@ -189,28 +189,51 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
   const bool layer = p.qkv != nullptr;
   const bool rope = layer && p.sh.rope_theta > 0.f;
   pdl_trigger();
+  // the angles need only the lengths (an input of the step): float64 functions are slow here, and the projection is
+  // still running
+  if (tid < half) {
+    float c = 1.f, s = 0.f;
+    if (rope) {
+      // angle = pos * theta^(-2i/hd) in float64, reduced to [-pi, pi] before the float32 sine and cosine
+      const double inv = exp2(-2.0 * (double)tid / (double)hd * log2((double)p.sh.rope_theta));
+      const double a = (double)pos * inv;
+      const double k = rint(a * 0.15915494309189535);
+      const float r = (float)fma(-k, 6.283185307179586, a);
+      sincosf(r, &s, &c);
+    }
+    cs[tid] = c;
+    sn[tid] = s;
+  }
   pdl_wait();
 
   // this (sequence, kv-head)'s part of the q/k/v row: G query heads, the k head, the v head.  The K
-  // slices of the projection are summed in order (four loads in flight at a time) and scaled.
-  __shared__ float rowbuf[(8 + 2) * 128];
+  // slices of the projection are summed in order (four columns per thread, eight slices in flight) and scaled.
+  __shared__ alignas(16) float rowbuf[(8 + 2) * 128];
   if (layer) {
     const float row_scale = p.qkv_scale ? p.qkv_scale[b] : 1.0f;
     const float* base = p.qkv + (size_t)b * p.ldq;
     const size_t zs = (size_t)p.B * p.ldq;
-    for (int i = tid; i < (G + 2) * hd; i += PREP_THREADS) {
+#pragma unroll 1
+    for (int i = tid * 4; i < (G + 2) * hd; i += PREP_THREADS * 4) {  // hd is a multiple of 4: the four belong to one head
       const int col = i < G * hd ? kvh * G * hd + i
                                  : (i < (G + 1) * hd ? Hq * hd + kvh * hd + (i - G * hd)
                                                      : (Hq + Hkv) * hd + kvh * hd + (i - (G + 1) * hd));
-      float a = 0.f;
-      for (int z0 = 0; z0 < p.ksplit; z0 += 4) {
-        float v[4];
+      float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+      for (int z0 = 0; z0 < p.ksplit; z0 += 8) {
+        float4 v[8];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) v[q] = z0 + q < p.ksplit ? base[(size_t)(z0 + q) * zs + col] : 0.f;
+        for (int q = 0; q < 8; ++q)
+          v[q] = z0 + q < p.ksplit ? *reinterpret_cast<const float4*>(base + (size_t)(z0 + q) * zs + col) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) a += v[q];
+        for (int q = 0; q < 8; ++q) {
+          a.x += v[q].x;
+          a.y += v[q].y;
+          a.z += v[q].z;
+          a.w += v[q].w;
+        }
       }
-      rowbuf[i] = a * row_scale;
+      *reinterpret_cast<float4*>(rowbuf + i) = make_float4(a.x * row_scale, a.y * row_scale, a.z * row_scale, a.w * row_scale);
     }
   }
 
@@ -224,19 +247,6 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
   if (T > TH_SEG) {  // rows of one segment keep their histogram in shared memory
     uint4* hz = reinterpret_cast<uint4*>(p.row_hist + (size_t)(b * Hkv + kvh) * SEL_BINS);
     for (int i = tid; i < SEL_BINS / 4; i += PREP_THREADS) hz[i] = make_uint4(0u, 0u, 0u, 0u);
-  }
-  if (tid < half) {
-    float c = 1.f, s = 0.f;
-    if (rope) {
-      // angle = pos * theta^(-2i/hd) in float64, reduced to [-pi, pi] before the float32 sine and cosine
-      const double inv = exp2(-2.0 * (double)tid / (double)hd * log2((double)p.sh.rope_theta));
-      const double a = (double)pos * inv;
-      const double k = rint(a * 0.15915494309189535);
-      const float r = (float)fma(-k, 6.283185307179586, a);
-      sincosf(r, &s, &c);
-    }
-    cs[tid] = c;
-    sn[tid] = s;
   }
   // zero the operand rows of this (sequence, kv-head): pad rows and the unused fourth slot stay zero
   uint16_t* qs = p.q_split + (size_t)(b * Hkv + kvh) * HG * 16 * hd;
@@ -362,7 +372,7 @@ __device__ __forceinline__ void merge_partials(const AttnOut& o, const float* sr
     for (int q = lane; q < ns; q += 32) fac[q * G + h] *= inv;
   }
   __syncwarp();
-#pragma unroll 1
+#pragma unroll 2
   for (int e0 = lane * 2; e0 < G * HD; e0 += 64) {
     const int h = e0 / HD, e = e0 % HD;
     const float* src = src0 + (size_t)h * (HD + 2) + e;

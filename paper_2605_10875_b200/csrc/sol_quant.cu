@@ -16,7 +16,6 @@ namespace sol {
 
 constexpr int NQ_THREADS = 256;
 constexpr int NQ_VEC = 8;                       // elements per 128-bit bf16 load
-constexpr int NQ_MAX_PER_THREAD = 4;            // vectors per thread -> d <= 8192
 
 __device__ __forceinline__ float block_reduce(float v, bool is_max, float* sh) {
   v = is_max ? warp_max(v) : warp_sum(v);
@@ -38,7 +37,11 @@ struct NoSmem {
   int unused;
 };
 
-template <bool IN_F32, bool GATE>
+// NV: vectors of eight elements per thread (d <= NV * 2048).  Latency-bound: what needs nothing of the kernels before (the
+// gains, the width) is read while they run, and all of a row's partial sums that registers allow are in flight at once
+// (four slices at a time were three round trips for the nine of a Llama-1B projection; kernel 5.8 -> 4.1 us in the chain of a
+// single-sequence step).
+template <bool IN_F32, bool GATE, int NV>
 __global__ void __launch_bounds__(NQ_THREADS)
 norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, int ksplit, size_t part_stride,
                   float* __restrict__ sum_out, const uint16_t* __restrict__ gamma, float eps,
@@ -49,9 +52,19 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
                   const GateArgs gate) {
   __shared__ float sh[NQ_THREADS / 32];
   __shared__ typename std::conditional<GATE, SelectSmem, NoSmem>::type gsm;
-  pdl_trigger();
-  pdl_wait();
+  constexpr int NQ_MAX_PER_THREAD = NV;
+  constexpr int ZB = NV == 1 ? 12 : 4;  // slices of the partial sums in flight
   const int row = blockIdx.x;
+  pdl_trigger();
+  uint4 gains[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) {
+    const int v = threadIdx.x + i * NQ_THREADS;
+    gains[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (gamma != nullptr && v < d / NQ_VEC) gains[i] = reinterpret_cast<const uint4*>(gamma)[v];
+  }
+  int b = bits ? bits[row] : 16;
+  pdl_wait();
   if (zero_flags != nullptr)
     for (int i = blockIdx.x * NQ_THREADS + threadIdx.x; i < n_zero_flags; i += gridDim.x * NQ_THREADS) zero_flags[i] = 0;
   if (clear != nullptr)  // this token's scratch of the kernels that follow
@@ -78,10 +91,11 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
         x[i][4] = bf16_lo(w.z); x[i][5] = bf16_hi(w.z); x[i][6] = bf16_lo(w.w); x[i][7] = bf16_hi(w.w);
       }
       if (part != nullptr) {  // partial sums of the projection that produced this row, in slice order
-        for (int z0 = 0; z0 < ksplit; z0 += 4) {  // four slices' loads in flight, added in slice order
-          float4 a[4], b[4];
+#pragma unroll 1
+        for (int z0 = 0; z0 < ksplit; z0 += ZB) {  // ZB slices' loads in flight, added in slice order
+          float4 a[ZB], b[ZB];
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < ZB; ++q) {
             a[q] = b[q] = make_float4(0.f, 0.f, 0.f, 0.f);
             if (z0 + q < ksplit) {
               const float4* src =
@@ -91,7 +105,7 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
             }
           }
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
+          for (int q = 0; q < ZB; ++q) {
             x[i][0] += a[q].x; x[i][1] += a[q].y; x[i][2] += a[q].z; x[i][3] += a[q].w;
             x[i][4] += b[q].x; x[i][5] += b[q].y; x[i][6] += b[q].z; x[i][7] += b[q].w;
           }
@@ -114,7 +128,7 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
     for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
       const int v = threadIdx.x + i * NQ_THREADS;
       if (v < nvec) {
-        uint4 w = reinterpret_cast<const uint4*>(gamma)[v];
+        const uint4 w = gains[i];
         float gm[NQ_VEC] = {bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y),
                             bf16_lo(w.z), bf16_hi(w.z), bf16_lo(w.w), bf16_hi(w.w)};
 #pragma unroll
@@ -200,7 +214,6 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
     }
   }
 
-  int b = bits ? bits[row] : 16;
   // widths of 9..15 bits need int16 codes, and their codes are no exact bf16 numbers: they are served only where
   // no tensor-core operand is produced (the stand-alone wide quantizer call)
   const int b_max = (codes16 != nullptr && a_op == nullptr) ? 15 : 8;
@@ -273,18 +286,25 @@ void launch_norm_quant(const NormQuantArgs& a, cudaStream_t st) {
   GateArgs g;
   g.p_permille = a.gate_p_permille;
   g.xm = a.xm;
-#define SOL_NQ_LAUNCH(F32, GATE)                                                                                       \
-  SOL_LAUNCH("norm_quant", (norm_quant_kernel<F32, GATE>), dim3(a.B), dim3(NQ_THREADS), 0, st, a.in, a.part, a.ksplit,  \
-             stride, a.sum_out, static_cast<const uint16_t*>(a.gamma_bf16), a.eps, a.bits, a.d,                        \
+#define SOL_NQ_LAUNCH(F32, GATE, NV)                                                                                   \
+  SOL_LAUNCH("norm_quant", (norm_quant_kernel<F32, GATE, NV>), dim3(a.B), dim3(NQ_THREADS), 0, st, a.in, a.part,         \
+             a.ksplit, stride, a.sum_out, static_cast<const uint16_t*>(a.gamma_bf16), a.eps, a.bits, a.d,              \
              static_cast<uint16_t*>(a.a_op), a.a_op_rows, a.scale, a.xn, a.codes, a.codes16, a.status, a.clear,         \
              a.clear_words, a.zero_flags, a.n_zero_flags, g)
+#define SOL_NQ_BY_SIZE(F32, GATE)                          \
+  do {                                                     \
+    if (a.d <= 2048) SOL_NQ_LAUNCH(F32, GATE, 1);          \
+    else if (a.d <= 4096) SOL_NQ_LAUNCH(F32, GATE, 2);     \
+    else SOL_NQ_LAUNCH(F32, GATE, 4);                      \
+  } while (0)
   if (a.gate_p_permille != nullptr) {
-    if (a.in_f32) SOL_NQ_LAUNCH(true, true);
-    else SOL_NQ_LAUNCH(false, true);
+    if (a.in_f32) SOL_NQ_BY_SIZE(true, true);
+    else SOL_NQ_BY_SIZE(false, true);
   } else {
-    if (a.in_f32) SOL_NQ_LAUNCH(true, false);
-    else SOL_NQ_LAUNCH(false, false);
+    if (a.in_f32) SOL_NQ_BY_SIZE(true, false);
+    else SOL_NQ_BY_SIZE(false, false);
   }
+#undef SOL_NQ_BY_SIZE
 #undef SOL_NQ_LAUNCH
 }
 
