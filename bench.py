@@ -91,8 +91,10 @@ def kept_tokens(r_permille, T):
 def kernel_bytes(cfg, seq_lens, r, union_rows):
     """Bytes each streaming kernel must move per launch (one layer)."""
     d, hq, hkv, hd, ff = cfg["d_model"], cfg["n_q_heads"], cfg["n_kv_heads"], cfg["head_dim"], cfg["d_ff"]
-    k_bytes = sum(hkv * int(T) * hd * 2 for T in seq_lens)
-    v_bytes = sum(hkv * kept_tokens(ri, T) * hd * 2 for ri, T in zip(r, seq_lens))
+    rows = [(int(T), kept_tokens(ri, T)) for ri, T in zip(r, seq_lens)]
+    # pass 2 reads the keys of the rows that keep every token with their values; pass 1 reads the others' keys
+    k_bytes = sum(hkv * T * hd * 2 for T, k in rows if k < T)
+    v_bytes = sum(hkv * (k + (T if k >= T else 0)) * hd * 2 for T, k in rows)
     return {
         "attn_score": k_bytes,
         "attn_gather_v": v_bytes,

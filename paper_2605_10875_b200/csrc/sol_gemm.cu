@@ -460,7 +460,7 @@ struct DownRowsDev {
 // MB: tokens the registers are laid out for (>= M).  Few tokens leave room for 32 warps, more need 16.
 template <int MB>
 struct DownRowsCfg {
-  static constexpr int WARPS = MB <= 2 ? 32 : 16;
+  static constexpr int WARPS = MB <= 2 ? 32 : (MB <= 4 ? 24 : 16);
   static constexpr int TAB_WORDS = 32 * (1 + MB);  // per warp: kept channels of the group, their t of every token
   static constexpr int SMEM = WARPS * (TAB_WORDS + MB * 128) * 4;
 };
