@@ -92,26 +92,30 @@ __device__ __forceinline__ void plan_scan(int cnt, int* cum, int* wsum) {
 }
 
 // The pass-2 items of every sequence into cum; returns the kept tokens c of an item, a power of two from 64 to 1024: the
-// one with the least time by the rounds its items take on the resident warps, each round as long as an item and the
-// ITEM_FILL tokens that filling a warp's ring of row copies is worth.  (Long items alone left the chip half empty in a
-// second round: 134 MB of values of 32 sequences in 55 us.)
+// one with the least time by the rounds its items take on the resident warps, each round as long as the longest item and
+// the ITEM_FILL tokens that filling a warp's ring of row copies is worth, and the ITEM_MERGE tokens that merging the
+// partial results is worth where a row has several.  (Long items alone left the chip half empty in a second round: 134 MB
+// of values of 32 sequences in 55 us.)
 constexpr int ITEM_FILL = 256;  // measured: 64 to 192 cut long rows into too many items (290 -> 365 us where all of
                                 // 128 ragged sequences' tokens are kept), 512 gave up balance (32 equal sequences 98 -> 122)
+constexpr int ITEM_MERGE = 160;
 constexpr int ITEM_C0 = 64, ITEM_NC = 5;
 struct PlanSmem {
   int cum[PLAN_STRIDE];
-  int n_items[ITEM_NC];
+  int n_items[ITEM_NC], longest[ITEM_NC];  // per option: items of a kv-head, kept tokens of the longest
   int wsum[4];
 };
 __device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t& kv, const int32_t* r_permille, int B, int min_len,
                                           int target_items, PlanSmem& ps) {
   const int tid = threadIdx.x, lane = tid & 31;
-  if (tid < ITEM_NC) ps.n_items[tid] = 0;
+  if (tid < ITEM_NC) ps.n_items[tid] = ps.longest[tid] = 0;
   __syncthreads();
   int per_seq[ITEM_NC] = {0, 0, 0, 0, 0};
   if (tid < 128) {
+    int kept = 0;
     if (tid < B) {
       const RowPlan rp = row_plan(sh, kv, r_permille, tid);
+      kept = max(rp.k, 0);
 #pragma unroll
       for (int q = 0; q < ITEM_NC; ++q) {  // one item at least, so that the output is always written
         const int len = gather_item_tokens(rp, ITEM_C0 << q, min_len);
@@ -121,7 +125,11 @@ __device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t&
 #pragma unroll
     for (int q = 0; q < ITEM_NC; ++q) {
       const int n = __reduce_add_sync(0xffffffffu, per_seq[q]);
-      if (lane == 0 && n) atomicAdd(&ps.n_items[q], n);
+      const int most = __reduce_max_sync(0xffffffffu, per_seq[q] > 0 ? kept / per_seq[q] : 0);
+      if (lane == 0 && n) {
+        atomicAdd(&ps.n_items[q], n);
+        atomicMax(&ps.longest[q], most);
+      }
     }
   }
   __syncthreads();
@@ -130,7 +138,7 @@ __device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t&
 #pragma unroll
   for (int q = 0; q < ITEM_NC; ++q) {
     const int rounds = (ps.n_items[q] * sh.n_kv_heads + target_items - 1) / target_items;
-    const long long cost = (long long)rounds * ((ITEM_C0 << q) + ITEM_FILL);
+    const long long cost = (long long)rounds * (ps.longest[q] + ITEM_FILL) + (ps.n_items[q] > B ? ITEM_MERGE : 0);
     if (cost <= best) {
       best = cost;
       pick = q;
@@ -372,25 +380,40 @@ __device__ __forceinline__ void merge_partials(const AttnOut& o, const float* sr
     for (int q = lane; q < ns; q += 32) fac[q * G + h] *= inv;
   }
   __syncwarp();
-#pragma unroll 2
-  for (int e0 = lane * 2; e0 < G * HD; e0 += 64) {
-    const int h = e0 / HD, e = e0 % HD;
-    const float* src = src0 + (size_t)h * (HD + 2) + e;
-    float a0 = 0.f, a1 = 0.f;
+  // a lane's columns 2 lane, 2 lane + 1 of every 64: four such pairs of four partials in flight (one pair of eight partials:
+  // twice the round trips, 7.6 us for the 16 partials of a 4096-token row, its last warp's alone)
 #pragma unroll 1
-    for (int q = 0; q < ns; q += 8) {  // eight partials' loads in flight
-      float2 v[8];
+  for (int p0 = 0; p0 < G * HD / 64; p0 += 4) {
+    float2 a[4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u)
-        v[u] = q + u < ns ? __ldcg(reinterpret_cast<const float2*>(src + (q + u) * stride)) : make_float2(0.f, 0.f);
+    for (int x = 0; x < 4; ++x) a[x] = make_float2(0.f, 0.f);
+#pragma unroll 1
+    for (int q = 0; q < ns; q += 4) {
+      float2 v[4][4];
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const float f = q + u < ns ? fac[(q + u) * G + h] : 0.f;
-        a0 = fmaf(v[u].x, f, a0);
-        a1 = fmaf(v[u].y, f, a1);
+      for (int x = 0; x < 4; ++x) {
+        const int e0 = lane * 2 + 64 * (p0 + x), h = e0 / HD, e = e0 % HD;
+        const float* src = src0 + (size_t)q * stride + (size_t)h * (HD + 2) + e;
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          v[x][u] = p0 + x < G * HD / 64 && q + u < ns ? __ldcg(reinterpret_cast<const float2*>(src + u * stride)) : make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int h = min((lane * 2 + 64 * (p0 + x)) / HD, G - 1);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float f = q + u < ns ? fac[(q + u) * G + h] : 0.f;
+          a[x].x = fmaf(v[x][u].x, f, a[x].x);
+          a[x].y = fmaf(v[x][u].y, f, a[x].y);
+        }
       }
     }
-    attn_write<HD>(o, b, kvh * G + h, e, a0, a1);
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      const int e0 = lane * 2 + 64 * (p0 + x);
+      if (p0 + x < G * HD / 64) attn_write<HD>(o, b, kvh * G + e0 / HD, e0 % HD, a[x].x, a[x].y);
+    }
   }
 }
 
