@@ -182,8 +182,8 @@ struct PrepDev {
 
 constexpr int PREP_THREADS = 128;
 // words of AttnArgs::row_ctl, per (sequence, kv-head): segments whose scores are in the histogram, largest |score|,
-// keep edge (float bits)
-enum : int { RC_DONE = 0, RC_MAX, RC_EDGE, RC_WORDS = 8 };
+// keep edge (float bits), non-zero if a score is not a number
+enum : int { RC_DONE = 0, RC_MAX, RC_EDGE, RC_NAN, RC_WORDS = 8 };
 
 // One CTA per (kv-head, sequence): the G query heads of the group, the new k row and the new v row.
 __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p) {
@@ -361,23 +361,24 @@ __device__ __forceinline__ void merge_partials(const AttnOut& o, const float* sr
       const float l = warp_sum(ml[h].y * f);
       if (lane < ns) fac[lane * G + h] = l > 0.f ? f * (1.0f / l) : 0.f;
     }
-  } else
+  } else {
 #pragma unroll 1
-  for (int h = 0; h < G; ++h) {
-    const float* src = src0 + (size_t)h * (HD + 2) + HD;
-    float mm = -INFINITY;
-    for (int q = lane; q < ns; q += 32) mm = fmaxf(mm, __ldcg(src + q * stride));
-    mm = warp_max(mm);
-    float l = 0.f;
-    for (int q = lane; q < ns; q += 32) {
-      const float m2 = __ldcg(src + q * stride);
-      const float f = m2 == -INFINITY ? 0.f : exp2f(m2 - mm);
-      fac[q * G + h] = f;
-      l += __ldcg(src + q * stride + 1) * f;
+    for (int h = 0; h < G; ++h) {
+      const float* src = src0 + (size_t)h * (HD + 2) + HD;
+      float mm = -INFINITY;
+      for (int q = lane; q < ns; q += 32) mm = fmaxf(mm, __ldcg(src + q * stride));
+      mm = warp_max(mm);
+      float l = 0.f;
+      for (int q = lane; q < ns; q += 32) {
+        const float m2 = __ldcg(src + q * stride);
+        const float f = m2 == -INFINITY ? 0.f : exp2f(m2 - mm);
+        fac[q * G + h] = f;
+        l += __ldcg(src + q * stride + 1) * f;
+      }
+      l = warp_sum(l);
+      const float inv = l > 0.f ? 1.0f / l : 0.f;
+      for (int q = lane; q < ns; q += 32) fac[q * G + h] *= inv;
     }
-    l = warp_sum(l);
-    const float inv = l > 0.f ? 1.0f / l : 0.f;
-    for (int q = lane; q < ns; q += 32) fac[q * G + h] *= inv;
   }
   __syncwarp();
   // a lane's columns 2 lane, 2 lane + 1 of every 64: four such pairs of four partials in flight (one pair of eight partials:
@@ -849,6 +850,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   phase ^= 1;
 
   float mx = 0.f;
+  bool nan_here = false;
 #pragma unroll 1
   for (int i = tid * 4; i < n_here; i += TS_THREADS * 4) {
     const float4 v = *reinterpret_cast<const float4*>(hs.score + i);
@@ -859,19 +861,23 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
       if (j < T && !rp.forced(j)) {
         atomicAdd(&hist[key_value_bin(float_key(vv[e]))], 1u);
         mx = fmaxf(mx, fabsf(vv[e]));
+        nan_here = nan_here || vv[e] != vv[e];
       }
     }
   }
   mx = warp_max(mx);
   if (lane == 0) hs.fmax_w[warp] = mx;
-  __syncthreads();
+  int any_nan = __syncthreads_or(nan_here ? 1 : 0);
   mx = warp_max(lane < TS_THREADS / 32 ? hs.fmax_w[lane] : 0.f);
   if (nseg > 1) {  // only the CTA that arrives last goes on
     for (int i = tid; i < SEL_BINS; i += TS_THREADS) {
       const uint32_t c = hist[i];
       if (c) atomicAdd(gh + i, c);
     }
-    if (tid == 0) atomicMax(ctl + RC_MAX, __float_as_uint(mx));
+    if (tid == 0) {
+      atomicMax(ctl + RC_MAX, __float_as_uint(mx));
+      if (any_nan) atomicOr(ctl + RC_NAN, 1u);
+    }
     __threadfence();
     __syncthreads();
     if (tid == 0) hs.s_flag = atomicAdd(ctl + RC_DONE, 1u) == (uint32_t)(nseg - 1) ? 1 : 0;
@@ -881,6 +887,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
     for (int i = tid; i < SEL_BINS / 4; i += TS_THREADS)
       reinterpret_cast<uint4*>(hist)[i] = __ldcg(reinterpret_cast<const uint4*>(gh) + i);
     mx = __uint_as_float(__ldcg(ctl + RC_MAX));
+    any_nan = (int)__ldcg(ctl + RC_NAN);
     __syncthreads();
   }
 
@@ -987,7 +994,13 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
     }
   }
   in_window = block_count<TS_THREADS>(in_window, 0, sm);  // the barrier inside also publishes the candidates
-  settle_row(p, sm, hs.qsum, rp, b, kvh, above - in_window + rp.nf, edge, lo, delta, sm.counts[0]);
+  above -= in_window;
+  if (any_nan) {  // the histogram ranks what is not a number as a large score, but it is never kept: counted again
+    int n = 0;
+    for (int j = tid; j < T; j += TS_THREADS) n += !rp.forced(j) && sig[j] > edge ? 1 : 0;
+    above = block_count<TS_THREADS>(n, 1, sm);
+  }
+  settle_row(p, sm, hs.qsum, rp, b, kvh, above + rp.nf, edge, lo, delta, sm.counts[0]);
 }
 
 // Persistent CTAs over the flat list of (sequence, kv-head, segment) units of the rows that need a selection.

@@ -2,6 +2,8 @@
 import numpy as np
 import pytest
 
+from paper_2605_10875_b200 import synth
+from tests import harness as H
 from tests.test_gpu_parity import TINY, _attention_case, _mlp_case
 
 pytestmark = pytest.mark.gpu
@@ -47,3 +49,21 @@ def test_channel_selection_exact_rescoring(d, ff):
 
     _mlp_case(cfg, 3, [500, 250, 900], seed=d)
     _mlp_case(cfg, 2, [500, 730], seed=d + 1, mutate=groups)
+
+
+# Keys that are not numbers: never kept, and the count says what the list holds (rows of one selection segment and of two).
+@pytest.mark.parametrize("T", [700, 9000])
+def test_attention_selection_with_nan_keys(T):
+    cfg = dict(TINY, n_q_heads=4, n_kv_heads=1)
+    shape, _ = H.make_shapes(cfg, 0, 1)
+    lens = np.asarray([T], np.int32)
+    k_pool, v_pool, table = H.make_case_kv(cfg, lens, 5)
+    bad = [3, 64, 200, T - 50]
+    for j in bad:
+        k_pool[table[0, j // 64], :, j % 64, :] = 0x7FC0
+    kv = H.device_kv(k_pool, v_pool, table, lens)
+    _, kept, st = H.gpu_attention(shape, synth.make_queries(cfg, 5, 1), kv, [250])
+    k = -(-T // 4)
+    row = np.asarray(kept[0][0])
+    assert st[0] == 0 and np.all(np.diff(row) > 0) and row[0] >= 0 and row[-1] == T - 1
+    assert k - len(bad) <= len(row) <= k and not set(bad) & set(row.tolist())
