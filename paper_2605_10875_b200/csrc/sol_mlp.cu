@@ -268,12 +268,16 @@ struct ChanMultiSmem {
   double2 part[CM_EXACT][CM_THREADS / 32];  // the warps' sums of g and u
 };
 
-// The two bf16 numbers of a word as float64, by bits (a conversion instruction runs at a small fraction of this rate).  Zeros
-// and denormals come out as numbers of magnitude 2^-127 or less, which is nothing beside the sums' other terms.
+// The bf16 number in the high half of a word, times 2^-896, as float64: its bits in float64's place (a conversion
+// instruction runs at a small fraction of this rate).  Exact for every number: zeros stay zeros and denormals come out as
+// float64 denormals; infinities and NaNs stay what they are.
 __device__ __forceinline__ double bf16_bits_to_f64(uint32_t high_half) {
-  const uint32_t hi = ((high_half >> 3) & 0x0fffe000u) + 0x38000000u;
-  return __hiloint2double((int)(hi | (high_half & 0x80000000u)), 0);
+  uint32_t mag = (high_half >> 3) & 0x0fffe000u;
+  if (mag >= 0x0ff00000u) mag |= 0x7ff00000u;
+  return __hiloint2double((int)(mag | (high_half & 0x80000000u)), 0);
 }
+// 2^896, the factor that bf16_bits_to_f64 leaves out
+__device__ __forceinline__ double bf16_f64_scale() { return __hiloint2double((1023 + 896) << 20, 0); }
 
 // Exact |t| of up to CM_EXACT open candidates, by the whole CTA: g_j = scale * sum_e x_e w_je with x the quantizer codes (or
 // the bf16 row), in float64.  A thread owns elements 8 tid .. + 7 of every 2048; the rows are on their way to L2 before the
@@ -307,8 +311,9 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
       const uint32_t xa[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        x[2 * q] = in ? bf16_bits_to_f64(xa[q] << 16) : 0.0;
-        x[2 * q + 1] = in ? bf16_bits_to_f64(xa[q]) : 0.0;
+        // the factor of both operands of a product (the largest number times 2^896 is still finite)
+        x[2 * q] = in ? bf16_bits_to_f64(xa[q] << 16) * bf16_f64_scale() * bf16_f64_scale() : 0.0;
+        x[2 * q + 1] = in ? bf16_bits_to_f64(xa[q]) * bf16_f64_scale() * bf16_f64_scale() : 0.0;
       }
     }
     const unsigned char* chunk_src = p.w_gu + (size_t)(e0 >> 6) * chunk_bytes;

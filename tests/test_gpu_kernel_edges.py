@@ -67,3 +67,30 @@ def test_attention_selection_with_nan_keys(T):
     row = np.asarray(kept[0][0])
     assert st[0] == 0 and np.all(np.diff(row) > 0) and row[0] >= 0 and row[-1] == T - 1
     assert k - len(bad) <= len(row) <= k and not set(bad) & set(row.tolist())
+
+
+# Exactly equal scores: a row of zeros (a padding row) ranks every channel equal, and so do channels whose up rows are
+# zeros of either sign beside gate rows that are not; denormal weights are smaller than everything but those.  The exact
+# sums have to say so: ties go to the lower index.
+def test_channel_selection_of_scores_that_are_zero():
+    cfg = dict(TINY, d_ff=1024)
+    shape, _ = H.make_shapes(cfg)
+    ff, d = cfg["d_ff"], cfg["d_model"]
+    rng = np.random.default_rng(17)
+    w = synth.make_layer_weights(cfg, 17)
+    order = rng.permutation(ff)
+    normal, tiny, zero = np.sort(order[:300]), np.sort(order[300:400]), order[400:]
+    w.w_up[zero] = rng.choice(np.array([0x0000, 0x8000], np.uint16), (len(zero), d))
+    w.w_up[tiny] = rng.integers(1, 0x80, (len(tiny), d)).astype(np.uint16)  # positive bf16 denormals
+    x = synth.make_hidden(cfg, 17, 4)
+    x[0] = 0
+    x[1] &= 0x7FFF  # no negative inputs: the sums over the denormal rows do not cancel
+    x[2] = x[1]
+    x[3] = np.where(np.arange(d) % 2, 0x8000, 0).astype(np.uint16)  # zeros of either sign
+    m = [-(-ff * (1000 - p) // 1000) for p in (500, 500, 650, 250)]
+    _, kept, st = H.gpu_mlp(shape, x, H.device_weights(w, shape), [500, 500, 650, 250])
+    assert st[0] == 0
+    zero = np.sort(zero)
+    assert np.array_equal(kept[0], np.arange(m[0])) and np.array_equal(kept[3], np.arange(m[3]))
+    assert np.array_equal(kept[1], np.sort(np.concatenate([normal, tiny, zero[:m[1] - 400]])))
+    assert len(kept[2]) == m[2] and np.isin(normal, kept[2]).all() and np.isin(kept[2], np.concatenate([normal, tiny])).all()
