@@ -995,7 +995,10 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   }
   in_window = block_count<TS_THREADS>(in_window, 0, sm);  // the barrier inside also publishes the candidates
   above -= in_window;
-  if (any_nan) {  // the histogram ranks what is not a number as a large score, but it is never kept: counted again
+  // Counted again where the histogram's ranks say something else than "above the edge": it ranks what is not a number as
+  // a large score, but that is never kept; and where the k-th score lies in the top bin, whose end is +inf, scores of
+  // +inf are no higher than the bin but above the edge, and all of them are kept.
+  if (any_nan || mx == INFINITY) {
     int n = 0;
     for (int j = tid; j < T; j += TS_THREADS) n += !rp.forced(j) && sig[j] > edge ? 1 : 0;
     above = block_count<TS_THREADS>(n, 1, sm);

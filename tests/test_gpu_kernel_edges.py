@@ -94,3 +94,25 @@ def test_channel_selection_of_scores_that_are_zero():
     assert np.array_equal(kept[0], np.arange(m[0])) and np.array_equal(kept[3], np.arange(m[3]))
     assert np.array_equal(kept[1], np.sort(np.concatenate([normal, tiny, zero[:m[1] - 400]])))
     assert len(kept[2]) == m[2] and np.isin(normal, kept[2]).all() and np.isin(kept[2], np.concatenate([normal, tiny])).all()
+
+
+# Scores of +inf are all kept, more of them than the budget included; the count says what the list holds (rows of one
+# selection segment and of two).
+@pytest.mark.parametrize("T,r,n_inf", [(60, 50, 5), (700, 4, 9), (9000, 1, 20), (700, 10, 4), (700, 1000, 4)])
+def test_attention_selection_with_infinite_scores(T, r, n_inf):
+    cfg = dict(TINY, n_q_heads=4, n_kv_heads=4)
+    shape, _ = H.make_shapes(cfg, 0, 1)
+    lens = np.asarray([T], np.int32)
+    k_pool, v_pool, table = H.make_case_kv(cfg, lens, 5)
+    q = synth.make_queries(cfg, 5, 1)
+    huge = np.where(q[0] & 0x8000, 0xFF61, 0x7F61).astype(np.uint16)  # +-2.99e38 with the query's signs
+    inf = np.sort(np.random.default_rng(T).permutation(T - 1)[:n_inf])
+    for j in inf:
+        k_pool[table[0, j // 64], :, j % 64, :] = huge
+    kv = H.device_kv(k_pool, v_pool, table, lens)
+    _, kept, st = H.gpu_attention(shape, q, kv, [r])
+    k = max(1, -(-T * r // 1000))
+    assert st[0] == 0
+    for h in range(4):
+        row = np.asarray(kept[0][h])
+        assert len(row) == max(k, n_inf + 1) and np.all(np.diff(row) > 0) and row[-1] == T - 1 and np.isin(inf, row).all()
