@@ -529,6 +529,7 @@ __global__ void __launch_bounds__(DownRowsCfg<MB>::WARPS * 32, 1) down_rows_kern
 #pragma unroll
       for (int m = 0; m < MB; ++m) tab_t[at * MB + m] = tl[m];
     }
+    if ((n & 1) && lane < MB) tab_t[n * MB + lane] = 0.f;  // an odd count: the absent second channel of the last pair
     __syncwarp();
 #pragma unroll 1
     for (int u0 = 0; u0 < n; u0 += 16) {  // warp-uniform
@@ -545,7 +546,7 @@ __global__ void __launch_bounds__(DownRowsCfg<MB>::WARPS * 32, 1) down_rows_kern
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         if (u0 + 2 * u >= n) break;  // warp-uniform
-        const int at = min(u0 + 2 * u + sub, n - 1);  // an absent second channel has zero weights
+        const int at = u0 + 2 * u + sub;  // an absent second channel has zero weights and a zero t
         const uint64_t w[4] = {f32x2(bf16_lo(wv[u].x), bf16_hi(wv[u].x)), f32x2(bf16_lo(wv[u].y), bf16_hi(wv[u].y)),
                                f32x2(bf16_lo(wv[u].z), bf16_hi(wv[u].z)), f32x2(bf16_lo(wv[u].w), bf16_hi(wv[u].w))};
 #pragma unroll

@@ -116,3 +116,20 @@ def test_attention_selection_with_infinite_scores(T, r, n_inf):
     for h in range(4):
         row = np.asarray(kept[0][h])
         assert len(row) == max(k, n_inf + 1) and np.all(np.diff(row) > 0) and row[-1] == T - 1 and np.isin(inf, row).all()
+
+
+# One kept channel with an infinite activation: its product with the weights is infinite, and nothing is multiplied by a
+# zero weight in its place (every register layout of the row-by-row down projection).
+@pytest.mark.parametrize("B", [1, 2, 3, 4, 8])
+def test_down_rows_with_an_infinite_activation(B):
+    cfg = dict(TINY, d_ff=96)
+    shape, _ = H.make_shapes(cfg)
+    w = synth.make_layer_weights(cfg, 3)
+    x = synth.make_hidden(cfg, 3, B)
+    x[:] = np.where(np.arange(cfg["d_model"]) == 0, 0x3F80, 0)  # 1, 0, 0, ...
+    w.w_gate[40], w.w_up[40] = 0x7149, 0x7149                   # about 1e30 each
+    w.w_down_t[40] = np.where(w.w_down_t[40] & 0x7FFF, w.w_down_t[40], 0x3C00)  # no zeros
+    out, kept, st = H.gpu_mlp(shape, x, H.device_weights(w, shape), [999] * B)
+    assert st[0] == 0 and all(np.array_equal(k, [40]) for k in kept)
+    want = np.where(synth.bf16_to_f32(w.w_down_t[40]) > 0, np.inf, -np.inf)
+    assert np.array_equal(out, np.broadcast_to(want, out.shape))
