@@ -268,16 +268,19 @@ struct ChanMultiSmem {
   double2 part[CM_EXACT][CM_THREADS / 32];  // the warps' sums of g and u
 };
 
-// The bf16 number in the high half of a word, times 2^-896, as float64: its bits in float64's place (a conversion
-// instruction runs at a small fraction of this rate).  Exact for every number: zeros stay zeros and denormals come out as
-// float64 denormals; infinities and NaNs stay what they are.
-__device__ __forceinline__ double bf16_bits_to_f64(uint32_t high_half) {
-  uint32_t mag = (high_half >> 3) & 0x0fffe000u;
-  if (mag >= 0x0ff00000u) mag |= 0x7ff00000u;
-  return __hiloint2double((int)(mag | (high_half & 0x80000000u)), 0);
+// bf16 numbers as float64 by their bits (a conversion instruction runs at a small fraction of this rate).
+// Operand elements, the number in the high half of a word: exact, whatever the number.
+__device__ __forceinline__ double operand_to_f64(uint32_t high_half) {
+  const uint32_t mag = (high_half >> 3) & 0x0fffe000u, sign = high_half & 0x80000000u;
+  if (mag - 1u < 0x000fffffu || mag >= 0x0ff00000u) return (double)__uint_as_float(high_half & 0xffff0000u);  // denormal, infinite, NaN
+  return __hiloint2double((int)((mag ? mag + 0x38000000u : 0u) | sign), 0);
 }
-// 2^896, the factor that bf16_bits_to_f64 leaves out
-__device__ __forceinline__ double bf16_f64_scale() { return __hiloint2double((1023 + 896) << 20, 0); }
+// Weights: times 2^-896, so that no bias is added and zeros and denormals need no case of their own (they come out as
+// zeros and float64 denormals; a product is good to 2^-178 at least).  A channel with an infinite or NaN weight has an
+// infinite or NaN |t| and is never a candidate.
+__device__ __forceinline__ double weight_to_f64(uint32_t high_half) {
+  return __hiloint2double((int)(((high_half >> 3) & 0x0fffe000u) | (high_half & 0x80000000u)), 0);
+}
 
 // Exact |t| of up to CM_EXACT open candidates, by the whole CTA: g_j = scale * sum_e x_e w_je with x the quantizer codes (or
 // the bf16 row), in float64.  A thread owns elements 8 tid .. + 7 of every 2048; the rows are on their way to L2 before the
@@ -311,9 +314,8 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
       const uint32_t xa[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        // the factor of both operands of a product (the largest number times 2^896 is still finite)
-        x[2 * q] = in ? bf16_bits_to_f64(xa[q] << 16) * bf16_f64_scale() * bf16_f64_scale() : 0.0;
-        x[2 * q + 1] = in ? bf16_bits_to_f64(xa[q]) * bf16_f64_scale() * bf16_f64_scale() : 0.0;
+        x[2 * q] = operand_to_f64(xa[q] << 16);
+        x[2 * q + 1] = operand_to_f64(xa[q]);
       }
     }
     const unsigned char* chunk_src = p.w_gu + (size_t)(e0 >> 6) * chunk_bytes;
@@ -333,10 +335,10 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
       double g = 0.0, u = 0.0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        g = fma(x[2 * q], bf16_bits_to_f64(ga[q] << 16), g);
-        u = fma(x[2 * q], bf16_bits_to_f64(ua[q] << 16), u);
-        g = fma(x[2 * q + 1], bf16_bits_to_f64(ga[q]), g);
-        u = fma(x[2 * q + 1], bf16_bits_to_f64(ua[q]), u);
+        g = fma(x[2 * q], weight_to_f64(ga[q] << 16), g);
+        u = fma(x[2 * q], weight_to_f64(ua[q] << 16), u);
+        g = fma(x[2 * q + 1], weight_to_f64(ga[q]), g);
+        u = fma(x[2 * q + 1], weight_to_f64(ua[q]), u);
       }
       g = warp_sum_d(g);
       u = warp_sum_d(u);
@@ -354,7 +356,8 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
       g += sm.part[tid][w].x;
       u += sm.part[tid][w].y;
     }
-    const double sc = (double)p.scale[b], ag = g * sc, au = u * sc;
+    const double unit = __hiloint2double((1023 + 896) << 20, 0);  // 2^896, see weight_to_f64
+    const double sc = (double)p.scale[b], ag = g * unit * sc, au = u * unit * sc;
     sm.val[sm.open[i0 + tid]] = fabs(ag / (1.0 + exp(-ag)) * au);
   }
   __syncthreads();
