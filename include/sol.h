@@ -17,7 +17,11 @@
  *     has finished; the library allocates no device memory on these calls
  *     (scratch comes from the caller's workspace `ws`);
  *   - work is enqueued on `stream` (a cudaStream_t); the call does not wait
- *     for it;
+ *     for it; whatever the stream held before the call has completed before
+ *     any input is read, also where the last of it is a kernel that lets its
+ *     dependents start early (programmatic dependent launch) and writes the
+ *     actions or lengths only then (the packed weights alone must not be
+ *     written by such a kernel: their first tiles are fetched ahead);
  *   - bf16 tensors are raw 16-bit patterns; matrices are row-major;
  *   - argument errors are detected on the host before anything is launched.
  */

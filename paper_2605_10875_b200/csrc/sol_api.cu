@@ -244,7 +244,7 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
                     const int32_t* p_permille, const void* resid, int resid_f32, void* out_bf16,
                     float* out_f32, float* out_f32_b, float* t_trace, int32_t* kept_ch, int32_t* kept_ch_cnt,
                     cudaStream_t st, const int32_t* out_bits = nullptr, const sol_layer_trace_t* tr = nullptr,
-                    LayerCarry* carry_out = nullptr) {
+                    LayerCarry* carry_out = nullptr, bool hold = false) {
   int* status = at<int>(ws, L.status);
   GemmNK gu;
   memset(&gu, 0, sizeof(gu));
@@ -260,6 +260,7 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
   gu.out2 = t_trace ? t_trace : at<float>(ws, L.t);
   gu.sel = at<uint32_t>(ws, L.ch_sel);
   gu.sel_p_permille = p_permille;
+  gu.hold = hold;
   gu.status = status;
   launch_gemm_nk(gu, EPI_SWIGLU, st);
 
@@ -327,8 +328,8 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
 static void run_layer(const sol_shape_t& s, const Layout& L, void* ws, const sol_layer_weights_t& w,
                       const sol_kv_t& kv, int B, const void* h_in, bool in_f32, void* h_out_bf16, float* h_out_f32,
                       const int32_t* r, const int32_t* p, const int32_t* bits, const sol_layer_trace_t* tr,
-                      cudaStream_t st, const LayerCarry* carry_in = nullptr, LayerCarry* carry_out = nullptr,
-                      int span_tokens = 0) {
+                      cudaStream_t st, bool first, const LayerCarry* carry_in = nullptr,
+                      LayerCarry* carry_out = nullptr, int span_tokens = 0) {
   int* status = at<int>(ws, L.status);
   const int d = s.d_model, Hq = s.n_q_heads, Hkv = s.n_kv_heads, hd = s.head_dim;
   const int Nqkv = (Hq + 2 * Hkv) * hd;
@@ -351,6 +352,7 @@ static void run_layer(const sol_shape_t& s, const Layout& L, void* ws, const sol
   n1.a_op = at<void>(ws, L.a_op); n1.a_op_rows = L.Mpad; n1.scale = scale; n1.xn = tr ? tr->xn1 : nullptr;
   n1.codes = tr ? tr->codes1 : nullptr;
   n1.status = status;
+  n1.first = first;
   launch_norm_quant(n1, st);
   if (tr && tr->scales1) cudaMemcpyAsync(tr->scales1, scale, sizeof(float) * B, cudaMemcpyDeviceToDevice, st);
 
@@ -365,6 +367,7 @@ static void run_layer(const sol_shape_t& s, const Layout& L, void* ws, const sol
   q.K = d;
   q.N = Nqkv;
   q.out0 = at<float>(ws, L.qkv);
+  q.hold = first;
   q.status = status;
   launch_gemm_nk(q, EPI_PARTIAL, st);
 
@@ -463,6 +466,7 @@ sol_status_t sol_quant_act(const void* x_bf16, int32_t B, int32_t d, const int32
   NormQuantArgs n;
   memset(&n, 0, sizeof(n));
   n.in = x_bf16; n.bits = bits; n.B = B; n.d = d; n.a_op = xhat_bf16; n.scale = scales; n.codes = codes;
+  n.first = true;
   launch_norm_quant(n, (cudaStream_t)stream);
   return finish();
 }
@@ -475,6 +479,7 @@ sol_status_t sol_quant_act_wide(const void* x_bf16, int32_t B, int32_t d, const 
   NormQuantArgs n;
   memset(&n, 0, sizeof(n));
   n.in = x_bf16; n.bits = bits; n.B = B; n.d = d; n.scale = scales; n.codes16 = codes;
+  n.first = true;
   launch_norm_quant(n, (cudaStream_t)stream);
   return finish();
 }
@@ -530,9 +535,10 @@ sol_status_t sol_pruned_swiglu_mlp(const sol_shape_t* shape, const void* x_bf16,
   n.scale = at<float>(ws, L.scale);
   n.clear = at<uint32_t>(ws, L.ch_sel);
   n.clear_words = CH_SEL_WORDS;
+  n.first = true;
   launch_norm_quant(n, st);
   run_mlp(*shape, L, ws, B, w_gate_up, w_down, p_permille, nullptr, 0, out_bf16, nullptr, nullptr, nullptr,
-          kept_ch, kept_ch_cnt, st);
+          kept_ch, kept_ch_cnt, st, nullptr, nullptr, nullptr, true);
   return finish();
 }
 
@@ -580,7 +586,7 @@ sol_status_t sol_decode_layer(const sol_shape_t* shape, const sol_layer_weights_
   const Layout L = make_layout(*shape, B, kv->max_pages_per_seq);
   if (ws_bytes < L.total) return SOL_ERR_WORKSPACE_TOO_SMALL;
   run_layer(*shape, L, ws, *w, *kv, B, h_in_bf16, false, h_out_bf16, nullptr, r_permille, p_permille, bits, trace,
-            (cudaStream_t)stream);
+            (cudaStream_t)stream, true);
   return finish();
 }
 
@@ -604,7 +610,8 @@ static sol_status_t decode_step_impl(const sol_shape_t* shape, int32_t n_layers,
     const bool defer = may_defer && !last;
     float* out32 = last ? h_out_f32 : at<float>(ws, (l & 1) ? L.h_b : L.h_a);
     run_layer(*shape, L, ws, layers[l], kv, B, h, in_f32, last ? h_out_bf16 : nullptr, out32, r, p, bits,
-              traces ? &traces[l] : nullptr, st, have ? &carry[(l + 1) & 1] : nullptr, defer ? &carry[l & 1] : nullptr);
+              traces ? &traces[l] : nullptr, st, l == 0, have ? &carry[(l + 1) & 1] : nullptr,
+              defer ? &carry[l & 1] : nullptr);
     have = defer;
     h = out32;
     in_f32 = true;
@@ -713,9 +720,10 @@ sol_status_t sol_kv_refresh(const sol_shape_t* shape, int32_t n_layers, const so
     int prev_mp = 0;
     for (int l = 0; l < n_layers; ++l) {
       sol_kv_t kv = kvs[l];
-      if (kv.page_table != prev_table || kv.seq_lens != prev_lens || kv.max_pages_per_seq != prev_mp) {
-        // a plain launch: it starts after everything before it on the stream has ended, and the layer's first
-        // kernel after it
+      const bool expand = kv.page_table != prev_table || kv.seq_lens != prev_lens || kv.max_pages_per_seq != prev_mp;
+      if (expand) {
+        // a plain launch: it starts after everything before it on the stream has ended; the layer's first kernel
+        // waits for it before it lets the others start
         refresh_expand_kernel<<<rows, 128, 0, st>>>(kv.page_table + (size_t)s0 * kv.max_pages_per_seq, kv.seq_lens + s0,
                                                     kv.max_pages_per_seq, n_tokens, rows, tab, act, at<int>(ws, L.status));
         if (record_cuda_error(cudaGetLastError(), "refresh: page-table rows")) return finish();
@@ -728,7 +736,7 @@ sol_status_t sol_kv_refresh(const sol_shape_t* shape, int32_t n_layers, const so
       // up to 16 tokens per sequence are the rows of one tensor-core tile of the span attention, which reads a
       // sequence's cache once for all of them; longer spans go through the decode step's attention row by row
       run_layer(dense, L, ws, layers[l], kv, rows, h, in_f32, last ? out : nullptr, last && out ? nullptr : out32, act,
-                act + rows, act + 2 * rows, nullptr, st, nullptr, nullptr, n_tokens <= 16 ? n_tokens : 0);
+                act + rows, act + 2 * rows, nullptr, st, expand, nullptr, nullptr, n_tokens <= 16 ? n_tokens : 0);
       h = out32;
       in_f32 = true;
     }

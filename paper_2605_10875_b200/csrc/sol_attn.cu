@@ -192,11 +192,12 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
   const int Hq = p.sh.n_q_heads, Hkv = p.sh.n_kv_heads, hd = p.sh.head_dim, half = hd / 2;
   const int G = Hq / Hkv, HG = (G + 3) / 4;
   const int tid = threadIdx.x;
-  const int T = min(p.kv.seq_lens[b], p.kv.max_pages_per_seq * PAGE);  // never index past the page table
-  const int pos = T - 1;
   const bool layer = p.qkv != nullptr;
   const bool rope = layer && p.sh.rope_theta > 0.f;
+  if (!layer) pdl_wait();  // the stand-alone attention begins with this kernel
   pdl_trigger();
+  const int T = min(p.kv.seq_lens[b], p.kv.max_pages_per_seq * PAGE);  // never index past the page table
+  const int pos = T - 1;
   // the angles need only the lengths (an input of the step): float64 functions are slow here, and the projection is
   // still running
   if (tid < half) {

@@ -132,9 +132,21 @@ constexpr int CH_CAND_CAP = 1024;  // exactly re-scored candidates per token bef
 // ---- programmatic dependent launch ---------------------------------------------
 // pdl_trigger: the next kernel in the stream may be scheduled from now on (it still waits in
 // pdl_wait for this grid to finish).  pdl_wait: returns once every earlier kernel has completed and
-// its writes are visible; until then only constants (weights, shapes) may be read.
+// its writes are visible.
+// Kernels trigger at their start, so a whole chain of them can be resident while the first one still
+// waits, and what the caller has put on the stream (a kernel of its own that triggers before it writes
+// the actions, say) need not be complete when they start.  So the chain of an entry point begins like this:
+//   - its first kernel reads nothing ahead of its wait;
+//   - if its second kernel is a projection, that one reads weights only ahead of its wait, and triggers
+//     after it (pdl_wait_hold); otherwise the first kernel triggers after its own wait.
+// Every later kernel starts when the inputs of the call are complete and may read them ahead of its own
+// wait: weights, gains, lengths, rates and widths, but never what a kernel of the chain writes.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait_hold(bool hold) {
+  pdl_wait();
+  if (hold) pdl_trigger();
+}
 
 // ---- small reductions ---------------------------------------------------------
 __device__ __forceinline__ float warp_sum(float v) {

@@ -78,6 +78,7 @@ struct NKDev {
   float* out2;
   uint32_t* sel;
   const int32_t* sel_p;  // [M] prune rates or nullptr
+  int hold;              // the next kernel starts after this one's wait (pdl_wait_hold)
   int* status;
 };
 
@@ -91,7 +92,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
   UmBarriers* bars = reinterpret_cast<UmBarriers*>(stages + (size_t)p.stages * stage_bytes + UM_TILE_SPAN);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_trigger();
+  if (!p.hold) pdl_trigger();
   if (threadIdx.x == 0) {
     for (int s = 0; s < p.stages; ++s) {
       mbar_init(&bars->full[s], 1);
@@ -120,14 +121,17 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
     // -------------------------------- producer -------------------------------
     // Weights do not depend on earlier kernels: the first ring of weight tiles is requested before
     // pdl_wait(), the activation tiles of those stages after it.
+    const int pre = min(n_iter, p.stages);
     if (lane == 0) {
-      const int pre = min(n_iter, p.stages);
       for (int it = 0; it < pre; ++it) {
         unsigned char* st = stages + (size_t)it * stage_bytes;
         mbar_expect_tx(&bars->full[it], stage_bytes);
         bulk_g2s(st, w_src + (size_t)it * p.cps * w_tile, p.cps * w_tile, &bars->full[it]);
       }
-      pdl_wait();
+    }
+    __syncwarp();
+    pdl_wait_hold(p.hold);
+    if (lane == 0) {
       for (int it = 0; it < pre; ++it) {
         unsigned char* xs = stages + (size_t)it * stage_bytes + p.cps * w_tile;
         bulk_g2s(xs, x_src + (size_t)it * p.cps * x_tile, p.cps * x_tile, &bars->full[it]);
@@ -154,7 +158,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
     bool acc = false, ok = true;
     // the first stage fills only after the producer's own pdl_wait(): without this wait the bounded poll
     // below would start counting while earlier kernels of the stream are still running
-    pdl_wait();
+    pdl_wait_hold(p.hold);
     int s = 0;
     uint32_t ph = 0;
     for (int it = 0; it < n_iter; ++it) {
@@ -183,7 +187,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
     if (ok && elect_one()) umma_commit(&bars->accum);
   } else {
     // -------------------------------- epilogue -------------------------------
-    pdl_wait();  // the epilogue reads scales and overwrites buffers earlier kernels used
+    pdl_wait_hold(p.hold);  // the epilogue reads scales and overwrites buffers earlier kernels used
     if (EPI == EPI_SWIGLU) {
       // the scales come to shared memory while the weights stream: a global load per token inside the loop
       // below would put its latency between every two tokens
@@ -706,6 +710,7 @@ void launch_gemm_nk(const GemmNK& g, GemmEpilogue epi, cudaStream_t st) {
   d.x = static_cast<const unsigned char*>(g.a);
   d.row_scale = g.row_scale;
   d.out0 = g.out0; d.out1 = g.out1; d.out2 = g.out2; d.sel = g.sel; d.sel_p = g.sel_p_permille; d.status = g.status;
+  d.hold = g.hold;
   const int smem = 1024 + stages * stage_bytes + UM_TILE_SPAN + (int)sizeof(UmBarriers);
   const dim3 grid(geo.tiles, d.ksplit);
   if (epi == EPI_SWIGLU) {

@@ -19,7 +19,9 @@ bool take_cuda_failure();  // true if a CUDA call of this thread failed since th
 
 // Every kernel is launched with programmatic stream serialization: it may start while the kernel
 // before it in the stream is still running, does its set-up (and, for the GEMMs, starts streaming
-// weights), and calls pdl_wait() before it touches anything an earlier kernel produced.
+// weights; the attention kernels make their work lists from the step's lengths and rates), and calls
+// pdl_wait() before it touches anything an earlier kernel of the chain produced.  What may be read ahead of
+// that wait, and what the first kernels of an entry point do so that it may: see pdl_wait in sol_common.cuh.
 #define SOL_LAUNCH(name, kernel, grid, block, smem, st, ...)                                   \
   do {                                                                                         \
     ::sol::note_launch_begin(name, st);                                                        \
@@ -74,6 +76,7 @@ struct NormQuantArgs {
   int clear_words;
   int32_t* zero_flags;  // optional: n_zero_flags words zeroed by the grid as a whole (the down projection's live flags,
   int n_zero_flags;     // when this kernel also stands in for the reduction of the previous layer's down projection)
+  bool first;           // the first kernel of an entry point: reads nothing ahead of its wait
 };
 void launch_norm_quant(const NormQuantArgs& a, cudaStream_t st);
 
@@ -169,6 +172,7 @@ struct GemmNK {
   float* out2;            // EPI_SWIGLU: t = silu(g) * u
   uint32_t* sel;          // EPI_SWIGLU: [M][CH_SEL_WORDS] histogram of |t| and max |g|, |u| per token (pre-cleared)
   const int32_t* sel_p_permille;  // EPI_SWIGLU, optional: [M] prune rates; tokens that keep all or no channels need no histogram
+  bool hold;              // the second kernel of an entry point (see pdl_wait in sol_common.cuh)
   int* status;
 };
 void launch_gemm_nk(const GemmNK& p, GemmEpilogue epi, cudaStream_t st);

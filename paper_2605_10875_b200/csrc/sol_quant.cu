@@ -38,8 +38,9 @@ struct NoSmem {
 };
 
 // NV: vectors of eight elements per thread (d <= NV * 2048).  Latency-bound: what needs nothing of the kernels before (the
-// gains, the width) is read while they run, and the code is compiled for the row's length (one code for all lengths: 5.96 us
-// in the chain of a single-sequence step, this 5.74; all nine slices of the partial sums in flight at once: the same).
+// gains, the width) is read while they run, unless it is the first kernel of a call, and the code is compiled for the row's
+// length (one code for all lengths: 5.96 us in the chain of a single-sequence step, this 5.74; all nine slices of the
+// partial sums in flight at once: the same).
 template <bool IN_F32, bool GATE, int NV>
 __global__ void __launch_bounds__(NQ_THREADS)
 norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, int ksplit, size_t part_stride,
@@ -48,13 +49,14 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
                   float* __restrict__ scale,
                   float* __restrict__ xn, int8_t* __restrict__ codes, int16_t* __restrict__ codes16, int* __restrict__ status,
                   uint32_t* __restrict__ clear, int clear_words, int32_t* __restrict__ zero_flags, int n_zero_flags,
-                  const GateArgs gate) {
+                  bool first, const GateArgs gate) {
   __shared__ float sh[NQ_THREADS / 32];
   __shared__ typename std::conditional<GATE, SelectSmem, NoSmem>::type gsm;
   constexpr int NQ_MAX_PER_THREAD = NV;
   constexpr int ZB = NV == 1 ? 12 : 4;  // slices of the partial sums in flight
   const int row = blockIdx.x;
   pdl_trigger();
+  if (first) pdl_wait();
   uint4 gains[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) {
@@ -62,7 +64,7 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
     gains[i] = make_uint4(0u, 0u, 0u, 0u);
     if (gamma != nullptr && v < d / NQ_VEC) gains[i] = reinterpret_cast<const uint4*>(gamma)[v];
   }
-  int b = bits ? bits[row] : 16;
+  int b = bits ? __ldcg(bits + row) : 16;
   pdl_wait();
   if (zero_flags != nullptr)
     for (int i = blockIdx.x * NQ_THREADS + threadIdx.x; i < n_zero_flags; i += gridDim.x * NQ_THREADS) zero_flags[i] = 0;
@@ -289,7 +291,7 @@ void launch_norm_quant(const NormQuantArgs& a, cudaStream_t st) {
   SOL_LAUNCH("norm_quant", (norm_quant_kernel<F32, GATE, NV>), dim3(a.B), dim3(NQ_THREADS), 0, st, a.in, a.part,         \
              a.ksplit, stride, a.sum_out, static_cast<const uint16_t*>(a.gamma_bf16), a.eps, a.bits, a.d,              \
              static_cast<uint16_t*>(a.a_op), a.a_op_rows, a.scale, a.xn, a.codes, a.codes16, a.status, a.clear,         \
-             a.clear_words, a.zero_flags, a.n_zero_flags, g)
+             a.clear_words, a.zero_flags, a.n_zero_flags, a.first, g)
 #define SOL_NQ_BY_SIZE(F32, GATE)                          \
   do {                                                     \
     if (a.d <= 2048) SOL_NQ_LAUNCH(F32, GATE, 1);          \

@@ -1,7 +1,9 @@
 """Kernels at the sizes where their tiling can go wrong: remainders, single tiles, the smallest and largest of a range."""
 import numpy as np
 import pytest
+import torch
 
+from paper_2605_10875_b200 import binding as sol
 from paper_2605_10875_b200 import synth
 from tests import harness as H
 from tests.test_gpu_parity import TINY, _attention_case, _mlp_case
@@ -133,3 +135,62 @@ def test_down_rows_with_an_infinite_activation(B):
     assert st[0] == 0 and all(np.array_equal(k, [40]) for k in kept)
     want = np.where(synth.bf16_to_f32(w.w_down_t[40]) > 0, np.inf, -np.inf)
     assert np.array_equal(out, np.broadcast_to(want, out.shape))
+
+
+# A program's own kernel may let its dependents start (programmatic dependent launch) before it has written the step's
+# actions and lengths: the calls must not read them earlier than that kernel's end.  What the arrays hold before is valid
+# as well, and other.
+_EARLY = """extern "C" __global__ void late_writer(int* dst, const int* src, int n) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  for (int i = 0; i < 300; ++i) __nanosleep(1000);
+  if (threadIdx.x < n) dst[threadIdx.x] = src[threadIdx.x];
+}"""
+
+
+@pytest.mark.parametrize("call", ["layer", "step", "attention", "mlp", "quantizer", "refresh"])
+def test_inputs_written_by_a_kernel_that_triggers_early(call):
+    writer = torch.cuda._compile_kernel(_EARLY, "late_writer")
+    cfg = dict(TINY, d_model=512, n_q_heads=8, n_kv_heads=2, d_ff=2080)
+    B, d, n_layers = 6, 512, 2
+    shape, _ = H.make_shapes(cfg)
+    lens = np.asarray([700, 64, 1500, 129, 300, 2049], np.int32)
+    pools = [H.make_case_kv(cfg, lens, 3, layer) for layer in range(n_layers)]
+    dws = [H.device_weights(synth.make_layer_weights(cfg, 3, layer), shape) for layer in range(n_layers)]
+    new, old = np.zeros((4, 8), np.int32), np.zeros((4, 8), np.int32)
+    new[:, :B] = [125, 1000, 500, 250, 999, 40], [0, 500, 250, 750, 999, 125], [4, 8, 16, 2, 3, 16], lens
+    old[:, :B] = [1000, 125, 1000, 1000, 125, 1000], [500, 0, 0, 0, 500, 500], [16, 4, 4, 8, 8, 2], [300, 33, 40, 100, 17, 500]
+    h = H.dev_bf16(synth.make_hidden(cfg, 3, B * 16)).view(B, 16, d)
+    q = H.dev_bf16(synth.make_queries(cfg, 3, B))
+
+    def run(act, before):
+        kvs = [H.device_kv(k, v, table, lens) for k, v, table in pools]
+        for kv in kvs:
+            kv.seq_lens = act[3]
+        structs, weights = [kv.struct() for kv in kvs], [w.struct() for w in dws]
+        r, p, b = act[0], act[1], act[2]
+        ws = H.Workspace(shape, B * 16, kvs[0].max_pages)
+        out = torch.zeros((B, 16, d), dtype=torch.bfloat16, device=H.DEV)
+        codes, scales = torch.zeros((B, d), dtype=torch.int8, device=H.DEV), torch.zeros(B, device=H.DEV)
+        torch.cuda.synchronize()
+        before()
+        if call == "layer":
+            sol.decode_layer(shape, weights[0], structs[0], B, h, out, r, p, b, None, ws.buf, ws.bytes)
+        elif call == "step":
+            sol.decode_step(shape, weights, structs, B, h, out, None, r, p, b, ws.buf, ws.bytes)
+        elif call == "attention":
+            sol.sparse_decode_attn(shape, q, structs[0], B, r, out, None, None, ws.buf, ws.bytes)
+        elif call == "mlp":
+            t = dws[0].tensors
+            sol.pruned_swiglu_mlp(shape, h, t["w_gate_up"], t["w_down"], B, p, out, None, None, ws.buf, ws.bytes)
+        elif call == "quantizer":
+            sol.quant_act(h, B, d, b, codes, scales, out)
+        else:
+            sol.kv_refresh(shape, weights, structs, B, 16, h, out, ws.buf, ws.bytes)
+        torch.cuda.synchronize()
+        assert call == "quantizer" or ws.status()[0] == 0
+        return [out, codes, scales] + [x for kv in kvs for x in (kv.k_pool, kv.v_pool)]
+
+    want = run(H.dev_i32(new), lambda: None)
+    act, src = H.dev_i32(old), H.dev_i32(new)
+    got = run(act, lambda: writer(grid=(1, 1, 1), block=(32, 1, 1), args=[act, src, new.size]))
+    assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(want, got))
