@@ -476,7 +476,8 @@ struct ScoreDev {
 
 constexpr int SC_WARPS = 4;  // pages per CTA
 static_assert(SC_WARPS * PAGE == PLAN_GROUP_TOKENS, "a unit of attn_score is one page per warp");
-constexpr int SC_PER_SM = 12;  // CTAs per SM of the grid: twice what is resident (6 and 24 measured the same within 1 %)
+constexpr int SC_PER_SM = 12;  // CTAs per SM of the grid: twice what is resident at head_dim 64 (6), four times at 128 (3: a CTA
+                               // holds 64 KB of keys); 6 and 24 measured the same within 1 %
 
 template <int HD, int HG>
 __global__ void __launch_bounds__(SC_WARPS * 32) attn_score_kernel(const ScoreDev p) {
@@ -650,7 +651,7 @@ struct SelectDev {
   int* status;
 };
 
-// Exclusive prefix sum of v over the 256 threads (in thread order) and the block total.
+// Exclusive prefix sum of v over the TS_THREADS threads (in thread order) and the block total.
 __device__ __forceinline__ int ts_block_scan(int v, int& total, int* warp_tot) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int incl = v;
@@ -1110,7 +1111,8 @@ constexpr int GA_DENSE = 16;   // tokens per warp step of a row that keeps every
 
 // Pass 2 is a gather of 128- or 256-byte V rows with G multiply-adds per element: bound by how many row
 // fetches are in flight, so the rows travel by asynchronous 16-byte copies into per-warp rings of shared
-// memory (about 190 KB per SM, three quarters of it in flight) and the registers only hold accumulators.
+// memory (about 190 KB per SM; of a ring's three batches one is worked on and two are in flight) and the registers only
+// hold accumulators.
 //
 // The warps of one persistent CTA per SM work through the list of items, each warp on its own: an item is
 // (sequence, kv-head, run of tokens of which about 64 to 1024 are kept); a warp's first item is dealt by its index

@@ -289,15 +289,10 @@ inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_page
   L.sigma = take(BK * Tmax * 4);
   L.row_hist = take(BK * 4096 * 4);
   L.row_ctl = take(BK * 8 * 4);
-  // not used; the sum stays what sol_workspace_bytes has always answered and the static scratch's limit is made of
-  take(BK * ((Tmax + 2047) / 2048) * 4);
-  take(BK * 1024 * 8);
-  L.kept_idx = take(BK * Tmax * 4);
+  L.kept_idx = take(BK * Tmax * 4);  // this list and kept_row: Quest mode
   L.kept_cnt = take(BK * 4);
   L.kept_row = take(BK * Tmax * 4);
   L.part = take(BK * L.splits * G * (hd + 2) * 4);
-  take(3 * 132 * 4);  // not used, see above
-  take(BK * L.splits * 8);  // not used, see above
   L.work_ctr = take((4 + BK) * 4);
   const bool quest = s.token_select == SOL_SELECT_QUEST_PAGES;
   L.page_mask = take(quest ? BK * (Tmax / 4) : 0);
@@ -307,6 +302,12 @@ inline AttnScratch attn_scratch_layout(const sol_shape_t& s, int B, int max_page
   L.quest_qsplit = take(quest ? (size_t)B * Hkv * ((Hq / Hkv + 3) / 4) * 16 * 2 * hd * 2 : 0);
   L.quest_l1 = take(quest ? (size_t)B * Hq * 4 : 0);
   L.quest_order = take(quest ? (size_t)B * 4 : 0);
+  // Reserved, as the lists above are in every mode: a program asks sol_workspace_bytes once and keeps the figure, and the
+  // static scratch must refuse the same problems in every build, so the sum does not shrink with what the kernels use.
+  take(BK * ((Tmax + 2047) / 2048) * 4);
+  take(BK * 1024 * 8);
+  take(3 * 132 * 4);
+  take(BK * L.splits * 8);
   L.end = at;
   return L;
 }

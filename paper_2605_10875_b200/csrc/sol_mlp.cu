@@ -442,6 +442,7 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
     // error taken for g_j, u_j: the tensor cores add each 16-long slice of the dot product to the running
     // float32 sum with truncation, so the error grows with the d/16 steps: (d/16) * 2^-24 of the largest
     // magnitude, and never less than 2^-18 of it; carried into t through |silu'| <= 1.1, |silu(g)| <= |g|
+    // (a multiple of the error that was measured, no proven bound; the product of both errors is left out)
     eps = fmaxf(3.814697265625e-06f, (float)(d / 16) * 5.9604644775390625e-08f) * fmaxf(gmax, umax);
     // the m-th largest exact |t| lies within the largest error any channel can carry of the bin; a channel is
     // settled when its own error cannot carry it across that

@@ -37,9 +37,9 @@ struct SelectSmem {
   int counts[4];
 };
 
-// The same members for a kernel that never needs the histogram and the candidate arrays at the same time (the
-// settling kernel: a row either fits the candidate list or is redone by the radix select, which alone uses the
-// histogram): they share their space, 19 KB instead of 35 KB, so that one more CTA fits on an SM.
+// The same members for a kernel that never needs the histogram and the candidate arrays at the same time (the token
+// selection: its candidates are listed when the row's histogram is no longer read, and a row that does not fit the
+// list is redone by the radix select, which takes the space back): they share their space, 19 KB instead of 35 KB.
 struct SelectSmemOverlay {
   union {
     uint32_t hist[SEL_BINS];

@@ -1,4 +1,5 @@
-"""Kernels at the sizes where their tiling can go wrong: remainders, single tiles, the smallest and largest of a range."""
+"""Kernels at the sizes where their tiling can go wrong: remainders, single tiles, the smallest and largest of a range;
+values that a wrong step shows in (zeros, infinities, NaNs); inputs that are written late."""
 import numpy as np
 import pytest
 import torch
@@ -11,9 +12,10 @@ from tests.test_gpu_parity import TINY, _attention_case, _mlp_case
 pytestmark = pytest.mark.gpu
 
 
-# The row-by-row down projection: every register layout (1, 2, 3-4, 5-8 tokens), channel ranges shorter than a warp's group
+# The row-by-row down projection: every register layout (1, 2, 3, 4, 5-8 tokens), channel ranges shorter than a warp's group
 # of 32, one group per warp, and several; rates that leave no kept row, a few (an odd last pair) and all of them.
-@pytest.mark.parametrize("B,ff", [(1, 32), (2, 96), (3, 2080), (5, 160), (7, 12320), (2, 20512), (8, 20512)])
+@pytest.mark.parametrize("B,ff", [(1, 32), (2, 96), (3, 2080), (4, 160), (5, 160), (4, 12320), (7, 12320), (2, 20512), (3, 20512),
+                                  (8, 20512)])
 def test_down_rows_tiles(B, ff):
     cfg = dict(TINY, d_ff=ff)
     rates = [1000, 999, 960, 500, 37, 0, 750, 875]
