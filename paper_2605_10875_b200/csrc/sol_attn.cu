@@ -33,7 +33,10 @@ namespace sol {
 
 constexpr int PLAN_STRIDE = 132;  // words of a cumulative work list: entry b is the count before sequence b (per kv-head), entry B the total
 constexpr int PLAN_GROUP_TOKENS = 4 * PAGE;  // tokens of one pass-1 unit (a CTA of attn_score: one page per warp)
-constexpr int TH_SEG = 8192;  // tokens per token_select CTA
+// Tokens per token_select CTA.  A row of several segments costs a flush of its histogram, a ticket and a second walk over its
+// scores: with 8192 (and three CTAs per SM) the selection of 64 sequences of 16384 tokens took 42 us, this 33; 128 ragged
+// sequences 39 and 34.
+constexpr int TH_SEG = 16384;
 
 // What every selection kernel derives from a row's length and keep-rate.
 struct RowPlan {
@@ -634,7 +637,7 @@ __global__ void __launch_bounds__(SC_WARPS * 32) attn_score_kernel(const ScoreDe
 // rolled loops over them in shared memory (unrolled over registers, the code of a unit was fetched cold for 14 us even
 // where a launch has one unit of 2000 scores), and 512 threads.
 constexpr int TS_THREADS = 512;
-constexpr int TS_PER_SM = 3;  // CTAs per SM of the persistent grid: 53 KB of shared memory and 48 warps
+constexpr int TS_PER_SM = 2;  // CTAs per SM of the persistent grid: 85 KB of shared memory
 constexpr float TS_FLT_MAX = 3.402823466e+38f;
 
 struct SelectDev {
@@ -680,8 +683,11 @@ struct SelSmem {
   uint64_t bar;
   double qsum[128];
   float fmax_w[TS_THREADS / 32];
-  int s_flag, s_next;
+  int s_flag;
   int cum[PLAN_STRIDE], wsum[4];
+  alignas(16) int len[128];      // tokens of a sequence that needs a selection, 0 of the others
+  unsigned char order[128];      // the sequences, those with the most units first
+  int unit_b, unit_kvh, unit_seg;  // the next unit (unit_b < 0: none)
 };
 
 // The end of a row's selection, by one CTA: n_list tokens lie above the edge or are forced; ns_all candidates lie
@@ -689,7 +695,7 @@ struct SelSmem {
 // float32, re-scores those within the window of the k-th value in float64 from the cache rows, and gives the
 // kept ones an infinite score.
 __device__ __forceinline__ void settle_row(const SelectDev& p, SelectSmemOverlay& sm, double* qsum, const RowPlan& rp, int b,
-                                           int kvh, int n_list, float edge, float lo, float delta, int ns_all) {
+                                           int kvh, int n_list, float edge, float lo, float delta, int ns_all, bool live) {
   const int Hkv = p.sh.n_kv_heads, hd = p.sh.head_dim, G = p.sh.n_q_heads / Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int WARPS = TS_THREADS / 32;
@@ -820,36 +826,48 @@ __device__ __forceinline__ void settle_row(const SelectDev& p, SelectSmemOverlay
         const double vo = sm.cand_val[o];
         rank += (vo > v) || (vo == v && sm.cand_idx[o] < j);
       }
-      if (__reduce_add_sync(0xffffffffu, rank) < need_s && lane == 0) sig[j] = INFINITY;
+      if (__reduce_add_sync(0xffffffffu, rank) < need_s && lane == 0 && live) sig[j] = INFINITY;
     }
     n_list += need_s;
   }
-  if (tid == 0) p.kept_cnt[bk] = n_list;
+  if (tid == 0 && live) p.kept_cnt[bk] = n_list;
 }
 
+constexpr int TS_REHEARSAL = 1024;  // scores of a rehearsal
+
 // One (sequence, kv-head, 8192-token segment) of a row that needs a selection; the phase of hs.bar is the caller's.
-__device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& hs, int b, int kvh, int seg, uint32_t& phase) {
+// live == false: a rehearsal on made-up scores, 1/64 apart, which reads and writes shared memory only.  scores_read: called
+// by all threads when hs.score is no longer needed (the caller then lets the next unit's scores come).
+template <typename ScoresRead>
+__device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& hs, int b, int kvh, int seg, uint32_t& phase, bool live,
+                                                  ScoresRead scores_read) {
   SelectSmemOverlay& sm = hs.sm;
   uint32_t* hist = sm.hist;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, b);
+  RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, b);
+  if (!live) {
+    rp.T = TS_REHEARSAL;
+    rp.k = TS_REHEARSAL / 4;
+    rp.n_sink = 0;
+    rp.nf = rp.n_win = 1;
+    rp.mode = 2;
+    seg = 0;
+  }
   const int T = rp.T;
-  if (rp.mode != 2 || seg * TH_SEG >= T) return;
   const int bk = b * p.sh.n_kv_heads + kvh;
   const float* sig = p.sigma + (size_t)bk * p.Tmax;
   uint32_t* ctl = p.row_ctl + (size_t)bk * RC_WORDS;
   uint32_t* gh = p.row_hist + (size_t)bk * SEL_BINS;
   const int nseg = (T + TH_SEG - 1) / TH_SEG;
   const int j_first = seg * TH_SEG, n_here = min(T - j_first, TH_SEG);
-  if (tid == 0) {  // a row's space ends on a full page, so whole groups of four may be read
-    const uint32_t bytes = (uint32_t)((n_here + 3) & ~3) * 4;
-    mbar_expect_tx(&hs.bar, bytes);
-    bulk_g2s(hs.score, sig + j_first, bytes, &hs.bar);
-  }
+  if (!live)
+    for (int i = tid; i < TS_REHEARSAL; i += TS_THREADS) hs.score[i] = (float)((i * 389) & (TS_REHEARSAL - 1)) * 0.015625f;
   for (int i = tid; i < SEL_BINS / 4; i += TS_THREADS) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
-  mbar_wait(&hs.bar, phase, p.status);  // a wait that gives up is reported; what follows stays in bounds
-  phase ^= 1;
+  if (live) {
+    mbar_wait(&hs.bar, phase, p.status);  // a wait that gives up is reported; what follows stays in bounds
+    phase ^= 1;
+  }
 
   float mx = 0.f;
   bool nan_here = false;
@@ -872,6 +890,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   int any_nan = __syncthreads_or(nan_here ? 1 : 0);
   mx = warp_max(lane < TS_THREADS / 32 ? hs.fmax_w[lane] : 0.f);
   if (nseg > 1) {  // only the CTA that arrives last goes on
+    scores_read();
     for (int i = tid; i < SEL_BINS; i += TS_THREADS) {
       const uint32_t c = hist[i];
       if (c) atomicAdd(gh + i, c);
@@ -954,7 +973,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   const float lo = key_to_float(klo) - delta;
   const float edge = fminf(bin_hi + delta, TS_FLT_MAX);
   if (tid == 0) {
-    ctl[RC_EDGE] = __float_as_uint(edge);  // for pass 2 and token_list
+    if (live) ctl[RC_EDGE] = __float_as_uint(edge);  // for pass 2 and token_list
     sm.counts[0] = 0;
   }
   __syncthreads();  // the histogram is not read any more: the candidates take its space
@@ -997,6 +1016,7 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
   }
   in_window = block_count<TS_THREADS>(in_window, 0, sm);  // the barrier inside also publishes the candidates
   above -= in_window;
+  if (nseg == 1) scores_read();
   // Counted again where the histogram's ranks say something else than "above the edge": it ranks what is not a number as
   // a large score, but that is never kept; and where the k-th score lies in the top bin, whose end is +inf, scores of
   // +inf are no higher than the bin but above the edge, and all of them are kept.
@@ -1005,37 +1025,89 @@ __device__ __forceinline__ void token_select_item(const SelectDev& p, SelSmem& h
     for (int j = tid; j < T; j += TS_THREADS) n += !rp.forced(j) && sig[j] > edge ? 1 : 0;
     above = block_count<TS_THREADS>(n, 1, sm);
   }
-  settle_row(p, sm, hs.qsum, rp, b, kvh, above + rp.nf, edge, lo, delta, sm.counts[0]);
+  settle_row(p, sm, hs.qsum, rp, b, kvh, above + rp.nf, edge, lo, delta, sm.counts[0], live);
 }
 
-// Persistent CTAs over the flat list of (sequence, kv-head, segment) units of the rows that need a selection.
-__global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(const SelectDev p) {
+// Persistent CTAs over the flat list of (sequence, kv-head, segment) units of the rows that need a selection, the longest
+// rows first: their last CTA has the whole row to settle.  A CTA's first unit is its index, the later ones are claimed; the
+// last warp claims a unit while the one before is worked on and requests its scores as soon as they may be overwritten
+// (with the units in batch order, claimed in the way of the first warp and their scores requested when the unit began, 128
+// ragged sequences took 48 us; this, with segments of 8192 tokens, 39).
+// `rehearse`: the unit's code is run once on made-up scores ahead of the wait and is then in the instruction caches; its first
+// pass through code that comes from L2 took as long again (a single sequence of 2000 tokens: 9.1 us in the chain, 6.8).
+__global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(const SelectDev p, int rehearse) {
   extern __shared__ __align__(128) unsigned char ts_smem[];
   SelSmem& hs = *reinterpret_cast<SelSmem*>(ts_smem);
+  const int tid = threadIdx.x, Hkv = p.sh.n_kv_heads;
+  const bool fetcher = tid == TS_THREADS - 32;
   pdl_trigger();
-  if (threadIdx.x == 0) {
+  if (fetcher) {
     mbar_init(&hs.bar, 1);
     fence_mbar_init();
   }
-  int cnt = 0;
-  if ((int)threadIdx.x < p.B) {
-    const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, threadIdx.x);
-    if (rp.mode == 2) cnt = (rp.T + TH_SEG - 1) / TH_SEG;
+  int len = 0;
+  if (tid < 128) {
+    if (tid < p.B) {
+      const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
+      if (rp.mode == 2) len = rp.T;
+    }
+    hs.len[tid] = len;
   }
-  plan_scan(cnt, hs.cum, hs.wsum);
-  pdl_wait();
-  const int Hkv = p.sh.n_kv_heads;
-  const int n_units = hs.cum[p.B] * Hkv;
+  __syncthreads();
+  if (tid < 128) {
+    int rank = 0;
+#pragma unroll 1
+    for (int j = 0; j < 128; j += 4) {
+      const int4 x = *reinterpret_cast<const int4*>(hs.len + j);
+      rank += (x.x > len || (x.x == len && j < tid)) + (x.y > len || (x.y == len && j + 1 < tid)) +
+              (x.z > len || (x.z == len && j + 2 < tid)) + (x.w > len || (x.w == len && j + 3 < tid));
+    }
+    hs.order[rank] = (unsigned char)tid;
+  }
+  __syncthreads();
+  plan_scan(tid < 128 ? (hs.len[hs.order[tid]] + TH_SEG - 1) / TH_SEG : 0, hs.cum, hs.wsum);
+  const int n_units = hs.cum[128] * Hkv;
   uint32_t phase = 0;
-  // a CTA's first unit is its index, the later ones are claimed (while the unit before is worked on): the CTA that
-  // comes last on a row has the whole of it to settle, and units dealt by index left some CTAs with several such rows
-  for (int u = blockIdx.x; u < n_units;) {
-    if (threadIdx.x == 0) hs.s_next = (int)gridDim.x + atomicAdd(p.work_ctr + WC_SELECT, 1);
-    const int b = plan_find(hs.cum, p.B, u / Hkv);
-    const int n = hs.cum[b + 1] - hs.cum[b], rem = u - hs.cum[b] * Hkv;
-    token_select_item(p, hs, b, rem / n, rem % n, phase);
-    __syncthreads();
-    u = hs.s_next;
+  int live = rehearse && (int)blockIdx.x < n_units ? 0 : 1;
+  int unit = blockIdx.x, next = blockIdx.x;
+  // by the fetcher: looks unit u up and requests its scores
+  auto fetch = [&](int u) {
+    hs.unit_b = -1;
+    if (u < n_units) {
+      const int at = plan_find(hs.cum, 128, u / Hkv), b = hs.order[at];
+      const int n = hs.cum[at + 1] - hs.cum[at], rem = u - hs.cum[at] * Hkv, kvh = rem / n, seg = rem - kvh * n;
+      hs.unit_b = b;
+      hs.unit_kvh = kvh;
+      hs.unit_seg = seg;
+      // a row's space ends on a full page, so whole groups of four may be read
+      const uint32_t bytes = (uint32_t)((min(hs.len[b] - seg * TH_SEG, TH_SEG) + 3) & ~3) * 4;
+      mbar_expect_tx(&hs.bar, bytes);
+      bulk_g2s(hs.score, p.sigma + (size_t)(b * Hkv + kvh) * p.Tmax + seg * TH_SEG, bytes, &hs.bar);
+    }
+  };
+  if (live) {
+    pdl_wait();
+    if (fetcher) fetch(unit);
+  } else if (tid == 0) {
+    hs.unit_b = hs.unit_kvh = hs.unit_seg = 0;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (;;) {
+    asm volatile("" : "+r"(live));  // one code for a rehearsal and a unit
+    const int b = hs.unit_b, kvh = hs.unit_kvh, seg = hs.unit_seg;
+    if (b < 0) break;
+    if (live && fetcher) next = n_units > (int)gridDim.x ? (int)gridDim.x + atomicAdd(p.work_ctr + WC_SELECT, 1) : n_units;
+    token_select_item(p, hs, b, kvh, seg, phase, live != 0, [&] {
+      if (live && fetcher) fetch(next);
+    });
+    if (!live) {
+      pdl_wait();
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the made-up scores are overwritten by a bulk copy
+      __syncthreads();
+      live = 1;
+      if (fetcher) fetch(unit);
+    }
     __syncthreads();
   }
 }
@@ -1631,8 +1703,13 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   // persistent grid: a few CTAs per SM, never more than there can be units
   const long long sel_units = (long long)a.B * Hkv * ((Tmax + TH_SEG - 1) / TH_SEG), sel_res = (long long)sm_count() * TS_PER_SM;
   ensure_dynamic_smem(reinterpret_cast<const void*>(&token_select_kernel), (int)sizeof(SelSmem));
-  SOL_LAUNCH("token_select", token_select_kernel, dim3((unsigned)(sel_units < sel_res ? sel_units : sel_res)),
-             dim3(TS_THREADS), sizeof(SelSmem), st, se);
+  const int sel_ctas = (int)(sel_units < sel_res ? sel_units : sel_res);
+  const long long score_ctas = (long long)a.B * Hkv * groups_per_row;
+  // A rehearsal (about 3 us) pays where a CTA is there well before the pass 1 ends: where the CTAs of both leave room for each
+  // other on every SM.  Elsewhere a CTA starts when one of pass 1 ends, and a rehearsal is in its way (16 sequences of 4096
+  // tokens: 10.2 us without, 12.9 with it).
+  const int rehearse_select = score_ctas + sel_ctas <= 3LL * sm_count();
+  SOL_LAUNCH("token_select", token_select_kernel, dim3((unsigned)sel_ctas), dim3(TS_THREADS), sizeof(SelSmem), st, se, rehearse_select);
   if (a.kept_idx_out != nullptr) {
     ListDev ld;
     ld.sh = sh; ld.kv = a.kv; ld.r_permille = a.r_permille; ld.Tmax = Tmax; ld.sigma = a.sigma; ld.row_ctl = a.row_ctl;

@@ -41,6 +41,19 @@ def test_attention_rows_around_a_selection_segment(hd):
     _attention_case(cfg, [8191, 8192, 8193, 16385, 40], [125, 500, 250, 1000, 300], seed=hd)
 
 
+# The token selection around one segment (16384 tokens) and over several, and more units than CTAs are resident.
+@pytest.mark.parametrize("lens,r", [([16383, 16384, 16385, 1], [125, 500, 999, 500]), ([33000, 100, 49152], [250, 500, 60])])
+def test_token_selection_segments(lens, r):
+    _attention_case(TINY, lens, r, seed=len(lens), n_sink=3, n_window=2)
+
+
+def test_attention_of_a_full_batch():
+    """More units of the selection and more items of pass 2 than are worked on at once, rows of every length and rate."""
+    cfg = dict(TINY, n_q_heads=8, n_kv_heads=8, d_model=512)
+    rng = np.random.default_rng(5)
+    _attention_case(cfg, rng.integers(1, 1300, 128), rng.choice([60, 125, 500, 999, 1000], 128), seed=5)
+
+
 # The exact re-scoring of the channel selection: rows shorter than, equal to and longer than what a CTA takes at once (2048
 # elements), and more open candidates than one pass takes (groups of identical channels around the threshold).
 @pytest.mark.parametrize("d,ff", [(256, 1056), (2048, 512), (2304, 512), (4096, 1024), (8192, 256)])
