@@ -74,8 +74,11 @@ __device__ __forceinline__ int gather_item_tokens(const RowPlan& rp, int c, int 
 // which are inputs of the step, while the kernels before are still running; a list made by one CTA of attn_prep stood in
 // that kernel's way and cost the readers a round trip to memory.
 
-// cum[b + 1] = cnt of sequences 0 .. b (cnt: this thread's sequence, threads 0 .. 127); cum[0] = 0.  Called by the whole
-// CTA (128 threads or more); wsum: four words of shared memory.
+// A barrier of the first 128 threads of a CTA.
+__device__ __forceinline__ void plan_sync() { asm volatile("bar.sync 1, 128;" ::: "memory"); }
+
+// cum[b + 1] = cnt of sequences 0 .. b (cnt: this thread's sequence); cum[0] = 0.  By the first 128 threads of the CTA; wsum:
+// four words of shared memory.
 __device__ __forceinline__ void plan_scan(int cnt, int* cum, int* wsum) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   int incl = cnt;
@@ -84,14 +87,12 @@ __device__ __forceinline__ void plan_scan(int cnt, int* cum, int* wsum) {
     const int x = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += x;
   }
-  if (lane == 31 && warp < 4) wsum[warp] = incl;
-  __syncthreads();
-  if (tid < 128) {
-    for (int w = 0; w < warp; ++w) incl += wsum[w];
-    cum[tid + 1] = incl;
-    if (tid == 0) cum[0] = 0;
-  }
-  __syncthreads();
+  if (lane == 31) wsum[warp] = incl;
+  plan_sync();
+  for (int w = 0; w < warp; ++w) incl += wsum[w];
+  cum[tid + 1] = incl;
+  if (tid == 0) cum[0] = 0;
+  plan_sync();
 }
 
 // The pass-2 items of every sequence into cum; returns the kept tokens c of an item, a power of two from 64 to 1024: the
@@ -106,50 +107,42 @@ constexpr int ITEM_C0 = 64, ITEM_NC = 5;
 struct PlanSmem {
   int cum[PLAN_STRIDE];
   int n_items[ITEM_NC], longest[ITEM_NC];  // per option: items of a kv-head, kept tokens of the longest
-  int wsum[4];
+  int wsum[4], per_item;
 };
+// By the first 128 threads of the CTA.  The options are tried in a rolled loop: this runs once per CTA, at the pace at which
+// its code is fetched.
 __device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t& kv, const int32_t* r_permille, int B, int min_len,
                                           int target_items, PlanSmem& ps) {
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < ITEM_NC) ps.n_items[tid] = ps.longest[tid] = 0;
-  __syncthreads();
-  int per_seq[ITEM_NC] = {0, 0, 0, 0, 0};
-  if (tid < 128) {
-    int kept = 0;
-    if (tid < B) {
-      const RowPlan rp = row_plan(sh, kv, r_permille, tid);
-      kept = max(rp.k, 0);
-#pragma unroll
-      for (int q = 0; q < ITEM_NC; ++q) {  // one item at least, so that the output is always written
-        const int len = gather_item_tokens(rp, ITEM_C0 << q, min_len);
-        per_seq[q] = max(1, (rp.T + len - 1) / len);
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < ITEM_NC; ++q) {
-      const int n = __reduce_add_sync(0xffffffffu, per_seq[q]);
-      const int most = __reduce_max_sync(0xffffffffu, per_seq[q] > 0 ? kept / per_seq[q] : 0);
-      if (lane == 0 && n) {
-        atomicAdd(&ps.n_items[q], n);
-        atomicMax(&ps.longest[q], most);
-      }
-    }
-  }
-  __syncthreads();
-  int pick = 0, cnt = 0;
-  long long best = 0x7fffffffffffffffLL;
-#pragma unroll
+  plan_sync();
+  RowPlan rp;
+  rp.T = rp.k = 0;
+  if (tid < B) rp = row_plan(sh, kv, r_permille, tid);
+  auto items_of = [&](int c) {  // one item at least, so that the output is always written
+    const int len = gather_item_tokens(rp, c, min_len);
+    return max(1, (rp.T + len - 1) / len);
+  };
+#pragma unroll 1
   for (int q = 0; q < ITEM_NC; ++q) {
-    const int rounds = (ps.n_items[q] * sh.n_kv_heads + target_items - 1) / target_items;
-    const long long cost = (long long)rounds * (ps.longest[q] + ITEM_FILL) + (ps.n_items[q] > B ? ITEM_MERGE : 0);
-    if (cost <= best) {
-      best = cost;
-      pick = q;
-      cnt = per_seq[q];
+    const int n = tid < B ? items_of(ITEM_C0 << q) : 0;
+    const int sum = __reduce_add_sync(0xffffffffu, n);
+    const int most = __reduce_max_sync(0xffffffffu, n > 0 ? max(rp.k, 0) / n : 0);
+    if (lane == 0 && sum) {
+      atomicAdd(&ps.n_items[q], sum);
+      atomicMax(&ps.longest[q], most);
     }
   }
-  plan_scan(cnt, ps.cum, ps.wsum);
-  return ITEM_C0 << pick;
+  plan_sync();
+  uint32_t key = 0xffffffffu;  // a lane per option; the larger c where two cost the same
+  if (lane < ITEM_NC) {
+    const int rounds = (ps.n_items[lane] * sh.n_kv_heads + target_items - 1) / target_items;
+    const int cost = rounds * (ps.longest[lane] + ITEM_FILL) + (ps.n_items[lane] > B ? ITEM_MERGE : 0);
+    key = ((uint32_t)cost << 3) | (uint32_t)(ITEM_NC - 1 - lane);
+  }
+  const int c = ITEM_C0 << (ITEM_NC - 1 - (int)(__reduce_min_sync(0xffffffffu, key) & 7u));
+  plan_scan(tid < B ? items_of(c) : 0, ps.cum, ps.wsum);
+  return c;
 }
 
 // The sequence that holds flat unit `u` of a cumulative list (cum[b] <= u < cum[b + 1]); n entries + total.
@@ -344,70 +337,79 @@ __device__ __forceinline__ void attn_write(const AttnOut& o, int b, int head, in
 }
 
 // Merges the ns partial results of a (sequence, kv-head), [ns][G][HD + 2] floats each (weighted sums, maximum in the
-// base-2 domain, sum of the weights), by one warp.  fac: ns * G floats of shared memory.
+// base-2 domain, sum of the weights), by one warp.  fac: ns * G floats of shared memory.  `live`: false for a rehearsal,
+// which writes nothing.
 template <int HD>
-__device__ __forceinline__ void merge_partials(const AttnOut& o, const float* src0, int ns, int b, int kvh, float* fac, int lane) {
+__device__ __forceinline__ void merge_partials(const AttnOut& o, const float* src0, int ns, int b, int kvh, float* fac, int lane,
+                                               bool live) {
   const int G = o.G;
   const size_t stride = (size_t)G * (HD + 2);
-  // factors of the partials: f[q][h] = 2^(m_q - M_h) / sum_q l_q 2^(m_q - M_h)
-  if (ns <= 32) {  // a partial per lane: every head's maximum and sum in one round trip
-    float2 ml[8];
+  // a lane's columns 2 lane, 2 lane + 1 of every 64: four such pairs of MU partials in flight, the first of them requested
+  // before the factors are made (four partials in flight, after the factors: 24 sequences of 2000 tokens 24.0 us, this 22.8;
+  // one pair of eight partials: 7.6 us for the 16 partials of a 4096-token row alone)
+  constexpr int MU = 8;
+  float2 v[4][MU];
+  auto request = [&](int p0, int q) {
 #pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      ml[h] = make_float2(-INFINITY, 0.f);
-      if (h < G && lane < ns) ml[h] = __ldcg(reinterpret_cast<const float2*>(src0 + (size_t)lane * stride + (size_t)h * (HD + 2) + HD));
-    }
+    for (int x = 0; x < 4; ++x) {
+      const int e0 = lane * 2 + 64 * (p0 + x), h = e0 / HD, e = e0 % HD;
+      const float* src = src0 + (size_t)q * stride + (size_t)h * (HD + 2) + e;
 #pragma unroll
-    for (int h = 0; h < 8; ++h) {
-      if (h >= G) break;
-      const float mm = warp_max(ml[h].x);
-      const float f = ml[h].x == -INFINITY ? 0.f : exp2f(ml[h].x - mm);
-      const float l = warp_sum(ml[h].y * f);
-      if (lane < ns) fac[lane * G + h] = l > 0.f ? f * (1.0f / l) : 0.f;
+      for (int u = 0; u < MU; ++u)
+        v[x][u] = p0 + x < G * HD / 64 && q + u < ns ? __ldcg(reinterpret_cast<const float2*>(src + u * stride)) : make_float2(0.f, 0.f);
     }
-  } else {
+  };
+  request(0, 0);
+  // factors of the partials: f[q][h] = 2^(m_q - M_h) / sum_q l_q 2^(m_q - M_h).  A lane takes head lane % 8 of every fourth
+  // partial, so that a head's maximum and sum are two exchanges
+  {
+    const int h = lane & 7, q0 = lane >> 3;
+    const float* src = src0 + (size_t)h * (HD + 2) + HD;
+    float mm = -INFINITY, l = 0.f;
 #pragma unroll 1
-    for (int h = 0; h < G; ++h) {
-      const float* src = src0 + (size_t)h * (HD + 2) + HD;
-      float mm = -INFINITY;
-      for (int q = lane; q < ns; q += 32) mm = fmaxf(mm, __ldcg(src + q * stride));
-      mm = warp_max(mm);
-      float l = 0.f;
-      for (int q = lane; q < ns; q += 32) {
-        const float m2 = __ldcg(src + q * stride);
-        const float f = m2 == -INFINITY ? 0.f : exp2f(m2 - mm);
-        fac[q * G + h] = f;
-        l += __ldcg(src + q * stride + 1) * f;
+    for (int q = q0; q < ns; q += 16) {
+      float2 ml[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        ml[u] = h < G && q + 4 * u < ns ? __ldcg(reinterpret_cast<const float2*>(src + (q + 4 * u) * stride)) : make_float2(-INFINITY, 0.f);
+      const float nm = fmaxf(fmaxf(mm, fmaxf(ml[0].x, ml[1].x)), fmaxf(ml[2].x, ml[3].x));
+      l *= mm == -INFINITY ? 0.f : exp2f(mm - nm);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        l += ml[u].x == -INFINITY ? 0.f : ml[u].y * exp2f(ml[u].x - nm);
+        if (h < G && q + 4 * u < ns) fac[(q + 4 * u) * G + h] = ml[u].x;
       }
-      l = warp_sum(l);
-      const float inv = l > 0.f ? 1.0f / l : 0.f;
-      for (int q = lane; q < ns; q += 32) fac[q * G + h] *= inv;
+      mm = nm;
     }
+#pragma unroll
+    for (int o2 = 8; o2 < 32; o2 <<= 1) {
+      const float m2 = __shfl_xor_sync(0xffffffffu, mm, o2), l2 = __shfl_xor_sync(0xffffffffu, l, o2);
+      const float nm = fmaxf(mm, m2);
+      l = (mm == -INFINITY ? 0.f : l * exp2f(mm - nm)) + (m2 == -INFINITY ? 0.f : l2 * exp2f(m2 - nm));
+      mm = nm;
+    }
+    const float inv = l > 0.f ? 1.0f / l : 0.f;
+    if (h < G)
+#pragma unroll 1
+      for (int q = q0; q < ns; q += 4) {
+        const float m2 = fac[q * G + h];
+        fac[q * G + h] = m2 == -INFINITY ? 0.f : exp2f(m2 - mm) * inv;
+      }
   }
   __syncwarp();
-  // a lane's columns 2 lane, 2 lane + 1 of every 64: four such pairs of four partials in flight (one pair of eight partials:
-  // twice the round trips, 7.6 us for the 16 partials of a 4096-token row, its last warp's alone)
 #pragma unroll 1
   for (int p0 = 0; p0 < G * HD / 64; p0 += 4) {
     float2 a[4];
 #pragma unroll
     for (int x = 0; x < 4; ++x) a[x] = make_float2(0.f, 0.f);
 #pragma unroll 1
-    for (int q = 0; q < ns; q += 4) {
-      float2 v[4][4];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int e0 = lane * 2 + 64 * (p0 + x), h = e0 / HD, e = e0 % HD;
-        const float* src = src0 + (size_t)q * stride + (size_t)h * (HD + 2) + e;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          v[x][u] = p0 + x < G * HD / 64 && q + u < ns ? __ldcg(reinterpret_cast<const float2*>(src + u * stride)) : make_float2(0.f, 0.f);
-      }
+    for (int q = 0; q < ns; q += MU) {
+      if (p0 + q > 0) request(p0, q);
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         const int h = min((lane * 2 + 64 * (p0 + x)) / HD, G - 1);
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < MU; ++u) {
           const float f = q + u < ns ? fac[(q + u) * G + h] : 0.f;
           a[x].x = fmaf(v[x][u].x, f, a[x].x);
           a[x].y = fmaf(v[x][u].y, f, a[x].y);
@@ -417,7 +419,7 @@ __device__ __forceinline__ void merge_partials(const AttnOut& o, const float* sr
 #pragma unroll
     for (int x = 0; x < 4; ++x) {
       const int e0 = lane * 2 + 64 * (p0 + x);
-      if (p0 + x < G * HD / 64) attn_write<HD>(o, b, kvh * G + e0 / HD, e0 % HD, a[x].x, a[x].y);
+      if (p0 + x < G * HD / 64 && live) attn_write<HD>(o, b, kvh * G + e0 / HD, e0 % HD, a[x].x, a[x].y);
     }
   }
 }
@@ -1045,16 +1047,14 @@ __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(con
     mbar_init(&hs.bar, 1);
     fence_mbar_init();
   }
-  int len = 0;
   if (tid < 128) {
+    int len = 0;
     if (tid < p.B) {
       const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
       if (rp.mode == 2) len = rp.T;
     }
     hs.len[tid] = len;
-  }
-  __syncthreads();
-  if (tid < 128) {
+    plan_sync();
     int rank = 0;
 #pragma unroll 1
     for (int j = 0; j < 128; j += 4) {
@@ -1063,9 +1063,10 @@ __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(con
               (x.z > len || (x.z == len && j + 2 < tid)) + (x.w > len || (x.w == len && j + 3 < tid));
     }
     hs.order[rank] = (unsigned char)tid;
+    plan_sync();
+    plan_scan((hs.len[hs.order[tid]] + TH_SEG - 1) / TH_SEG, hs.cum, hs.wsum);
   }
   __syncthreads();
-  plan_scan(tid < 128 ? (hs.len[hs.order[tid]] + TH_SEG - 1) / TH_SEG : 0, hs.cum, hs.wsum);
   const int n_units = hs.cum[128] * Hkv;
   uint32_t phase = 0;
   int live = rehearse && (int)blockIdx.x < n_units ? 0 : 1;
@@ -1174,6 +1175,7 @@ struct GatherDev {
   float scale_log2;
   AttnOut out;
   int* status;
+  int rehearse;
 };
 
 constexpr int GA_BATCH = 32;   // kept tokens per warp step: one per lane in the softmax part
@@ -1214,6 +1216,7 @@ struct GatherCfg {
   static constexpr int WARPS = gather_warps(HD, GMAX);
   static constexpr int NST = 3;                              // batches of rows per warp ring
   static constexpr int STAGE_BYTES = GA_BATCH * HD * 2;      // 4 KB / 8 KB
+  static constexpr int REHEARSE = WARPS - WARPS / 4;         // the first of the warps that rehearse
   static constexpr int THREADS = WARPS * 32;
   static constexpr int RING_BYTES = WARPS * NST * STAGE_BYTES;  // 192 KB (hd 64, G > 4: 144 KB)
   static constexpr int LOG_BYTES = GA_BATCH * GMAX * 4;         // logits of a batch, then its weights
@@ -1240,24 +1243,56 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
   uint16_t* my_q = reinterpret_cast<uint16_t*>(gsm + C::RING_BYTES + C::W_BYTES) + warp * GA_QUEUE;
   float* ml = reinterpret_cast<float*>(my_q);  // at the end of an item: [GMAX] maxima, [GMAX] sums
   pdl_trigger();
-  const int per_item = plan_items(p.sh, p.kv, p.r_permille, p.B, p.min_len, p.sms * WARPS, ps);
-  pdl_wait();
-  const int n_items = cum[p.B] * Hkv;
+  // The first four warps make the list of items; the others wait for it at a barrier that the first four only arrive at.
+  // Where CTAs are there early (`rehearse`), the last quarter of the warps rehearse meanwhile: they run the code of an item
+  // on absent tokens (even warps that of a selected row, odd ones that of a row that keeps every token), write nothing and
+  // leave the code in the instruction caches.  The first pass through code that comes from L2 was half of the time of a
+  // launch with one item per warp (a single sequence of 2000 tokens: 19.5 us in the chain, 11.8 with the rehearsal).
+  int live = 1, per_item = 0, n_items = 0, item = warp * gridDim.x + blockIdx.x;
+  bool planned = false, waited = false;
   const int total_warps = gridDim.x * WARPS;
-
+  if (warp < 4) {
+    per_item = plan_items(p.sh, p.kv, p.r_permille, p.B, p.min_len, p.sms * WARPS, ps);
+    if (threadIdx.x == 0) ps.per_item = per_item;
+    n_items = cum[p.B] * Hkv;
+    planned = true;
+    asm volatile("bar.arrive 2, %0;" ::"n"(C::THREADS) : "memory");  // the list is there
+  } else if (p.rehearse && warp >= C::REHEARSE) {
+    live = 0;
+  }
 #pragma unroll 1
-  for (int item = warp * gridDim.x + blockIdx.x; item < n_items;) {
-    // the next item is claimed now, while this one is worked on
-    int claimed = 0;
-    if (lane == 0) claimed = total_warps + atomicAdd(p.work_ctr + WC_NEXT, 1);
-    const int b = plan_find(cum, p.B, item / Hkv);
-    const int ns = cum[b + 1] - cum[b], rem = item - cum[b] * Hkv;  // items of every (sequence, kv-head) of this sequence
-    const int kvh = rem / ns, slot = rem - kvh * ns;
+  for (;;) {
+    asm volatile("" : "+r"(live));  // one code for both
+    if (live) {
+      if (!planned) {
+        asm volatile("bar.sync 2, %0;" ::"n"(C::THREADS) : "memory");
+        planned = true;
+        per_item = ps.per_item;
+        n_items = cum[p.B] * Hkv;
+      }
+      if (item >= n_items) break;
+    }
+    int b = 0, ns = 1, kvh = 0, slot = 0;
+    if (live) {
+      b = plan_find(cum, p.B, item / Hkv);
+      ns = cum[b + 1] - cum[b];  // items of every (sequence, kv-head) of this sequence
+      const int rem = item - cum[b] * Hkv;
+      kvh = rem / ns;
+      slot = rem - kvh * ns;
+    }
+    const bool split = !live || ns > 1;
     const int bk = b * Hkv + kvh;
     const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, b);
-    const int len = gather_item_tokens(rp, per_item, p.min_len);
+    const int len = gather_item_tokens(rp, live ? per_item : ITEM_C0, p.min_len);
     const int n0 = slot * len, n1 = min(rp.T, n0 + len);  // this item's tokens; n0 is a multiple of 128
     const int32_t* table = p.kv.page_table + (size_t)b * p.kv.max_pages_per_seq;
+    if (live && !waited) {
+      pdl_wait();
+      waited = true;
+    }
+    // the next item is claimed now, while this one is worked on
+    int claimed = n_items;
+    if (live && n_items > total_warps && lane == 0) claimed = total_warps + atomicAdd(p.work_ctr + WC_NEXT, 1);
 
     float acc[HD / 16][4];
 #pragma unroll
@@ -1265,11 +1300,11 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
 #pragma unroll
       for (int c = 0; c < 4; ++c) acc[j][c] = 0.f;
 
-    if (rp.dense()) {
+    if (live ? rp.dense() : (warp & 1) != 0) {
       // ================= a run of a row that keeps every token =================
       // a lane's page of the run (1024 tokens at most)
       int pg = -1;
-      if (n0 + lane * PAGE < n1) {
+      if (live && n0 + lane * PAGE < n1) {
         pg = table[n0 / PAGE + lane];
         if (pg < 0 || pg >= p.kv.num_pages) {
           atomicOr(p.status + ST_ERR, ERR_BAD_PAGE);
@@ -1288,7 +1323,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
 #pragma unroll
             for (int x = 0; x < 2; ++x)
               qb[hg][ks][n][x] =
-                  hg * 4 < G ? *reinterpret_cast<const uint32_t*>(q + (size_t)(8 * n + g) * HD + ks * 16 + x * 8 + 2 * t) : 0u;
+                  hg * 4 < G && live ? *reinterpret_cast<const uint32_t*>(q + (size_t)(8 * n + g) * HD + ks * 16 + x * 8 + 2 * t) : 0u;
       }
       float mt[HG], lt[HG];  // head 4 hg + t: running maximum, this lane's share of the sum
 #pragma unroll
@@ -1296,7 +1331,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         mt[hg] = -INFINITY;
         lt[hg] = 0.f;
       }
-      const int nstep = (n1 - n0 + GA_DENSE - 1) / GA_DENSE;
+      const int nstep = live ? (n1 - n0 + GA_DENSE - 1) / GA_DENSE : 1;
       int slot_w = 0;
 #pragma unroll 1
       for (int s = 0; s - (NST - 1) < nstep; ++s) {
@@ -1406,7 +1441,8 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
       const size_t row = (size_t)bk * p.Tmax;
       const float* sig = p.sigma + row;
       const float* lgrow = p.logits + row * G;
-      const float edge = rp.mode == 2 ? __uint_as_float(p.row_ctl[(size_t)bk * RC_WORDS + RC_EDGE]) : INFINITY;
+      const bool scored = rp.mode == 2 && live;
+      const float edge = scored ? __uint_as_float(p.row_ctl[(size_t)bk * RC_WORDS + RC_EDGE]) : INFINITY;
 
       // ---- the queue of kept tokens' offsets from n0; the scores of the next two chunks wait in registers: lane l holds
       //      tokens 4 l .. 4 l + 3 of both halves of a chunk ----
@@ -1417,7 +1453,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         for (int x = 0; x < 2; ++x) {
           const int j = base + x * (GA_CHUNK / 2) + lane * 4;
           v[x] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-          if (j < n1 && rp.mode == 2) v[x] = *reinterpret_cast<const float4*>(sig + j);  // a row's space ends on a full page
+          if (j < n1 && scored) v[x] = *reinterpret_cast<const float4*>(sig + j);  // a row's space ends on a full page
         }
       };
       fetch_scores(c_at, sv);
@@ -1446,6 +1482,10 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
               if (rp.forced(j)) keep |= 1u << e;
               if (j >= n1) keep &= ~(1u << e);
             }
+          }
+          if (!live) {
+            keep = 0;
+            c_at = n1;
           }
           __syncwarp();
           if (lane < left) my_q[lane] = moved;
@@ -1476,13 +1516,12 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         mt[hg] = -INFINITY;
         lt[hg] = 0.f;
       }
-      int2 e_cur = pop();
-      int nb = q_tail > q_head ? 0x7fffffff : 0;  // batches of the item: known once a pop comes back empty
-      q_head = min(q_tail, q_head + GA_BATCH);
-      int slot_w = 0;  // ring slot of batch s
+      int2 e_cur = make_int2(-1, 0);
+      int nb = 0x7fffffff;   // batches of the item: known once a pop comes back empty
+      int slot_w = NST - 1;  // ring slot of batch s
 #pragma unroll 1
-      for (int s = 0; s - (NST - 1) < nb; ++s) {
-        if (s < nb) {  // the rows and the logits of batch s
+      for (int s = -1; s - (NST - 1) < nb; ++s) {
+        if (s >= 0 && s < nb) {  // the rows and the logits of batch s
           const uint32_t dst0 = smem_u32(my_ring + slot_w * C::STAGE_BYTES);
 #pragma unroll
           for (int i = 0; i < CPR; ++i) {
@@ -1509,7 +1548,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
         e_cur = make_int2(-1, 0);
         if (s + 1 < nb) {
           e_cur = pop();
-          if (q_tail == q_head) nb = s + 1;
+          if (q_tail == q_head && (live || s >= 0)) nb = s + 1;  // (a rehearsal takes one batch of absent tokens)
           q_head = min(q_tail, q_head + GA_BATCH);
         }
         slot_w = slot_w + 1 == NST ? 0 : slot_w + 1;
@@ -1607,28 +1646,32 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
     for (int e0 = lane * 2; e0 < G * HD; e0 += 64) {
       const int h = e0 / HD, e = e0 % HD;
       const float2 v = *reinterpret_cast<const float2*>(ob + e0);
-      if (ns == 1) {  // the row is this one item: its output goes out directly
+      if (!split) {  // the row is this one item: its output goes out directly
         const float l = ml[GMAX + h], inv = l > 0.f ? 1.0f / l : 0.f;
         attn_write<HD>(p.out, b, kvh * G + h, e, v.x * inv, v.y * inv);
-      } else {
+      } else if (live) {
         *reinterpret_cast<float2*>(dst + h * (HD + 2) + e) = v;
         if (e == 0) *reinterpret_cast<float2*>(dst + h * (HD + 2) + HD) = make_float2(ml[h], ml[GMAX + h]);
       }
     }
-    if (ns > 1) {  // the last item of this (sequence, kv-head) merges the partials
-      __threadfence();
-      __syncwarp();
-      int last = 0;
-      if (lane == 0) last = atomicAdd(p.work_ctr + WC_DONE + bk, 1) == ns - 1 ? 1 : 0;
-      last = __shfl_sync(0xffffffffu, last, 0);
-      if (last) {
+    if (split) {  // the last item of this (sequence, kv-head) merges the partials
+      int last = 1;
+      if (live) {
         __threadfence();
-        merge_partials<HD>(p.out, p.part + (size_t)bk * p.S * G * (HD + 2), ns, b, kvh, ob, lane);
+        __syncwarp();
+        if (lane == 0) last = atomicAdd(p.work_ctr + WC_DONE + bk, 1) == ns - 1 ? 1 : 0;
+        last = __shfl_sync(0xffffffffu, last, 0);
+      }
+      if (last) {
+        if (live) __threadfence();
+        merge_partials<HD>(p.out, p.part + (size_t)bk * p.S * G * (HD + 2), ns, b, kvh, ob, lane, live);
       }
     }
     __syncwarp();  // the ring and the tables are rewritten by the next item
-    item = __shfl_sync(0xffffffffu, claimed, 0);
+    if (live) item = __shfl_sync(0xffffffffu, claimed, 0);
+    else live = 1;
   }
+  if (!waited) pdl_wait();
 }
 
 // ============================================================================
@@ -1642,13 +1685,12 @@ static void launch_score(const ScoreDev& d, int groups_per_row, cudaStream_t st)
   SOL_LAUNCH("attn_score", (attn_score_kernel<HD, HG>), dim3((unsigned)(units < ctas ? units : ctas)), dim3(SC_WARPS * 32), smem, st, d);
 }
 
-// Persistent: one CTA per SM.
+// Persistent: at most one CTA per SM.
 template <int HD, int GMAX>
-static void launch_gather(const GatherDev& d, long long items, cudaStream_t st) {
+static void launch_gather(const GatherDev& d, long long items, int ctas, cudaStream_t st) {
   using C = GatherCfg<HD, GMAX>;
   ensure_dynamic_smem(reinterpret_cast<const void*>(&attn_gather_kernel<HD, GMAX>), C::SMEM);
-  const long long resident = sm_count();
-  const int grid = (int)(items < resident ? items : resident);
+  const int grid = (int)(items < ctas ? items : ctas);
   SOL_LAUNCH("attn_gather_v", (attn_gather_kernel<HD, GMAX>), dim3(grid), dim3(C::THREADS), C::SMEM, st, d);
 }
 
@@ -1705,7 +1747,7 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   ensure_dynamic_smem(reinterpret_cast<const void*>(&token_select_kernel), (int)sizeof(SelSmem));
   const int sel_ctas = (int)(sel_units < sel_res ? sel_units : sel_res);
   const long long score_ctas = (long long)a.B * Hkv * groups_per_row;
-  // A rehearsal (about 3 us) pays where a CTA is there well before the pass 1 ends: where the CTAs of both leave room for each
+  // A rehearsal (about 3 us) pays where a CTA is there well before pass 1 ends: where the CTAs of both leave room for each
   // other on every SM.  Elsewhere a CTA starts when one of pass 1 ends, and a rehearsal is in its way (16 sequences of 4096
   // tokens: 10.2 us without, 12.9 with it).
   const int rehearse_select = score_ctas + sel_ctas <= 3LL * sm_count();
@@ -1724,12 +1766,17 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   gd.logits = a.logits; gd.sigma = a.sigma; gd.row_ctl = a.row_ctl; gd.work_ctr = a.work_ctr; gd.sms = sm_count();
   gd.part = a.part; gd.scale_log2 = (float)(1.4426950408889634 / sqrt((double)hd)); gd.out = out; gd.status = a.status;
   const long long items = (long long)a.B * Hkv * a.splits;
+  // The selection's CTAs hold their SMs until it ends.  Where they are few, pass 2 leaves those SMs alone: its CTAs are then
+  // there early and have the time for a rehearsal.  Where they are many, a rehearsal delays the items (24 sequences of about
+  // 2000 tokens: 22.8 us without, 25.2 with it).
+  const int gather_ctas = sel_ctas <= sm_count() / 4 ? sm_count() - sel_ctas : sm_count();
+  gd.rehearse = gather_ctas < sm_count();
   if (hd == 64) {
-    if (G <= 4) launch_gather<64, 4>(gd, items, st);
-    else launch_gather<64, 8>(gd, items, st);
+    if (G <= 4) launch_gather<64, 4>(gd, items, gather_ctas, st);
+    else launch_gather<64, 8>(gd, items, gather_ctas, st);
   } else {
-    if (G <= 4) launch_gather<128, 4>(gd, items, st);
-    else launch_gather<128, 8>(gd, items, st);
+    if (G <= 4) launch_gather<128, 4>(gd, items, gather_ctas, st);
+    else launch_gather<128, 8>(gd, items, gather_ctas, st);
   }
 }
 
