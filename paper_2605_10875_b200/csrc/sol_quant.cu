@@ -37,10 +37,26 @@ struct NoSmem {
   int unused;
 };
 
+// Four floats, or zeros where there are none.  Volatile: the loads of a group stay together ahead of their uses (left to
+// itself the compiler takes a few at a time, each with a round trip to L2).
+__device__ __forceinline__ float4 load4_if(const float* p, bool there) {
+  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %5, 0;\n\t"
+      "@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
+      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
+      : "l"(p), "r"((uint32_t)there)
+      : "memory");
+  return v;
+}
+
 // NV: vectors of eight elements per thread (d <= NV * 2048).  Latency-bound: what needs nothing of the kernels before (the
 // gains, the width) is read while they run, unless it is the first kernel of a call, and the code is compiled for the row's
-// length (one code for all lengths: 5.96 us in the chain of a single-sequence step, this 5.74; all nine slices of the
-// partial sums in flight at once: the same).
+// length.  Where it is not the first kernel of a call, the row's code is run once on zeros ahead of the wait (a rehearsal, which
+// reads nothing that an earlier kernel writes and writes nothing), so that it is in the instruction caches.
+// In the chain, per launch: a single sequence 4.9 us, this 3.3; 24 to 32 sequences 7.3 and 5.5; with the input gating 16.5
+// and 12.1.
 template <bool IN_F32, bool GATE, int NV>
 __global__ void __launch_bounds__(NQ_THREADS)
 norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, int ksplit, size_t part_stride,
@@ -64,221 +80,239 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
     gains[i] = make_uint4(0u, 0u, 0u, 0u);
     if (gamma != nullptr && v < d / NQ_VEC) gains[i] = reinterpret_cast<const uint4*>(gamma)[v];
   }
-  int b = bits ? __ldcg(bits + row) : 16;
-  pdl_wait();
-  if (zero_flags != nullptr)
-    for (int i = blockIdx.x * NQ_THREADS + threadIdx.x; i < n_zero_flags; i += gridDim.x * NQ_THREADS) zero_flags[i] = 0;
-  if (clear != nullptr)  // this token's scratch of the kernels that follow
-    for (int i = threadIdx.x; i < clear_words; i += NQ_THREADS) clear[(size_t)row * clear_words + i] = 0u;
-  const int nvec = d / NQ_VEC;
-  float x[NQ_MAX_PER_THREAD][NQ_VEC];
-
-  // load the row (zero-fill vectors beyond d)
-  float ss = 0.f;
-#pragma unroll
-  for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
-    const int v = threadIdx.x + i * NQ_THREADS;
-#pragma unroll
-    for (int e = 0; e < NQ_VEC; ++e) x[i][e] = 0.f;
-    if (v < nvec) {
-      if (IN_F32) {
-        const float4* p = reinterpret_cast<const float4*>(static_cast<const float*>(in) + (size_t)row * d) + 2 * v;
-        float4 a = p[0], b = p[1];
-        x[i][0] = a.x; x[i][1] = a.y; x[i][2] = a.z; x[i][3] = a.w;
-        x[i][4] = b.x; x[i][5] = b.y; x[i][6] = b.z; x[i][7] = b.w;
-      } else {
-        uint4 w = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(in) + (size_t)row * d)[v];
-        x[i][0] = bf16_lo(w.x); x[i][1] = bf16_hi(w.x); x[i][2] = bf16_lo(w.y); x[i][3] = bf16_hi(w.y);
-        x[i][4] = bf16_lo(w.z); x[i][5] = bf16_hi(w.z); x[i][6] = bf16_lo(w.w); x[i][7] = bf16_hi(w.w);
-      }
-      if (part != nullptr) {  // partial sums of the projection that produced this row, in slice order
+  const int width = bits ? __ldcg(bits + row) : 16;
+  int live = first ? 1 : 0;
 #pragma unroll 1
-        for (int z0 = 0; z0 < ksplit; z0 += ZB) {  // ZB slices' loads in flight, added in slice order
-          float4 a[ZB], b[ZB];
+  for (;; live = 1) {
+    asm volatile("" : "+r"(live));  // one code for a rehearsal and the row
+    if (live) pdl_wait();
+    int b = width;
+    if (zero_flags != nullptr && live)
+      for (int i = blockIdx.x * NQ_THREADS + threadIdx.x; i < n_zero_flags; i += gridDim.x * NQ_THREADS) zero_flags[i] = 0;
+    if (clear != nullptr && live)  // this token's scratch of the kernels that follow
+      for (int i = threadIdx.x; i < clear_words; i += NQ_THREADS) clear[(size_t)row * clear_words + i] = 0u;
+    const int nvec = d / NQ_VEC;
+    float x[NQ_MAX_PER_THREAD][NQ_VEC];
+
+    // load the row (zero-fill vectors beyond d)
+    float ss = 0.f;
+#pragma unroll
+    for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
+      const int v = threadIdx.x + i * NQ_THREADS;
+#pragma unroll
+      for (int e = 0; e < NQ_VEC; ++e) x[i][e] = 0.f;
+      if (v < nvec) {
+        float4 a[ZB], b4[ZB];
+        const float* src = part + (size_t)row * d + 8 * v;
+        if (part != nullptr) {  // partial sums of the projection that produced this row: ZB slices' loads in flight
 #pragma unroll
           for (int q = 0; q < ZB; ++q) {
-            a[q] = b[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (z0 + q < ksplit) {
-              const float4* src =
-                  reinterpret_cast<const float4*>(part + (size_t)(z0 + q) * part_stride + (size_t)row * d) + 2 * v;
-              a[q] = src[0];
-              b[q] = src[1];
+            a[q] = load4_if(src + (size_t)q * part_stride, live && q < ksplit);
+            b4[q] = load4_if(src + (size_t)q * part_stride + 4, live && q < ksplit);
+          }
+        }
+        if (IN_F32) {
+          const float* p = static_cast<const float*>(in) + (size_t)row * d + 8 * v;
+          const float4 a0 = load4_if(p, live), b0 = load4_if(p + 4, live);
+          x[i][0] = a0.x; x[i][1] = a0.y; x[i][2] = a0.z; x[i][3] = a0.w;
+          x[i][4] = b0.x; x[i][5] = b0.y; x[i][6] = b0.z; x[i][7] = b0.w;
+        } else {
+          uint4 w = make_uint4(0u, 0u, 0u, 0u);
+          if (live) w = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(in) + (size_t)row * d)[v];
+          x[i][0] = bf16_lo(w.x); x[i][1] = bf16_hi(w.x); x[i][2] = bf16_lo(w.y); x[i][3] = bf16_hi(w.y);
+          x[i][4] = bf16_lo(w.z); x[i][5] = bf16_hi(w.z); x[i][6] = bf16_lo(w.w); x[i][7] = bf16_hi(w.w);
+        }
+        if (GATE && !live) {  // distinct values for the selection
+#pragma unroll
+          for (int e = 0; e < NQ_VEC; ++e) x[i][e] = (float)((8 * v + e) * 389 & 0x1fff);
+        }
+        if (part != nullptr) {  // added in slice order
+#pragma unroll 1
+          for (int z0 = 0;;) {
+#pragma unroll
+            for (int q = 0; q < ZB; ++q) {
+              x[i][0] += a[q].x; x[i][1] += a[q].y; x[i][2] += a[q].z; x[i][3] += a[q].w;
+              x[i][4] += b4[q].x; x[i][5] += b4[q].y; x[i][6] += b4[q].z; x[i][7] += b4[q].w;
+            }
+            z0 += ZB;
+            if (z0 >= ksplit) break;
+#pragma unroll
+            for (int q = 0; q < ZB; ++q) {
+              a[q] = load4_if(src + (size_t)(z0 + q) * part_stride, live && z0 + q < ksplit);
+              b4[q] = load4_if(src + (size_t)(z0 + q) * part_stride + 4, live && z0 + q < ksplit);
             }
           }
-#pragma unroll
-          for (int q = 0; q < ZB; ++q) {
-            x[i][0] += a[q].x; x[i][1] += a[q].y; x[i][2] += a[q].z; x[i][3] += a[q].w;
-            x[i][4] += b[q].x; x[i][5] += b[q].y; x[i][6] += b[q].z; x[i][7] += b[q].w;
-          }
         }
-      }
-      if (sum_out != nullptr) {
-        float4* o = reinterpret_cast<float4*>(sum_out + (size_t)row * d) + 2 * v;
-        o[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
-        o[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
-      }
+        if (sum_out != nullptr && live) {
+          float4* o = reinterpret_cast<float4*>(sum_out + (size_t)row * d) + 2 * v;
+          o[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
+          o[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
+        }
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) ss += x[i][e] * x[i][e];
+        for (int e = 0; e < NQ_VEC; ++e) ss += x[i][e] * x[i][e];
+      }
     }
-  }
 
-  if (gamma != nullptr) {
-    const float tot = block_reduce(ss, false, sh);
-    const float inv = 1.0f / sqrtf(tot / (float)d + eps);
-#pragma unroll
-    for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
-      const int v = threadIdx.x + i * NQ_THREADS;
-      if (v < nvec) {
-        const uint4 w = gains[i];
-        float gm[NQ_VEC] = {bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y),
-                            bf16_lo(w.z), bf16_hi(w.z), bf16_lo(w.w), bf16_hi(w.w)};
-#pragma unroll
-        for (int e = 0; e < NQ_VEC; ++e) x[i][e] = (x[i][e] * gm[e]) * inv;
-      }
-    }
-  }
-
-  if (xn != nullptr) {
-#pragma unroll
-    for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
-      const int v = threadIdx.x + i * NQ_THREADS;
-      if (v < nvec) {
-        float4* p = reinterpret_cast<float4*>(xn + (size_t)row * d) + 2 * v;
-        p[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
-        p[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
-      }
-    }
-  }
-
-  if constexpr (GATE) {
-    // The paper's structured MLP pruning (appendix "Structured MLP activation pruning"): keep the
-    // m = ceil((1 - p) d) channels of largest |x|, ties to the lower index, zero the rest.  |x| orders like its
-    // bit pattern; element j = 8 v + e of the row is slot i * 8 + e of thread v - 256 i.
-    const int m = (int)(((long long)(1000 - gate.p_permille[row]) * d + 999) / 1000);
-    if (m < d) {
-      auto key = [&](int q) -> uint32_t {
-        const int v = threadIdx.x + (q >> 3) * NQ_THREADS;
-        return v < nvec ? __float_as_uint(fabsf(x[q >> 3][q & 7])) : 0u;
-      };
-      int tie_need = 0;
-      uint32_t thr = 0xffffffffu;
-      if (m > 0) thr = select_kth<NQ_THREADS, NQ_MAX_PER_THREAD * NQ_VEC>(key, m, tie_need, gsm, NQ_MAX_PER_THREAD * NQ_VEC);
-      // ties at the threshold are kept in index order until tie_need runs out: index order is (i, thread, e)
-      int taken = 0;  // ties granted to earlier rounds (block-uniform)
-#pragma unroll
-      for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
-        const int v = threadIdx.x + i * NQ_THREADS;
-        uint32_t tie_mask = 0;
-#pragma unroll
-        for (int e = 0; e < NQ_VEC; ++e)
-          if (m > 0 && v < nvec && __float_as_uint(fabsf(x[i][e])) == thr) tie_mask |= 1u << e;
-        // exclusive prefix of the tie counts over the threads of this round
-        const int mine = __popc(tie_mask);
-        int incl = mine;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(0xffffffffu, incl, o);
-          if ((threadIdx.x & 31) >= o) incl += y;
-        }
-        __syncthreads();
-        if ((threadIdx.x & 31) == 31) gsm.scan[0][threadIdx.x >> 5] = incl;
-        __syncthreads();
-        int before = taken + incl - mine, total = 0;
-        for (int wq = 0; wq < NQ_THREADS / 32; ++wq) {
-          const int y = gsm.scan[0][wq];
-          if (wq < (int)(threadIdx.x >> 5)) before += y;
-          total += y;
-        }
-        taken += total;
-#pragma unroll
-        for (int e = 0; e < NQ_VEC; ++e) {
-          const uint32_t kk = __float_as_uint(fabsf(x[i][e]));
-          bool keep = m > 0 && kk > thr;
-          if ((tie_mask >> e) & 1u) {
-            keep = before < tie_need;
-            ++before;
-          }
-          if (!keep) x[i][e] = 0.f;
-        }
-      }
-    }
-    if (gate.xm != nullptr) {
+    if (gamma != nullptr) {
+      const float tot = block_reduce(ss, false, sh);
+      const float inv = 1.0f / sqrtf(tot / (float)d + eps);
 #pragma unroll
       for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
         const int v = threadIdx.x + i * NQ_THREADS;
         if (v < nvec) {
-          float4* p = reinterpret_cast<float4*>(gate.xm + (size_t)row * d) + 2 * v;
+          const uint4 w = gains[i];
+          float gm[NQ_VEC] = {bf16_lo(w.x), bf16_hi(w.x), bf16_lo(w.y), bf16_hi(w.y),
+                              bf16_lo(w.z), bf16_hi(w.z), bf16_lo(w.w), bf16_hi(w.w)};
+#pragma unroll
+          for (int e = 0; e < NQ_VEC; ++e) x[i][e] = (x[i][e] * gm[e]) * inv;
+        }
+      }
+    }
+
+    if (xn != nullptr && live) {
+#pragma unroll
+      for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
+        const int v = threadIdx.x + i * NQ_THREADS;
+        if (v < nvec) {
+          float4* p = reinterpret_cast<float4*>(xn + (size_t)row * d) + 2 * v;
           p[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
           p[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
         }
       }
     }
-  }
 
-  // widths of 9..15 bits need int16 codes, and their codes are no exact bf16 numbers: they are served only where
-  // no tensor-core operand is produced (the stand-alone wide quantizer call)
-  const int b_max = (codes16 != nullptr && a_op == nullptr) ? 15 : 8;
-  if (b != 16 && (b < 2 || b > b_max)) {  // no kernel for this width: pass through and flag it
-    if (threadIdx.x == 0 && status != nullptr) atomicOr(status + ST_ERR, ERR_BAD_ACTION);
-    b = 16;
-  }
-  float s = 1.0f;
-  float q_max = 0.f;
-  if (b != 16) {
-    float a = 0.f;
+    if constexpr (GATE) {
+      // The paper's structured MLP pruning (appendix "Structured MLP activation pruning"): keep the
+      // m = ceil((1 - p) d) channels of largest |x|, ties to the lower index, zero the rest.  |x| orders like its
+      // bit pattern; element j = 8 v + e of the row is slot i * 8 + e of thread v - 256 i.
+      const int m = (int)(((long long)(1000 - gate.p_permille[row]) * d + 999) / 1000);
+      if (m < d) {
+        auto key = [&](int q) -> uint32_t {
+          const int v = threadIdx.x + (q >> 3) * NQ_THREADS;
+          return v < nvec ? __float_as_uint(fabsf(x[q >> 3][q & 7])) : 0u;
+        };
+        int tie_need = 0;
+        uint32_t thr = 0xffffffffu;
+        if (m > 0) thr = select_kth<NQ_THREADS, NQ_MAX_PER_THREAD * NQ_VEC>(key, m, tie_need, gsm, NQ_MAX_PER_THREAD * NQ_VEC);
+        // ties at the threshold are kept in index order until tie_need runs out: index order is (i, thread, e)
+        int taken = 0;  // ties granted to earlier rounds (block-uniform)
 #pragma unroll
-    for (int i = 0; i < NQ_MAX_PER_THREAD; ++i)
+        for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
+          const int v = threadIdx.x + i * NQ_THREADS;
+          uint32_t tie_mask = 0;
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) a = fmaxf(a, fabsf(x[i][e]));
-    a = block_reduce(a, true, sh);
-    q_max = (float)((1 << (b - 1)) - 1);
-    s = __fdiv_rn(a, q_max);
-  }
-  if (threadIdx.x == 0 && scale != nullptr) scale[row] = s;
-
+          for (int e = 0; e < NQ_VEC; ++e)
+            if (m > 0 && v < nvec && __float_as_uint(fabsf(x[i][e])) == thr) tie_mask |= 1u << e;
+          // exclusive prefix of the tie counts over the threads of this round
+          const int mine = __popc(tie_mask);
+          int incl = mine;
 #pragma unroll
-  for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
-    const int v = threadIdx.x + i * NQ_THREADS;
-    if (v >= nvec) continue;
-    float c[NQ_VEC];
-    if (b == 16) {
+          for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if ((threadIdx.x & 31) >= o) incl += y;
+          }
+          __syncthreads();
+          if ((threadIdx.x & 31) == 31) gsm.scan[0][threadIdx.x >> 5] = incl;
+          __syncthreads();
+          int before = taken + incl - mine, total = 0;
+          for (int wq = 0; wq < NQ_THREADS / 32; ++wq) {
+            const int y = gsm.scan[0][wq];
+            if (wq < (int)(threadIdx.x >> 5)) before += y;
+            total += y;
+          }
+          taken += total;
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) c[e] = x[i][e];
-    } else {
+          for (int e = 0; e < NQ_VEC; ++e) {
+            const uint32_t kk = __float_as_uint(fabsf(x[i][e]));
+            bool keep = m > 0 && kk > thr;
+            if ((tie_mask >> e) & 1u) {
+              keep = before < tie_need;
+              ++before;
+            }
+            if (!keep) x[i][e] = 0.f;
+          }
+        }
+      }
+      if (gate.xm != nullptr && live) {
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) {
-        float r = (s == 0.f) ? 0.f : rintf(__fdiv_rn(x[i][e], s));
-        c[e] = fminf(fmaxf(r, -q_max), q_max) + 0.0f;  // +0.0f turns a rounded -0 into +0
+        for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
+          const int v = threadIdx.x + i * NQ_THREADS;
+          if (v < nvec) {
+            float4* p = reinterpret_cast<float4*>(gate.xm + (size_t)row * d) + 2 * v;
+            p[0] = make_float4(x[i][0], x[i][1], x[i][2], x[i][3]);
+            p[1] = make_float4(x[i][4], x[i][5], x[i][6], x[i][7]);
+          }
+        }
       }
     }
-    if (a_op != nullptr) {
-      uint4 w;
-      w.x = pack_bf16(c[0], c[1]); w.y = pack_bf16(c[2], c[3]);
-      w.z = pack_bf16(c[4], c[5]); w.w = pack_bf16(c[6], c[7]);
-      // vector v is the 16-byte piece of elements 8 v .. 8 v + 7: its place in the packed operand layout, or in the plain row
-      if (a_op_rows > 0) *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(a_op) + act_piece_offset(a_op_rows, row, v)) = w;
-      else reinterpret_cast<uint4*>(a_op + (size_t)row * d)[v] = w;
+
+    // widths of 9..15 bits need int16 codes, and their codes are no exact bf16 numbers: they are served only where
+    // no tensor-core operand is produced (the stand-alone wide quantizer call)
+    const int b_max = (codes16 != nullptr && a_op == nullptr) ? 15 : 8;
+    if (b != 16 && (b < 2 || b > b_max)) {  // no kernel for this width: pass through and flag it
+      if (threadIdx.x == 0 && status != nullptr && live) atomicOr(status + ST_ERR, ERR_BAD_ACTION);
+      b = 16;
     }
-    if (codes16 != nullptr) {
-      int q[NQ_VEC];
+    float s = 1.0f;
+    float q_max = 0.f;
+    if (b != 16) {
+      float a = 0.f;
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) q[e] = (b == 16) ? 0 : (int)c[e];
-      uint4 w;
-      w.x = (q[0] & 0xffff) | ((uint32_t)(q[1] & 0xffff) << 16);
-      w.y = (q[2] & 0xffff) | ((uint32_t)(q[3] & 0xffff) << 16);
-      w.z = (q[4] & 0xffff) | ((uint32_t)(q[5] & 0xffff) << 16);
-      w.w = (q[6] & 0xffff) | ((uint32_t)(q[7] & 0xffff) << 16);
-      reinterpret_cast<uint4*>(codes16 + (size_t)row * d)[v] = w;
-    }
-    if (codes != nullptr) {
-      int q[NQ_VEC];
+      for (int i = 0; i < NQ_MAX_PER_THREAD; ++i)
 #pragma unroll
-      for (int e = 0; e < NQ_VEC; ++e) q[e] = (b == 16) ? 0 : (int)c[e];
-      uint2 w;
-      w.x = (q[0] & 0xff) | ((q[1] & 0xff) << 8) | ((q[2] & 0xff) << 16) | ((uint32_t)(q[3] & 0xff) << 24);
-      w.y = (q[4] & 0xff) | ((q[5] & 0xff) << 8) | ((q[6] & 0xff) << 16) | ((uint32_t)(q[7] & 0xff) << 24);
-      reinterpret_cast<uint2*>(codes + (size_t)row * d)[v] = w;
+        for (int e = 0; e < NQ_VEC; ++e) a = fmaxf(a, fabsf(x[i][e]));
+      a = block_reduce(a, true, sh);
+      q_max = (float)((1 << (b - 1)) - 1);
+      s = __fdiv_rn(a, q_max);
     }
+    if (threadIdx.x == 0 && scale != nullptr && live) scale[row] = s;
+
+#pragma unroll
+    for (int i = 0; i < NQ_MAX_PER_THREAD; ++i) {
+      const int v = threadIdx.x + i * NQ_THREADS;
+      if (v >= nvec) continue;
+      float c[NQ_VEC];
+      if (b == 16) {
+#pragma unroll
+        for (int e = 0; e < NQ_VEC; ++e) c[e] = x[i][e];
+      } else {
+#pragma unroll
+        for (int e = 0; e < NQ_VEC; ++e) {
+          float r = (s == 0.f) ? 0.f : rintf(__fdiv_rn(x[i][e], s));
+          c[e] = fminf(fmaxf(r, -q_max), q_max) + 0.0f;  // +0.0f turns a rounded -0 into +0
+        }
+      }
+      if (a_op != nullptr && live) {
+        uint4 w;
+        w.x = pack_bf16(c[0], c[1]); w.y = pack_bf16(c[2], c[3]);
+        w.z = pack_bf16(c[4], c[5]); w.w = pack_bf16(c[6], c[7]);
+        // vector v is the 16-byte piece of elements 8 v .. 8 v + 7: its place in the packed operand layout, or in the plain row
+        if (a_op_rows > 0) *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(a_op) + act_piece_offset(a_op_rows, row, v)) = w;
+        else reinterpret_cast<uint4*>(a_op + (size_t)row * d)[v] = w;
+      }
+      if (codes16 != nullptr && live) {
+        int q[NQ_VEC];
+#pragma unroll
+        for (int e = 0; e < NQ_VEC; ++e) q[e] = (b == 16) ? 0 : (int)c[e];
+        uint4 w;
+        w.x = (q[0] & 0xffff) | ((uint32_t)(q[1] & 0xffff) << 16);
+        w.y = (q[2] & 0xffff) | ((uint32_t)(q[3] & 0xffff) << 16);
+        w.z = (q[4] & 0xffff) | ((uint32_t)(q[5] & 0xffff) << 16);
+        w.w = (q[6] & 0xffff) | ((uint32_t)(q[7] & 0xffff) << 16);
+        reinterpret_cast<uint4*>(codes16 + (size_t)row * d)[v] = w;
+      }
+      if (codes != nullptr && live) {
+        int q[NQ_VEC];
+#pragma unroll
+        for (int e = 0; e < NQ_VEC; ++e) q[e] = (b == 16) ? 0 : (int)c[e];
+        uint2 w;
+        w.x = (q[0] & 0xff) | ((q[1] & 0xff) << 8) | ((q[2] & 0xff) << 16) | ((uint32_t)(q[3] & 0xff) << 24);
+        w.y = (q[4] & 0xff) | ((q[5] & 0xff) << 8) | ((q[6] & 0xff) << 16) | ((uint32_t)(q[7] & 0xff) << 24);
+        reinterpret_cast<uint2*>(codes + (size_t)row * d)[v] = w;
+      }
+    }
+    if (live) return;
+    if (GATE) __syncthreads();  // the rehearsal's selection is not read any more
   }
 }
 
