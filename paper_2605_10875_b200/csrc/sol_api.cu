@@ -279,7 +279,6 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
   cs.cand_val = at<double>(ws, L.ch_cand_val);
   cs.cand_idx = at<int32_t>(ws, L.ch_cand_idx);
   cs.keep = at<unsigned char>(ws, L.ch_keep);
-  cs.scratch_idx = at<int32_t>(ws, L.kept_ch);
   cs.kept_ch = kept_ch;
   cs.kept_cnt = kept_ch_cnt ? kept_ch_cnt : at<int32_t>(ws, L.kept_ch_cnt);
   cs.t_op = at<void>(ws, L.t_hi);

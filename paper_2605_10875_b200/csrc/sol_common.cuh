@@ -126,7 +126,7 @@ __device__ __forceinline__ float chan_bin_lo(int b) {  // smallest value of bin 
 }
 // Per-token scratch words of the channel selection, cleared by the RMSNorm kernel before the projection:
 // the histogram, then these.
-enum : int { CH_GMAX = CH_BINS, CH_UMAX, CH_N_ABOVE, CH_N_CAND, CH_DONE, CH_FALLBACK, CH_SEL_WORDS = CH_BINS + 8 };
+enum : int { CH_GMAX = CH_BINS, CH_UMAX, CH_N_ABOVE, CH_N_CAND, CH_DONE, CH_FALLBACK, CH_OPEN, CH_DONE_OPEN, CH_SEL_WORDS = CH_BINS + 8 };
 constexpr int CH_CAND_CAP = 1024;  // exactly re-scored candidates per token before the single-CTA path takes over
 
 // ---- programmatic dependent launch ---------------------------------------------

@@ -353,7 +353,6 @@ struct ChannelSelectArgs {
   double* cand_val;    // [B][CH_CAND_CAP]
   int32_t* cand_idx;   // [B][CH_CAND_CAP]
   unsigned char* keep; // [B][ff] 1 = kept
-  int32_t* scratch_idx; // [B][ff] scratch of the single-CTA path
   int32_t* kept_ch;    // optional [B][ff]: ascending list, written only when requested
   int32_t* kept_cnt;   // [B]
   void* t_op;          // packed operand of the down projection: 2 pad_rows(B) rows (bf16 high parts, then low parts)

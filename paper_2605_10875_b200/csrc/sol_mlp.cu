@@ -9,13 +9,14 @@
 // ff/1024 CTAs: each finds the histogram bin that holds the m-th largest |t|,
 // keeps what lies above that bin (by more than the float32 error bound of t),
 // drops what lies below, and lists the channels in between; the last CTA of a
-// token ranks those candidates within their error bounds, recomputes the few
-// that the bounds leave open exactly from the weight rows, and patches the
-// kept ones in.  Outputs: the masked activations as two bf16
+// token ranks those candidates within their error bounds and patches the
+// surely kept ones in; the few that the bounds leave open are recomputed
+// exactly from the weight rows (many of a small batch by channel_select_rest,
+// whose CTAs share them).  Outputs: the masked activations as two bf16
 // parts (hi + lo) for the tensor-core down projection, a keep mask, and the
 // "granule is live" flags that let the down projection skip weight rows
 // nobody keeps.  A token with more candidates than the list holds (massive
-// ties) is redone by the single-CTA kernel channel_select, which is exact for
+// ties) is redone by one CTA of channel_select_rest, which is exact for
 // any input; channel_list turns the mask into the ascending index list when a
 // caller asks for it.
 #include <math.h>
@@ -41,11 +42,11 @@ struct ChanDev {
   int32_t* cand_idx;
   unsigned char* keep;
   int32_t* kept_ch;
-  int32_t* scratch_idx;  // [B][ff] list written by the single-CTA kernel (not an output)
   int32_t* kept_cnt;
   unsigned char* t_op;  // packed operand of the down projection: 2 Mpad rows (high parts, then low parts)
   int32_t* live;
   int* status;
+  int hand_over;        // elements of open candidates above which the next kernel recomputes them; 0: never
 };
 
 // Running sum held as an unevaluated pair of floats (hi + lo): adds x with the rounding error of
@@ -58,215 +59,6 @@ __device__ __forceinline__ void pair_add(float& hi, float& lo, float x) {
   hi = s;
   lo = __fadd_rn(lo, e);
 }
-
-template <int THREADS, int KPT>
-__global__ void __launch_bounds__(THREADS) channel_select_kernel(const ChanDev p) {
-  __shared__ SelectSmem sm;
-  static_assert(KPT % 8 == 0 && KPT <= 64, "a thread owns whole 16-byte groups of bf16 outputs");
-  const int b = blockIdx.x;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  constexpr int WARPS = THREADS / 32;
-  const int ff = p.ff, d = p.d;
-  pdl_trigger();
-  pdl_wait();
-  if (p.sel[(size_t)b * CH_SEL_WORDS + CH_FALLBACK] == 0u) return;  // the multi-CTA kernel settled this token
-  const float* tt = p.t + (size_t)b * ff;
-  const int m = (int)(((long long)(1000 - p.p_permille[b]) * ff + 999) / 1000);
-  const int j0 = tid * KPT;
-  if (tid < 4) sm.counts[tid] = 0;
-
-  // one pass over global memory: |t| as keys (0: absent) and signs in registers, and (when a selection
-  // is needed) the largest |g|, |u| for the error window
-  const bool select = m < ff && m > 0;
-  uint32_t key[KPT];
-  uint64_t neg = 0;
-  float gmax = 0.f, umax = 0.f;
-  {
-    const float* gg = p.g + (size_t)b * ff;
-    const float* uu = p.u + (size_t)b * ff;
-#pragma unroll
-    for (int i = 0; i < KPT; i += 4) {
-      float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-      const bool in = j0 + i < ff;  // ff is a multiple of 4, so a group is present or absent as a whole
-      if (in) v = *reinterpret_cast<const float4*>(tt + j0 + i);
-      const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        key[i + e] = in ? float_key(fabsf(vv[e])) : 0u;
-        if (vv[e] < 0.f) neg |= 1ull << (i + e);
-      }
-      if (select && in) {
-        const float4 g4 = *reinterpret_cast<const float4*>(gg + j0 + i), u4 = *reinterpret_cast<const float4*>(uu + j0 + i);
-        gmax = fmaxf(fmaxf(gmax, fmaxf(fabsf(g4.x), fabsf(g4.y))), fmaxf(fabsf(g4.z), fabsf(g4.w)));
-        umax = fmaxf(fmaxf(umax, fmaxf(fabsf(u4.x), fabsf(u4.y))), fmaxf(fabsf(u4.z), fabsf(u4.w)));
-      }
-    }
-  }
-
-  // mode 0: keep all; 1: keep none; 2: kept iff |t| above the window or a candidate decided in float64;
-  // 3: float32 order with index-ordered ties (candidate list overflowed)
-  int mode, tie_need = 0, n_cand = 0;
-  uint32_t key_thr = 0;
-  float hi = 0.f, lo = 0.f;
-
-  if (m >= ff) {
-    mode = 0;
-  } else if (m <= 0) {
-    mode = 1;
-  } else {
-    gmax = block_max<THREADS>(gmax, 0, sm);
-    umax = block_max<THREADS>(umax, 1, sm);
-    key_thr = select_kth<THREADS, KPT>([&](int i) { return key[i]; }, m, tie_need, sm, KPT);
-    mode = 3;
-    const float thr32 = key_to_float(key_thr);
-    // error taken for g_j, u_j: the tensor cores add each 16-long slice of the dot product to the running
-    // float32 sum with truncation, so the error grows with the d/16 steps: (d/16) * 2^-24 of the largest
-    // magnitude, and never less than 2^-18 of it
-    const float eps = fmaxf(3.814697265625e-06f, (float)(d / 16) * 5.9604644775390625e-08f) * fmaxf(gmax, umax);
-    const float delta = 2.0f * eps * (1.1f * umax + gmax) + 1e-6f * thr32;  // |silu'| <= 1.1, |silu(g)| <= |g|
-    hi = thr32 + delta;
-    lo = thr32 - delta;
-    int n_in = 0;
-#pragma unroll
-    for (int i = 0; i < KPT; ++i) {
-      if (key[i] == 0u) continue;
-      const float sv = key_to_float(key[i]);
-      if (sv > hi) {
-        ++n_in;
-      } else if (sv >= lo) {
-        const int slot = atomicAdd(&sm.counts[0], 1);
-        if (slot < SEL_CAND_CAP) sm.cand_idx[slot] = j0 + i;
-      }
-    }
-    n_in = block_count<THREADS>(n_in, 0, sm);
-    n_cand = sm.counts[0];
-    const int need = m - n_in;
-    if (n_cand > SEL_CAND_CAP) {
-      if (tid == 0) atomicAdd(p.status + ST_CH_OVERFLOW, 1);
-      n_cand = 0;
-    } else {
-      if (n_cand != need) {
-        if (tid == 0) atomicAdd(p.status + ST_CH_REFINED, n_cand);
-        // g_j = scale * sum_e x_e w_je with x the quantizer codes (or the bf16 row): every product of two
-        // bf16 numbers is an exact float32, so the sums are gathered exactly in float pairs
-        const double sc = (double)p.scale[b];
-        for (int c = warp; c < n_cand; c += WARPS) {
-          const int j = sm.cand_idx[c];
-          float gh = 0.f, gl = 0.f, uh = 0.f, ul = 0.f;
-          // RB 256-wide slices per round, all loads of a round issued before the first use
-          constexpr int RB = THREADS >= 1024 ? 2 : 4;  // 64 registers per thread at 1024 threads
-          for (int e0 = lane * 8; e0 < d; e0 += RB * 256) {
-            uint4 xv[RB], gv[RB], uv[RB];
-#pragma unroll
-            for (int r = 0; r < RB; ++r) {
-              const int e = e0 + r * 256;
-              if (e < d) {  // the piece of elements e .. e + 7 of the operand row and of the channel's two weight rows
-                xv[r] = *reinterpret_cast<const uint4*>(p.a_op + act_piece_offset(p.Mpad, b, e >> 3));
-                gv[r] = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j, e >> 6, (e >> 3) & 7));
-                uv[r] = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j + 1, e >> 6, (e >> 3) & 7));
-              }
-            }
-#pragma unroll
-            for (int r = 0; r < RB; ++r) {
-              if (e0 + r * 256 >= d) break;
-              const uint32_t xa[4] = {xv[r].x, xv[r].y, xv[r].z, xv[r].w}, ga[4] = {gv[r].x, gv[r].y, gv[r].z, gv[r].w},
-                             ua[4] = {uv[r].x, uv[r].y, uv[r].z, uv[r].w};
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const float x0 = bf16_lo(xa[q]), x1 = bf16_hi(xa[q]);
-                pair_add(gh, gl, __fmul_rn(x0, bf16_lo(ga[q])));
-                pair_add(gh, gl, __fmul_rn(x1, bf16_hi(ga[q])));
-                pair_add(uh, ul, __fmul_rn(x0, bf16_lo(ua[q])));
-                pair_add(uh, ul, __fmul_rn(x1, bf16_hi(ua[q])));
-              }
-            }
-          }
-          const double ag = warp_sum_d((double)gh + (double)gl) * sc;
-          const double au = warp_sum_d((double)uh + (double)ul) * sc;
-          if (lane == 0) sm.cand_val[c] = fabs(ag / (1.0 + exp(-ag)) * au);
-        }
-        __syncthreads();
-        rank_candidates<THREADS>(n_cand, need, sm);
-      } else {
-        for (int c = tid; c < n_cand; c += THREADS) sm.cand_keep[c] = 1;
-      }
-      mode = 2;
-      __syncthreads();
-    }
-  }
-
-  auto klass = [&](int i) -> int {
-    const int j = j0 + i;
-    if (j >= ff || mode == 1) return 0;
-    if (mode == 0) return 2;
-    if (mode == 2) {
-      const float sv = key_to_float(key[i]);
-      if (sv > hi) return 2;
-      if (sv >= lo) {  // within the window: look the channel up in the decided list
-        for (int q = 0; q < n_cand; ++q)
-          if (sm.cand_idx[q] == j) return sm.cand_keep[q] ? 2 : 0;
-      }
-      return 0;
-    }
-    return key[i] > key_thr ? 2 : (key[i] == key_thr ? 1 : 0);
-  };
-  // masked activations as bf16 high + low parts, 8 channels (16 bytes) at a time, and the live flags
-  uint32_t hw[4], lw[4];
-  bool any = false;
-  auto emit = [&](int i, bool keep, int) {
-    uint16_t hv = 0, lv = 0;
-    if (keep) {
-      const float a = key_to_float(key[i]);
-      const float v = ((neg >> i) & 1ull) ? -a : a;
-      hv = f2bf(v);
-      lv = f2bf(v - bf2f(hv));
-      any = true;
-    }
-    const int e = i & 7;
-    if ((e & 1) == 0) {
-      hw[e >> 1] = hv;
-      lw[e >> 1] = lv;
-    } else {
-      hw[e >> 1] |= (uint32_t)hv << 16;
-      lw[e >> 1] |= (uint32_t)lv << 16;
-    }
-    if (j0 + i < ff) p.keep[(size_t)b * ff + j0 + i] = keep ? 1 : 0;
-    if (e == 7 && j0 + i < ff) {  // channels j0 + i - 7 .. j0 + i are one piece of the packed operand
-      unsigned char* dst = p.t_op + act_piece_offset(2 * p.Mpad, b, (j0 + i) >> 3);
-      *reinterpret_cast<uint4*>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-      *reinterpret_cast<uint4*>(dst + (size_t)p.Mpad * 128) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
-    }
-    if (((j0 + i) & 31) == 31 || i == KPT - 1) {  // end of a 32-channel granule or of this thread's range
-      if (any && j0 + i < ff) p.live[(j0 + i) >> 5] = 1;
-      any = false;
-    }
-  };
-  // the index list itself is written by channel_list from the mask; here it goes to the candidate scratch
-  const int total =
-      compact_indices<THREADS, KPT>(klass, emit, mode == 3 ? tie_need : 0, p.scratch_idx + (size_t)b * ff, sm, KPT);
-  if (tid == 0) p.kept_cnt[b] = total;
-}
-
-// ============================================================================
-// channel_select_multi
-// ============================================================================
-constexpr int CM_THREADS = 256;
-
-constexpr int CM_EXACT = 32;
-struct ChanMultiSmem {
-  int scan[CM_THREADS / 32];
-  int pick;
-  int n_open;
-  int flag;
-  float thr_hi, thr_lo;
-  int idx[CH_CAND_CAP];
-  float2 av[CH_CAND_CAP];          // a candidate's float32 |t| and the bound of its error
-  double val[CH_CAND_CAP];         // its exact |t|; +-1e300 where the bounds settle it
-  int open[CH_CAND_CAP];           // the candidates to recompute
-  size_t row_off[CM_EXACT];        // of up to CM_EXACT of them: where their weight rows start, the rows' swizzle,
-  int row_swz[CM_EXACT];
-  double2 part[CM_EXACT][CM_THREADS / 32];  // the warps' sums of g and u
-};
 
 // bf16 numbers as float64 by their bits (a conversion instruction runs at a small fraction of this rate).
 // Operand elements, the number in the high half of a word: exact, whatever the number.
@@ -281,6 +73,313 @@ __device__ __forceinline__ double operand_to_f64(uint32_t high_half) {
 __device__ __forceinline__ double weight_to_f64(uint32_t high_half) {
   return __hiloint2double((int)(((high_half >> 3) & 0x0fffe000u) | (high_half & 0x80000000u)), 0);
 }
+
+// From the exact sums of a candidate's gate and up products (weights times 2^-896, see weight_to_f64) to its exact |t|.
+__device__ __forceinline__ double exact_score(double g, double u, double scale) {
+  const double unit = __hiloint2double((1023 + 896) << 20, 0);  // 2^896
+  const double ag = g * unit * scale, au = u * unit * scale;
+  return fabs(ag / (1.0 + exp(-ag)) * au);
+}
+// Patches a kept candidate into the masked activations, the mask and the live flags.
+__device__ __forceinline__ void keep_channel(const ChanDev& p, int b, int j) {
+  const float tv = p.t[(size_t)b * p.ff + j];
+  const uint16_t hv = f2bf(tv);
+  uint16_t* dst = reinterpret_cast<uint16_t*>(p.t_op + act_piece_offset(2 * p.Mpad, b, j >> 3) + (j & 7) * 2);
+  dst[0] = hv;
+  dst[(size_t)p.Mpad * 64] = f2bf(tv - bf2f(hv));
+  p.keep[(size_t)b * p.ff + j] = 1;
+  p.live[j >> 5] = 1;
+}
+
+// ============================================================================
+// channel_select_rest: what channel_select_multi leaves to it
+// ============================================================================
+constexpr int CR_THREADS = 512;
+
+// The open candidates of a token: their exact |t| in float64 (g_j = scale * sum_e x_e w_je with x the quantizer codes or the
+// bf16 row), shared out over the token's CTAs; the last of them keeps the `need` best (ties: lower index).  Four warps per
+// candidate, eight elements of both rows per thread and step, the next step's on their way.
+// live == 0: a rehearsal on one made-up candidate, which reads weights only and writes nothing outside the CTA.
+__device__ __forceinline__ void settle_open(const ChanDev& p, SelectSmem& sm, int b, int n_open, int need, int live) {
+  constexpr int GROUPS = CR_THREADS / 128;
+  __shared__ double2 part[GROUPS][4];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, group = tid >> 7, gt = tid & 127, lane = tid & 31, d = p.d, X = gridDim.x;
+  const uint32_t chunk_bytes = (uint32_t)p.R * 128;
+  const int32_t* idx = p.cand_idx + (size_t)b * CH_CAND_CAP;
+  double* val = p.cand_val + (size_t)b * CH_CAND_CAP;
+#pragma unroll 1
+  for (int i0 = live ? blockIdx.x * GROUPS : 0; i0 < n_open; i0 += GROUPS * X) {
+    const int i = i0 + group;
+    double g = 0.0, u = 0.0;
+    if (i < n_open) {
+      const int n = live ? 2 * __ldcg(idx + i) : 0, tile = n / p.R, r = n - tile * p.R;
+      const unsigned char* row = p.w_gu + ((size_t)tile * p.chunks * p.R + r) * 128;  // the gate row; the up row follows
+      const int swz = r & 7;                                                          // even: a gate row is an even row
+      uint4 gn = make_uint4(0u, 0u, 0u, 0u), un = gn, xn = gn;
+      auto load = [&](int e0) {
+        if (e0 < d) {
+          const int piece = (e0 >> 3) & 7;
+          const unsigned char* src = row + (size_t)(e0 >> 6) * chunk_bytes;
+          gn = *reinterpret_cast<const uint4*>(src + ((piece ^ swz) * 16));
+          un = *reinterpret_cast<const uint4*>(src + 128 + ((piece ^ (swz + 1)) * 16));
+          if (live) xn = *reinterpret_cast<const uint4*>(p.a_op + act_piece_offset(p.Mpad, b, e0 >> 3));
+        }
+      };
+      load(gt * 8);
+#pragma unroll 1
+      for (int e0 = gt * 8; e0 < d; e0 += 1024) {
+        const uint32_t ga[4] = {gn.x, gn.y, gn.z, gn.w}, ua[4] = {un.x, un.y, un.z, un.w}, xa[4] = {xn.x, xn.y, xn.z, xn.w};
+        load(e0 + 1024);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const double x0 = operand_to_f64(xa[e] << 16), x1 = operand_to_f64(xa[e]);
+          g = fma(x0, weight_to_f64(ga[e] << 16), g);
+          u = fma(x0, weight_to_f64(ua[e] << 16), u);
+          g = fma(x1, weight_to_f64(ga[e]), g);
+          u = fma(x1, weight_to_f64(ua[e]), u);
+        }
+      }
+    }
+    g = warp_sum_d(g);
+    u = warp_sum_d(u);
+    if (lane == 0) part[group][gt >> 5] = make_double2(g, u);
+    __syncthreads();
+    if (gt == 0 && i < n_open) {
+      const double2 a = part[group][0], b2 = part[group][1], c = part[group][2], e = part[group][3];
+      const double v = exact_score((a.x + b2.x) + (c.x + e.x), (a.y + b2.y) + (c.y + e.y), live ? (double)p.scale[b] : 1.0);
+      if (live) val[i] = v;
+    }
+    __syncthreads();
+  }
+  if (live && X > 1) {  // the token's last CTA goes on
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) s_last = atomicAdd(p.sel + (size_t)b * CH_SEL_WORDS + CH_DONE_OPEN, 1u) == (uint32_t)(X - 1) ? 1 : 0;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+  }
+  for (int c = tid; c < n_open; c += CR_THREADS) {
+    sm.cand_val[c] = live ? __ldcg(val + c) : 0.0;
+    sm.cand_idx[c] = live ? __ldcg(idx + c) : c;
+  }
+  __syncthreads();
+  rank_candidates<CR_THREADS>(n_open, need, sm);
+  for (int c = tid; c < n_open; c += CR_THREADS)
+    if (live && sm.cand_keep[c]) keep_channel(p, b, sm.cand_idx[c]);
+  if (live && tid == 0) atomicAdd(p.status + ST_CH_REFINED, n_open);
+}
+
+// A token whose candidates did not fit the list (long runs of equal scores), from the beginning and for any input, by one
+// CTA: the m-th largest |t| by a radix select, the channels within the error bound of it by their exact scores, or, where
+// those do not fit the list either, in float32 order with ties to the lower index.  Rare, so its loops over the row
+// are short and read it from L2 each time.
+__device__ __noinline__ void redo_token(const ChanDev& p, SelectSmem& sm, int b) {
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  constexpr int WARPS = CR_THREADS / 32;
+  const int ff = p.ff, d = p.d;
+  const float* tt = p.t + (size_t)b * ff;
+  const int m = (int)(((long long)(1000 - p.p_permille[b]) * ff + 999) / 1000);
+  if (tid < 4) sm.counts[tid] = 0;
+  float gmax = 0.f, umax = 0.f;  // for the error window
+#pragma unroll 1
+  for (int j = tid; j < ff; j += CR_THREADS) {
+    gmax = fmaxf(gmax, fabsf(p.g[(size_t)b * ff + j]));
+    umax = fmaxf(umax, fabsf(p.u[(size_t)b * ff + j]));
+  }
+  gmax = block_max<CR_THREADS>(gmax, 0, sm);
+  umax = block_max<CR_THREADS>(umax, 1, sm);
+  int tie_need = 0;
+  auto key = [&](int i) -> uint32_t {
+    const int j = i * CR_THREADS + tid;
+    return j < ff ? float_key(fabsf(tt[j])) : 0u;
+  };
+  const uint32_t key_thr = select_kth<CR_THREADS, 0>(key, m, tie_need, sm, (ff + CR_THREADS - 1) / CR_THREADS);
+  const float thr32 = key_to_float(key_thr);
+  // error taken for g_j, u_j: the tensor cores add each 16-long slice of the dot product to the running
+  // float32 sum with truncation, so the error grows with the d/16 steps: (d/16) * 2^-24 of the largest
+  // magnitude, and never less than 2^-18 of it
+  const float eps = fmaxf(3.814697265625e-06f, (float)(d / 16) * 5.9604644775390625e-08f) * fmaxf(gmax, umax);
+  const float delta = 2.0f * eps * (1.1f * umax + gmax) + 1e-6f * thr32;  // |silu'| <= 1.1, |silu(g)| <= |g|
+  const float hi = thr32 + delta, lo = thr32 - delta;
+  int n_in = 0;
+#pragma unroll 1
+  for (int j = tid; j < ff; j += CR_THREADS) {
+    const float sv = key_to_float(float_key(fabsf(tt[j])));
+    if (sv > hi) {
+      ++n_in;
+    } else if (sv >= lo) {
+      const int slot = atomicAdd(&sm.counts[0], 1);
+      if (slot < SEL_CAND_CAP) sm.cand_idx[slot] = j;
+    }
+  }
+  n_in = block_count<CR_THREADS>(n_in, 0, sm);
+  int n_cand = sm.counts[0];
+  const int need = m - n_in;
+  const bool by_window = n_cand <= SEL_CAND_CAP;  // else float32 order
+  if (!by_window) {
+    if (tid == 0) atomicAdd(p.status + ST_CH_OVERFLOW, 1);
+    n_cand = 0;
+  } else if (n_cand != need) {
+    if (tid == 0) atomicAdd(p.status + ST_CH_REFINED, n_cand);
+    // every product of two bf16 numbers is an exact float32, so the sums are gathered exactly in float pairs
+    const double sc = (double)p.scale[b];
+#pragma unroll 1
+    for (int c = warp; c < n_cand; c += WARPS) {
+      const int j = sm.cand_idx[c];
+      float gh = 0.f, gl = 0.f, uh = 0.f, ul = 0.f;
+#pragma unroll 1
+      for (int e = lane * 8; e < d; e += 256) {  // the piece of elements e .. e + 7 of the operand row and of the channel's rows
+        const uint4 xv = *reinterpret_cast<const uint4*>(p.a_op + act_piece_offset(p.Mpad, b, e >> 3));
+        const uint4 gv = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j, e >> 6, (e >> 3) & 7));
+        const uint4 uv = *reinterpret_cast<const uint4*>(p.w_gu + nk_piece_offset(p.R, p.chunks, 2 * j + 1, e >> 6, (e >> 3) & 7));
+        const uint32_t xa[4] = {xv.x, xv.y, xv.z, xv.w}, ga[4] = {gv.x, gv.y, gv.z, gv.w}, ua[4] = {uv.x, uv.y, uv.z, uv.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float x0 = bf16_lo(xa[q]), x1 = bf16_hi(xa[q]);
+          pair_add(gh, gl, __fmul_rn(x0, bf16_lo(ga[q])));
+          pair_add(gh, gl, __fmul_rn(x1, bf16_hi(ga[q])));
+          pair_add(uh, ul, __fmul_rn(x0, bf16_lo(ua[q])));
+          pair_add(uh, ul, __fmul_rn(x1, bf16_hi(ua[q])));
+        }
+      }
+      const double ag = warp_sum_d((double)gh + (double)gl) * sc;
+      const double au = warp_sum_d((double)uh + (double)ul) * sc;
+      if (lane == 0) sm.cand_val[c] = fabs(ag / (1.0 + exp(-ag)) * au);
+    }
+    __syncthreads();
+    rank_candidates<CR_THREADS>(n_cand, need, sm);
+  } else {
+    for (int c = tid; c < n_cand; c += CR_THREADS) sm.cand_keep[c] = 1;
+  }
+  __syncthreads();
+
+  // the masked activations as bf16 high and low parts, eight channels (one piece of the packed operand) per thread and round,
+  // in index order: ties are kept until tie_need runs out
+  int total = 0, ties_taken = 0;
+#pragma unroll 1
+  for (int base0 = 0; base0 < ff; base0 += CR_THREADS * 8) {
+    const int j0 = base0 + tid * 8;  // ff is a multiple of 32, so eight are present or absent as a whole
+    float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (j0 < ff) {
+      const float4 v0 = *reinterpret_cast<const float4*>(tt + j0), v1 = *reinterpret_cast<const float4*>(tt + j0 + 4);
+      v[0] = v0.x; v[1] = v0.y; v[2] = v0.z; v[3] = v0.w; v[4] = v1.x; v[5] = v1.y; v[6] = v1.z; v[7] = v1.w;
+    }
+    uint32_t keep = 0, tie = 0;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const uint32_t kk = float_key(fabsf(v[e]));
+      if (j0 >= ff) continue;
+      if (by_window) {
+        const float sv = key_to_float(kk);
+        if (sv > hi) {
+          keep |= 1u << e;
+        } else if (sv >= lo) {  // within the window: look the channel up in the decided list
+          for (int q = 0; q < n_cand; ++q)
+            if (sm.cand_idx[q] == j0 + e && sm.cand_keep[q]) keep |= 1u << e;
+        }
+      } else {
+        if (kk > key_thr) keep |= 1u << e;
+        if (kk == key_thr) tie |= 1u << e;
+      }
+    }
+    int incl = __popc(tie);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    __syncthreads();  // earlier readers of sm.scan are done
+    if (lane == 31) sm.scan[0][warp] = incl;
+    __syncthreads();
+    int before = ties_taken + incl - __popc(tie);
+    for (int w = 0; w < WARPS; ++w) {
+      const int x = sm.scan[0][w];
+      if (w < warp) before += x;
+      ties_taken += x;
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e)
+      if ((tie >> e) & 1u) {
+        if (before < tie_need) keep |= 1u << e;
+        ++before;
+      }
+    if (j0 < ff) {
+      uint32_t hw[4] = {0, 0, 0, 0}, lw[4] = {0, 0, 0, 0}, kw[2] = {0, 0};
+#pragma unroll
+      for (int e = 0; e < 8; ++e)
+        if ((keep >> e) & 1u) {
+          const uint16_t hv = f2bf(v[e]), lv = f2bf(v[e] - bf2f(hv));
+          hw[e >> 1] |= (uint32_t)hv << (16 * (e & 1));
+          lw[e >> 1] |= (uint32_t)lv << (16 * (e & 1));
+          kw[e >> 2] |= 1u << (8 * (e & 3));
+        }
+      unsigned char* dst = p.t_op + act_piece_offset(2 * p.Mpad, b, j0 >> 3);
+      *reinterpret_cast<uint4*>(dst) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+      *reinterpret_cast<uint4*>(dst + (size_t)p.Mpad * 128) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+      *reinterpret_cast<uint2*>(p.keep + (size_t)b * ff + j0) = make_uint2(kw[0], kw[1]);
+      if (keep) p.live[j0 >> 5] = 1;
+    }
+    total += __popc(keep);
+  }
+  total = block_count<CR_THREADS>(total, 1, sm);
+  if (tid == 0) p.kept_cnt[b] = total;
+}
+
+// Grid (CTAs per token, tokens).  Nearly always most CTAs leave at once, so the kernel is kept small enough to be resident
+// beside any other (as a kernel of 124 registers and 100 KB of unrolled code it took 1.7 us of a single sequence's layer,
+// this 0.7).  Where open candidates may be handed over, a CTA of a token with a selection to make rehearses settle_open
+// while the kernels before are still running, so that its code is in the instruction caches.
+__global__ void __launch_bounds__(CR_THREADS, 2) channel_select_rest_kernel(const ChanDev p) {
+  __shared__ SelectSmem sm;
+  const int b = blockIdx.y;
+  pdl_trigger();
+  const int m = (int)(((long long)(1000 - p.p_permille[b]) * p.ff + 999) / 1000);
+  if (m <= 0 || m >= p.ff) {  // all or nothing: never left to this kernel
+    pdl_wait();
+    return;
+  }
+  int live = 0, n_open = p.hand_over > 0 ? 1 : 0, need = 1;
+#pragma unroll 1
+  for (;;) {
+    asm volatile("" : "+r"(live));  // one code for both
+    if (n_open > 0) settle_open(p, sm, b, n_open, need, live);
+    if (live) return;
+    pdl_wait();
+    const uint32_t* sel = p.sel + (size_t)b * CH_SEL_WORDS;
+    if (__ldcg(sel + CH_FALLBACK) != 0u) {
+      if (blockIdx.x == 0) redo_token(p, sm, b);
+      return;
+    }
+    const uint32_t open = __ldcg(sel + CH_OPEN);
+    n_open = (int)(open >> 16);
+    need = (int)(open & 0xffffu);
+    live = 1;
+    __syncthreads();  // the rehearsal's candidate is not read any more
+  }
+}
+
+// ============================================================================
+// channel_select_multi
+// ============================================================================
+constexpr int CM_THREADS = 256;
+
+constexpr int CM_EXACT = 32;  // candidates recomputed at a time
+struct ChanMultiSmem {
+  int scan[CM_THREADS / 32];
+  int pick;
+  int n_open, n_sure;
+  int flag;
+  float thr_hi, thr_lo;
+  int idx[CH_CAND_CAP];
+  float2 av[CH_CAND_CAP];          // a candidate's float32 |t| and the bound of its error
+  int open[CH_CAND_CAP];           // the candidates to recompute
+  double val[CH_CAND_CAP];         // their exact |t|
+  size_t row_off[CM_EXACT];        // of up to CM_EXACT of them: where their weight rows start, the rows' swizzle,
+  int row_swz[CM_EXACT];
+  double2 part[CM_EXACT][CM_THREADS / 32];  // the warps' sums of g and u
+};
 
 // Exact |t| of up to CM_EXACT open candidates, by the whole CTA: g_j = scale * sum_e x_e w_je with x the quantizer codes (or
 // the bf16 row), in float64.  A thread owns elements 8 tid .. + 7 of every 2048; the rows are on their way to L2 before the
@@ -356,9 +455,7 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
       g += sm.part[tid][w].x;
       u += sm.part[tid][w].y;
     }
-    const double unit = __hiloint2double((1023 + 896) << 20, 0);  // 2^896, see weight_to_f64
-    const double sc = (double)p.scale[b], ag = g * unit * sc, au = u * unit * sc;
-    sm.val[sm.open[i0 + tid]] = fabs(ag / (1.0 + exp(-ag)) * au);
+    sm.val[i0 + tid] = exact_score(g, u, (double)p.scale[b]);
   }
   __syncthreads();
 }
@@ -453,6 +550,7 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
 
   // ---- classify this CTA's channels: CM_GROUPS groups of four per thread ----
   int n_above = 0;
+  uint32_t between = 0;  // bit 4 gi + e
 #pragma unroll
   for (int gi = 0; gi < CM_GROUPS; ++gi) {
     const int j0 = slice * CM_SLICE + (gi * CM_THREADS + tid) * 4;
@@ -475,11 +573,7 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
         ++n_above;
         any = true;
       } else if (a >= lo_edge - ej) {
-        const uint32_t slot = atomicAdd(sel + CH_N_CAND, 1u);
-        if (slot < (uint32_t)CH_CAND_CAP) {
-          reinterpret_cast<float2*>(p.cand_val)[(size_t)b * CH_CAND_CAP + slot] = make_float2(a, ej + 2e-6f * a);  // and what the fast exponential and division add
-          p.cand_idx[(size_t)b * CH_CAND_CAP + slot] = j0 + e;
-        }
+        between |= 1u << (4 * gi + e);
       }
     }
     if (in) {  // four channels: half a piece of the packed operand
@@ -494,15 +588,44 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
     if (slice == 0 && tid == 0) p.kept_cnt[b] = m >= ff ? ff : 0;
     return;
   }
+  // the candidates' places: one request per warp
   n_above = __reduce_add_sync(0xffffffffu, n_above);
   if (lane == 0 && n_above) atomicAdd(sel + CH_N_ABOVE, (uint32_t)n_above);
+  {
+    const int mine = __popc(between);
+    int incl = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    uint32_t slot = 0;
+    if (lane == 31 && incl) slot = atomicAdd(sel + CH_N_CAND, (uint32_t)incl);
+    slot = __shfl_sync(0xffffffffu, slot, 31) + (uint32_t)(incl - mine);
+#pragma unroll
+    for (int gi = 0; gi < CM_GROUPS; ++gi) {
+      const float vv[4] = {v[gi].x, v[gi].y, v[gi].z, v[gi].w}, gg[4] = {gq[gi].x, gq[gi].y, gq[gi].z, gq[gi].w},
+                  uu[4] = {uq[gi].x, uq[gi].y, uq[gi].z, uq[gi].w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        if (!((between >> (4 * gi + e)) & 1u)) continue;
+        if (slot < (uint32_t)CH_CAND_CAP) {
+          const float a = fabsf(vv[e]), ej = eps * (1.1f * fabsf(uu[e]) + fabsf(gg[e]));
+          // and what the fast exponential and division add
+          reinterpret_cast<float2*>(p.cand_val)[(size_t)b * CH_CAND_CAP + slot] = make_float2(a, ej + 2e-6f * a);
+          p.cand_idx[(size_t)b * CH_CAND_CAP + slot] = slice * CM_SLICE + (gi * CM_THREADS + tid) * 4 + e;
+        }
+        ++slot;
+      }
+    }
+  }
 
   // ---- the last CTA of the token settles the candidates ----
   __threadfence();
   __syncthreads();
   if (tid == 0) {
     sm.flag = atomicAdd(sel + CH_DONE, 1u) == (uint32_t)(S - 1) ? 1 : 0;
-    sm.n_open = 0;
+    sm.n_open = sm.n_sure = 0;
   }
   __syncthreads();
   if (!sm.flag) return;
@@ -551,40 +674,33 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
   __syncthreads();
   for (int c = tid; c < n_cand; c += CM_THREADS) {
     const float2 a = sm.av[c];
-    double val = 1e300;                          // surely kept
-    if (a.x + a.y < sm.thr_lo) val = -1e300;     // surely dropped
-    else if (!(a.x - a.y > sm.thr_hi)) sm.open[atomicAdd(&sm.n_open, 1)] = c;
-    sm.val[c] = val;
+    if (a.x + a.y < sm.thr_lo) continue;  // surely dropped
+    if (a.x - a.y > sm.thr_hi) {          // surely kept: fewer than `need` candidates can be
+      atomicAdd(&sm.n_sure, 1);
+      keep_channel(p, b, sm.idx[c]);
+    } else {
+      sm.open[atomicAdd(&sm.n_open, 1)] = c;
+    }
   }
   __syncthreads();
-  const int n_open = sm.n_open;
+  const int n_open = sm.n_open, need_open = min(max(need - sm.n_sure, 0), n_open);
+  if (tid == 0) p.kept_cnt[b] = m;
+  if (p.hand_over > 0 && n_open * d > p.hand_over) {
+    for (int i = tid; i < n_open; i += CM_THREADS) p.cand_idx[(size_t)b * CH_CAND_CAP + i] = sm.idx[sm.open[i]];
+    if (tid == 0) sel[CH_OPEN] = ((uint32_t)n_open << 16) | (uint32_t)need_open;
+    return;
+  }
+  if (n_open == 0) return;
 #pragma unroll 1
   for (int i0 = 0; i0 < n_open; i0 += CM_EXACT) exact_candidates(p, sm, b, i0, min(CM_EXACT, n_open - i0));
-  for (int c0 = 0; c0 < n_cand; c0 += CM_THREADS / 4) {
-    const int c = c0 + (tid >> 2);
-    const double vc = c < n_cand ? sm.val[c] : 0.0;
-    const int j = c < n_cand ? sm.idx[c] : 0;
+  for (int c = tid; c < n_open; c += CM_THREADS) {
+    const double mine = sm.val[c];
+    const int j = sm.idx[sm.open[c]];
     int rank = 0;
-    for (int o = tid & 3; o < n_cand; o += 4) {
-      const double vo = sm.val[o];
-      rank += (vo > vc) || (vo == vc && sm.idx[o] < j);
-    }
-    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
-    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
-    if (c < n_cand && rank < need && (tid & 3) == 0) {
-      const float tv = p.t[(size_t)b * ff + j];
-      const uint16_t hv = f2bf(tv);
-      uint16_t* dst = reinterpret_cast<uint16_t*>(p.t_op + act_piece_offset(2 * p.Mpad, b, j >> 3) + (j & 7) * 2);
-      dst[0] = hv;
-      dst[(size_t)p.Mpad * 64] = f2bf(tv - bf2f(hv));
-      p.keep[(size_t)b * ff + j] = 1;
-      p.live[j >> 5] = 1;
-    }
+    for (int o = 0; o < n_open; ++o) rank += sm.val[o] > mine || (sm.val[o] == mine && sm.idx[sm.open[o]] < j);
+    if (rank < need_open) keep_channel(p, b, j);
   }
-  if (tid == 0) {
-    p.kept_cnt[b] = m;
-    atomicAdd(p.status + ST_CH_REFINED, n_open);
-  }
+  if (tid == 0) atomicAdd(p.status + ST_CH_REFINED, n_open);
 }
 
 // ============================================================================
@@ -610,21 +726,23 @@ void launch_channel_select(const ChannelSelectArgs& a, cudaStream_t st) {
   const NKGeom geo = nk_geom_gate_up(a.ff, a.d, sm_count());
   c.R = geo.R; c.chunks = geo.chunks; c.Mpad = pad_rows(a.B);
   c.sel = a.sel; c.cand_val = a.cand_val; c.cand_idx = a.cand_idx; c.keep = a.keep;
-  c.kept_ch = a.kept_ch; c.scratch_idx = a.scratch_idx; c.kept_cnt = a.kept_cnt;
+  c.kept_ch = a.kept_ch; c.kept_cnt = a.kept_cnt;
   c.t_op = static_cast<unsigned char*>(a.t_op);
   c.live = a.live; c.status = a.status;
   const long long resident = 3LL * sm_count();
   const int groups = (long long)((a.ff + CM_THREADS * 4 - 1) / (CM_THREADS * 4)) * a.B > resident ? 2 : 1;
   const dim3 mgrid((a.ff + CM_THREADS * 4 * groups - 1) / (CM_THREADS * 4 * groups), a.B);
+  // Where a token can have eight CTAs of its own, more than CH_HAND_OVER elements of open candidates are recomputed by them
+  // instead of by its last CTA of the first kernel: three tokens of a Llama-8B layer with 13 to 20 candidates of 4096 elements
+  // each 38 us for both kernels, this 21; 16 tokens of a Llama-1B layer with 4 of 2048 16 and 18; 64 tokens of a Llama-8B layer,
+  // two CTAs each, 44 both ways.
+  constexpr int CH_HAND_OVER = 24576;
+  const int per_token = sm_count() >= 8 * a.B ? 8 : 1;
+  c.hand_over = per_token > 1 ? CH_HAND_OVER : 0;
   if (groups == 1) SOL_LAUNCH("channel_select", channel_select_multi_kernel<1>, mgrid, dim3(CM_THREADS), 0, st, c);
   else SOL_LAUNCH("channel_select", channel_select_multi_kernel<2>, mgrid, dim3(CM_THREADS), 0, st, c);
   const dim3 grid(a.B);
-  // tokens the multi-CTA kernel handed over (it sets their flag); every other CTA leaves at once
-  if (a.ff <= 2048) SOL_LAUNCH("channel_select_exact", (channel_select_kernel<256, 8>), grid, dim3(256), 0, st, c);
-  else if (a.ff <= 8192) SOL_LAUNCH("channel_select_exact", (channel_select_kernel<512, 16>), grid, dim3(512), 0, st, c);
-  else if (a.ff <= 16384) SOL_LAUNCH("channel_select_exact", (channel_select_kernel<1024, 16>), grid, dim3(1024), 0, st, c);
-  else if (a.ff <= 32768) SOL_LAUNCH("channel_select_exact", (channel_select_kernel<1024, 32>), grid, dim3(1024), 0, st, c);
-  else SOL_LAUNCH("channel_select_exact", (channel_select_kernel<1024, 48>), grid, dim3(1024), 0, st, c);
+  SOL_LAUNCH("channel_select_exact", channel_select_rest_kernel, dim3(per_token, a.B), dim3(CR_THREADS), 0, st, c);
   if (a.kept_ch != nullptr) {
     if (a.ff <= 4096) SOL_LAUNCH("channel_list", (channel_list_kernel<256, 16>), grid, dim3(256), 0, st, a.keep, a.ff, a.kept_ch);
     else if (a.ff <= 16384) SOL_LAUNCH("channel_list", (channel_list_kernel<1024, 16>), grid, dim3(1024), 0, st, a.keep, a.ff, a.kept_ch);
