@@ -37,20 +37,6 @@ struct NoSmem {
   int unused;
 };
 
-// Four floats, or zeros where there are none.  Volatile: the loads of a group stay together ahead of their uses (left to
-// itself the compiler takes a few at a time, each with a round trip to L2).
-__device__ __forceinline__ float4 load4_if(const float* p, bool there) {
-  float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.u32 p, %5, 0;\n\t"
-      "@p ld.global.v4.f32 {%0, %1, %2, %3}, [%4];\n\t}"
-      : "+f"(v.x), "+f"(v.y), "+f"(v.z), "+f"(v.w)
-      : "l"(p), "r"((uint32_t)there)
-      : "memory");
-  return v;
-}
-
 // NV: vectors of eight elements per thread (d <= NV * 2048).  Latency-bound: what needs nothing of the kernels before (the
 // gains, the width) is read while they run, unless it is the first kernel of a call, and the code is compiled for the row's
 // length.  Where it is not the first kernel of a call, the row's code is run once on zeros ahead of the wait (a rehearsal, which
