@@ -187,108 +187,123 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
     if (ok && elect_one()) umma_commit(&bars->accum);
   } else {
     // -------------------------------- epilogue -------------------------------
-    pdl_wait_hold(p.hold);  // the epilogue reads scales and overwrites buffers earlier kernels used
-    if (EPI == EPI_SWIGLU) {
-      // the scales come to shared memory while the weights stream: a global load per token inside the loop
-      // below would put its latency between every two tokens
-      if ((int)threadIdx.x < p.Mpad) bars->scale[threadIdx.x] = (p.row_scale && (int)threadIdx.x < p.M) ? p.row_scale[threadIdx.x] : 1.0f;
-      if ((int)threadIdx.x < p.Mpad) {
-        bool need = (int)threadIdx.x < p.M;
-        if (need && p.sel_p != nullptr) {  // the kept count as the selection kernel computes it
-          const int m = (int)(((long long)(1000 - p.sel_p[threadIdx.x]) * p.N + 999) / 1000);
-          need = m > 0 && m < p.N;
-        }
-        bars->need_hist[threadIdx.x] = need ? 1 : 0;
-      }
-      asm volatile("bar.sync 1, %0;" ::"n"(UM_EPI_WARPS * 32) : "memory");  // the epilogue warps
-    }
-    // warps w, w + 4, w + 8, w + 12 share the accumulator lanes 32 (w % 4) .. and take alternate groups of tokens
-    const int quarter = warp & 3, half = warp >> 2;
-    if (quarter * 32 < p.R) {
-      const bool ok = mbar_wait(&bars->accum, 0, p.status);
-      tc_fence_after();
-      const int r = quarter * 32 + lane;  // row of the tile = accumulator lane
-      const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
-      if (EPI == EPI_SWIGLU) {
-        // Even lanes hold a channel's gate sums, their odd neighbours its up sums.  Every CTA runs this code
-        // once, so it is fetched cold: a short loop body (eight tokens, not unrolled further) that is fetched once
-        // and then runs from the instruction cache beats straight-line code for all tokens, which ran at ~14
-        // cycles per instruction.  The tokens are taken in pairs: the even lane gives away its gate sum of the
-        // second token and gets the up sum of the first, so each lane of a pair computes SwiGLU for one of the
-        // two tokens and no lane repeats its neighbour's work.  The chains of the four pairs are independent and
-        // branch-free (fast exponential and division: relative errors of about 2^-21 |g| and 2^-22, far inside
-        // the error the channel selection already allows for g itself).
-        const int ch = (tile * p.R + r) >> 1;
-        const bool valid = r < p.R && ch < p.N;
-        const bool even = (lane & 1) == 0;
-        float* const dst = even ? p.out0 : p.out1;
+    // SwiGLU: the first round is a rehearsal ahead of the wait, one group of tokens without the accumulators and without a
+    // store, so that the code is in the instruction caches when the sums are there (24 sequences: 16.1 us in the chain, this
+    // 14.2; the short code of the partial sums gains nothing).
+    int live = EPI == EPI_SWIGLU ? 0 : 1;
 #pragma unroll 1
-        for (int c0 = half * 8; c0 < p.M && ok; c0 += 8 * UM_EPI_SETS) {
-          uint32_t ra[8], rb[8];
-          tmem_ld8_issue(tl + c0, ra);
-          tmem_ld8_issue(tl + (p.n_b == 2 ? p.Mpad : 0) + c0, rb);  // high-part and low-part products
-          const float4 s0 = *reinterpret_cast<const float4*>(&bars->scale[c0]);
-          const float4 s1 = *reinterpret_cast<const float4*>(&bars->scale[c0 + 4]);
-          const float sc[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
-          tmem_ld_wait8(ra, rb);
-          float v[8], tv[4];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) v[i] = (__uint_as_float(ra[i]) + (p.n_b == 2 ? __uint_as_float(rb[i]) : 0.f)) * sc[i];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float got = __shfl_xor_sync(0xffffffffu, even ? v[2 * j + 1] : v[2 * j], 1);
-            const float g = even ? v[2 * j] : got, u = even ? got : v[2 * j + 1];
-            tv[j] = __fdividef(g, 1.0f + __expf(-g)) * u;
+    for (;; live = 1) {
+      asm volatile("" : "+r"(live));  // one code for both
+      if (live) {
+        pdl_wait_hold(p.hold);  // the epilogue reads scales and overwrites buffers earlier kernels used
+        if (EPI == EPI_SWIGLU) {
+          // the scales come to shared memory while the weights stream: a global load per token inside the loop
+          // below would put its latency between every two tokens
+          if ((int)threadIdx.x < p.Mpad) bars->scale[threadIdx.x] = (p.row_scale && (int)threadIdx.x < p.M) ? p.row_scale[threadIdx.x] : 1.0f;
+          if ((int)threadIdx.x < p.Mpad) {
+            bool need = (int)threadIdx.x < p.M;
+            if (need && p.sel_p != nullptr) {  // the kept count as the selection kernel computes it
+              const int m = (int)(((long long)(1000 - p.sel_p[threadIdx.x]) * p.N + 999) / 1000);
+              need = m > 0 && m < p.N;
+            }
+            bars->need_hist[threadIdx.x] = need ? 1 : 0;
           }
+          asm volatile("bar.sync 1, %0;" ::"n"(UM_EPI_WARPS * 32) : "memory");  // the epilogue warps
+        }
+      }
+      // warps w, w + 4, w + 8, w + 12 share the accumulator lanes 32 (w % 4) .. and take alternate groups of tokens
+      const int quarter = warp & 3, half = warp >> 2;
+      if (quarter * 32 < p.R) {
+        const bool ok = !live || mbar_wait(&bars->accum, 0, p.status);
+        tc_fence_after();
+        const int r = quarter * 32 + lane;  // row of the tile = accumulator lane
+        const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
+        if (EPI == EPI_SWIGLU) {
+          // Even lanes hold a channel's gate sums, their odd neighbours its up sums.  Every CTA runs this code
+          // once, so it is fetched cold: a short loop body (eight tokens, not unrolled further) that is fetched once
+          // and then runs from the instruction cache beats straight-line code for all tokens, which ran at ~14
+          // cycles per instruction.  The tokens are taken in pairs: the even lane gives away its gate sum of the
+          // second token and gets the up sum of the first, so each lane of a pair computes SwiGLU for one of the
+          // two tokens and no lane repeats its neighbour's work.  The chains of the four pairs are independent and
+          // branch-free (fast exponential and division: relative errors of about 2^-21 |g| and 2^-22, far inside
+          // the error the channel selection already allows for g itself).
+          const int ch = (tile * p.R + r) >> 1;
+          const bool valid = r < p.R && ch < p.N;
+          const bool even = (lane & 1) == 0;
+          float* const dst = even ? p.out0 : p.out1;
+#pragma unroll 1
+          for (int c0 = half * 8; c0 < (live ? p.M : half * 8 + 1) && ok; c0 += 8 * UM_EPI_SETS) {
+            uint32_t ra[8] = {0, 0, 0, 0, 0, 0, 0, 0}, rb[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+            if (live) {
+              tmem_ld8_issue(tl + c0, ra);
+              tmem_ld8_issue(tl + (p.n_b == 2 ? p.Mpad : 0) + c0, rb);  // high-part and low-part products
+            }
+            const float4 s0 = *reinterpret_cast<const float4*>(&bars->scale[c0]);
+            const float4 s1 = *reinterpret_cast<const float4*>(&bars->scale[c0 + 4]);
+            const float sc[8] = {s0.x, s0.y, s0.z, s0.w, s1.x, s1.y, s1.z, s1.w};
+            tmem_ld_wait8(ra, rb);
+            float v[8], tv[4];
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            if (c0 + i < p.M && valid) dst[(size_t)(c0 + i) * p.N + ch] = v[i];
-          const int mine = c0 + (even ? 0 : 1);  // the token of pair 0 whose t this lane holds
+            for (int i = 0; i < 8; ++i) v[i] = (__uint_as_float(ra[i]) + (p.n_b == 2 ? __uint_as_float(rb[i]) : 0.f)) * sc[i];
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if (mine + 2 * j < p.M && valid) p.out2[(size_t)(mine + 2 * j) * p.N + ch] = tv[j];
-          if (p.sel != nullptr) {
-            // what the channel selection needs from all of a token's channels: a histogram of |t| and the largest
-            // |g|, |u| (non-negative floats order like their bit patterns).  The maxima of this warp's 16 channels
-            // go to the warp's own words in shared memory (no atomics); the CTA merges them at the end.
+            for (int j = 0; j < 4; ++j) {
+              const float got = __shfl_xor_sync(0xffffffffu, even ? v[2 * j + 1] : v[2 * j], 1);
+              const float g = even ? v[2 * j] : got, u = even ? got : v[2 * j + 1];
+              tv[j] = __fdividef(g, 1.0f + __expf(-g)) * u;
+            }
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+              if (live && c0 + i < p.M && valid) dst[(size_t)(c0 + i) * p.N + ch] = v[i];
+            const int mine = c0 + (even ? 0 : 1);  // the token of pair 0 whose t this lane holds
 #pragma unroll
             for (int j = 0; j < 4; ++j)
-              if (mine + 2 * j < p.M && valid && bars->need_hist[mine + 2 * j])
-                atomicAdd(p.sel + (size_t)(mine + 2 * j) * CH_SEL_WORDS + chan_bin(fabsf(tv[j])), 1u);
-            uint32_t gs = 0u, us = 0u;
+              if (live && mine + 2 * j < p.M && valid) p.out2[(size_t)(mine + 2 * j) * p.N + ch] = tv[j];
+            if (p.sel != nullptr) {
+              // what the channel selection needs from all of a token's channels: a histogram of |t| and the largest
+              // |g|, |u| (non-negative floats order like their bit patterns).  The maxima of this warp's 16 channels
+              // go to the warp's own words in shared memory (no atomics); the CTA merges them at the end.
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const uint32_t a = valid ? __float_as_uint(fabsf(v[i])) : 0u;
-              const uint32_t gm = __reduce_max_sync(0xffffffffu, even ? a : 0u);
-              const uint32_t um = __reduce_max_sync(0xffffffffu, even ? 0u : a);
-              gs = lane == i ? gm : gs;
-              us = lane == i ? um : us;
-            }
-            if (lane < 8) {
-              bars->gmax[quarter][c0 + lane] = gs;
-              bars->umax[quarter][c0 + lane] = us;
+              for (int j = 0; j < 4; ++j)
+                if (live && mine + 2 * j < p.M && valid && bars->need_hist[mine + 2 * j])
+                  atomicAdd(p.sel + (size_t)(mine + 2 * j) * CH_SEL_WORDS + chan_bin(fabsf(tv[j])), 1u);
+              uint32_t gs = 0u, us = 0u;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const uint32_t a = valid ? __float_as_uint(fabsf(v[i])) : 0u;
+                const uint32_t gm = __reduce_max_sync(0xffffffffu, even ? a : 0u);
+                const uint32_t um = __reduce_max_sync(0xffffffffu, even ? 0u : a);
+                gs = lane == i ? gm : gs;
+                us = lane == i ? um : us;
+              }
+              if (live && lane < 8) {
+                bars->gmax[quarter][c0 + lane] = gs;
+                bars->umax[quarter][c0 + lane] = us;
+              }
             }
           }
-        }
-      } else {
-        const int n = tile * p.R + r;
-        const bool valid = r < p.R && n < p.N;
-        for (int c0 = half * 16; c0 < p.Mpad && ok; c0 += 16 * UM_EPI_SETS) {
-          float v[16];
-          tmem_ld16(tl + c0, v);
-          if (p.n_b == 2) {  // high-part and low-part products
-            float w2[16];
-            tmem_ld16(tl + p.Mpad + c0, w2);
+        } else {
+          const int n = tile * p.R + r;
+          const bool valid = r < p.R && n < p.N;
+          for (int c0 = half * 16; c0 < (live ? p.Mpad : half * 16 + 1) && ok; c0 += 16 * UM_EPI_SETS) {
+            float v[16];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] += w2[i];
-          }
+            for (int i = 0; i < 16; ++i) v[i] = 0.f;
+            if (live) tmem_ld16(tl + c0, v);
+            if (p.n_b == 2 && live) {  // high-part and low-part products
+              float w2[16];
+              tmem_ld16(tl + p.Mpad + c0, w2);
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const int m = c0 + i;
-            if (m < p.M && valid) p.out0[((size_t)blockIdx.y * p.M + m) * p.N + n] = v[i];
+              for (int i = 0; i < 16; ++i) v[i] += w2[i];
+            }
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+              const int m = c0 + i;
+              if (live && m < p.M && valid) p.out0[((size_t)blockIdx.y * p.M + m) * p.N + n] = v[i];
+            }
           }
         }
       }
+      if (live) break;
     }
   }
   tc_fence_before();
