@@ -244,7 +244,7 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
                     const int32_t* p_permille, const void* resid, int resid_f32, void* out_bf16,
                     float* out_f32, float* out_f32_b, float* t_trace, int32_t* kept_ch, int32_t* kept_ch_cnt,
                     cudaStream_t st, const int32_t* out_bits = nullptr, const sol_layer_trace_t* tr = nullptr,
-                    LayerCarry* carry_out = nullptr, bool hold = false) {
+                    LayerCarry* carry_out = nullptr, bool hold = false, bool keeps_all = false) {
   int* status = at<int>(ws, L.status);
   GemmNK gu;
   memset(&gu, 0, sizeof(gu));
@@ -283,6 +283,7 @@ static void run_mlp(const sol_shape_t& s, const Layout& L, void* ws, int B, cons
   cs.kept_cnt = kept_ch_cnt ? kept_ch_cnt : at<int32_t>(ws, L.kept_ch_cnt);
   cs.t_op = at<void>(ws, L.t_hi);
   cs.live = at<int32_t>(ws, L.live);
+  cs.keeps_all = keeps_all;
   cs.status = status;
   launch_channel_select(cs, st);
 
@@ -328,7 +329,7 @@ static void run_layer(const sol_shape_t& s, const Layout& L, void* ws, const sol
                       const sol_kv_t& kv, int B, const void* h_in, bool in_f32, void* h_out_bf16, float* h_out_f32,
                       const int32_t* r, const int32_t* p, const int32_t* bits, const sol_layer_trace_t* tr,
                       cudaStream_t st, bool first, const LayerCarry* carry_in = nullptr,
-                      LayerCarry* carry_out = nullptr, int span_tokens = 0) {
+                      LayerCarry* carry_out = nullptr, int span_tokens = 0, bool dense = false) {
   int* status = at<int>(ws, L.status);
   const int d = s.d_model, Hq = s.n_q_heads, Hkv = s.n_kv_heads, hd = s.head_dim;
   const int Nqkv = (Hq + 2 * Hkv) * hd;
@@ -413,7 +414,7 @@ static void run_layer(const sol_shape_t& s, const Layout& L, void* ws, const sol
   run_mlp(s, L, ws, B, w.w_gate_up, w.w_down, gate_inputs ? at<int32_t>(ws, L.zero_p) : p, at<float>(ws, L.h_mid), 1,
           h_out_bf16, h_out_f32,
           tr ? tr->h_out : nullptr, tr ? tr->t : nullptr, tr ? tr->kept_ch : nullptr, tr ? tr->kept_ch_cnt : nullptr,
-          st, out_quant ? bits : nullptr, tr, carry_out);
+          st, out_quant ? bits : nullptr, tr, carry_out, false, gate_inputs || dense);
 }
 
 static bool weights_ok(const sol_layer_weights_t* w) {
@@ -735,7 +736,7 @@ sol_status_t sol_kv_refresh(const sol_shape_t* shape, int32_t n_layers, const so
       // up to 16 tokens per sequence are the rows of one tensor-core tile of the span attention, which reads a
       // sequence's cache once for all of them; longer spans go through the decode step's attention row by row
       run_layer(dense, L, ws, layers[l], kv, rows, h, in_f32, last ? out : nullptr, last && out ? nullptr : out32, act,
-                act + rows, act + 2 * rows, nullptr, st, expand, nullptr, nullptr, n_tokens <= 16 ? n_tokens : 0);
+                act + rows, act + 2 * rows, nullptr, st, expand, nullptr, nullptr, n_tokens <= 16 ? n_tokens : 0, true);
       h = out32;
       in_f32 = true;
     }

@@ -357,6 +357,7 @@ struct ChannelSelectArgs {
   int32_t* kept_cnt;   // [B]
   void* t_op;          // packed operand of the down projection: 2 pad_rows(B) rows (bf16 high parts, then low parts)
   int32_t* live;       // [ff/32], all zero on entry (cleared by reduce_out after the down projection)
+  bool keeps_all;      // the caller knows that no token prunes: nothing can be left to the second kernel
   int* status;
 };
 void launch_channel_select(const ChannelSelectArgs& a, cudaStream_t st);

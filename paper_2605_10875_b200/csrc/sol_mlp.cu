@@ -742,7 +742,8 @@ void launch_channel_select(const ChannelSelectArgs& a, cudaStream_t st) {
   if (groups == 1) SOL_LAUNCH("channel_select", channel_select_multi_kernel<1>, mgrid, dim3(CM_THREADS), 0, st, c);
   else SOL_LAUNCH("channel_select", channel_select_multi_kernel<2>, mgrid, dim3(CM_THREADS), 0, st, c);
   const dim3 grid(a.B);
-  SOL_LAUNCH("channel_select_exact", channel_select_rest_kernel, dim3(per_token, a.B), dim3(CR_THREADS), 0, st, c);
+  if (!a.keeps_all)
+    SOL_LAUNCH("channel_select_exact", channel_select_rest_kernel, dim3(per_token, a.B), dim3(CR_THREADS), 0, st, c);
   if (a.kept_ch != nullptr) {
     if (a.ff <= 4096) SOL_LAUNCH("channel_list", (channel_list_kernel<256, 16>), grid, dim3(256), 0, st, a.keep, a.ff, a.kept_ch);
     else if (a.ff <= 16384) SOL_LAUNCH("channel_list", (channel_list_kernel<1024, 16>), grid, dim3(1024), 0, st, a.keep, a.ff, a.kept_ch);
