@@ -43,7 +43,10 @@ struct NoSmem {
 // reads nothing that an earlier kernel writes and writes nothing), so that it is in the instruction caches.
 // In the chain, per launch: a single sequence 4.9 us, this 3.3; 24 to 32 sequences 7.3 and 5.5; with the input gating 16.5
 // and 12.1.
-template <bool IN_F32, bool GATE, int NV>
+// PART: the row comes with the partial sums of a projection.  Their loads in flight take up to 200 registers, one CTA per SM,
+// which a layer's 128 rows fit; the stand-alone quantizer takes any number of rows and has none (26 to 64 registers; a call
+// of thousands of rows took 29 us with the registers of the partial sums, 9 without).
+template <bool IN_F32, bool GATE, int NV, bool PART>
 __global__ void __launch_bounds__(NQ_THREADS)
 norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, int ksplit, size_t part_stride,
                   float* __restrict__ sum_out, const uint16_t* __restrict__ gamma, float eps,
@@ -67,10 +70,12 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
     if (gamma != nullptr && v < d / NQ_VEC) gains[i] = reinterpret_cast<const uint4*>(gamma)[v];
   }
   const int width = bits ? __ldcg(bits + row) : 16;
-  int live = first ? 1 : 0;
+  // a bf16 row without partial sums is an input of the call: that kernel is the first one, or the stand-alone quantizer
+  constexpr bool REHEARSE = PART || GATE || IN_F32;
+  int live = !REHEARSE || first ? 1 : 0;
 #pragma unroll 1
   for (;; live = 1) {
-    asm volatile("" : "+r"(live));  // one code for a rehearsal and the row
+    if (REHEARSE) asm volatile("" : "+r"(live));  // one code for a rehearsal and the row
     if (live) pdl_wait();
     int b = width;
     if (zero_flags != nullptr && live)
@@ -88,9 +93,9 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
 #pragma unroll
       for (int e = 0; e < NQ_VEC; ++e) x[i][e] = 0.f;
       if (v < nvec) {
-        float4 a[ZB], b4[ZB];
+        float4 a[PART ? ZB : 1], b4[PART ? ZB : 1];
         const float* src = part + (size_t)row * d + 8 * v;
-        if (part != nullptr) {  // partial sums of the projection that produced this row: ZB slices' loads in flight
+        if (PART && part != nullptr) {  // partial sums of the projection that produced this row: ZB slices' loads in flight
 #pragma unroll
           for (int q = 0; q < ZB; ++q) {
             a[q] = load4_if(src + (size_t)q * part_stride, live && q < ksplit);
@@ -112,7 +117,7 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
 #pragma unroll
           for (int e = 0; e < NQ_VEC; ++e) x[i][e] = (float)((8 * v + e) * 389 & 0x1fff);
         }
-        if (part != nullptr) {  // added in slice order
+        if (PART && part != nullptr) {  // added in slice order
 #pragma unroll 1
           for (int z0 = 0;;) {
 #pragma unroll
@@ -307,24 +312,30 @@ void launch_norm_quant(const NormQuantArgs& a, cudaStream_t st) {
   GateArgs g;
   g.p_permille = a.gate_p_permille;
   g.xm = a.xm;
-#define SOL_NQ_LAUNCH(F32, GATE, NV)                                                                                   \
-  SOL_LAUNCH("norm_quant", (norm_quant_kernel<F32, GATE, NV>), dim3(a.B), dim3(NQ_THREADS), 0, st, a.in, a.part,         \
+#define SOL_NQ_LAUNCH(F32, GATE, NV, PART)                                                                                   \
+  SOL_LAUNCH("norm_quant", (norm_quant_kernel<F32, GATE, NV, PART>), dim3(a.B), dim3(NQ_THREADS), 0, st, a.in, a.part,         \
              a.ksplit, stride, a.sum_out, static_cast<const uint16_t*>(a.gamma_bf16), a.eps, a.bits, a.d,              \
              static_cast<uint16_t*>(a.a_op), a.a_op_rows, a.scale, a.xn, a.codes, a.codes16, a.status, a.clear,         \
              a.clear_words, a.zero_flags, a.n_zero_flags, a.first, g)
-#define SOL_NQ_BY_SIZE(F32, GATE)                          \
+#define SOL_NQ_BY_SIZE(F32, GATE, PART)                    \
   do {                                                     \
-    if (a.d <= 2048) SOL_NQ_LAUNCH(F32, GATE, 1);          \
-    else if (a.d <= 4096) SOL_NQ_LAUNCH(F32, GATE, 2);     \
-    else SOL_NQ_LAUNCH(F32, GATE, 4);                      \
+    if (a.d <= 2048) SOL_NQ_LAUNCH(F32, GATE, 1, PART);      \
+    else if (a.d <= 4096) SOL_NQ_LAUNCH(F32, GATE, 2, PART); \
+    else SOL_NQ_LAUNCH(F32, GATE, 4, PART);                  \
+  } while (0)
+#define SOL_NQ_BY_PART(F32, GATE)                          \
+  do {                                                     \
+    if (a.part != nullptr) SOL_NQ_BY_SIZE(F32, GATE, true); \
+    else SOL_NQ_BY_SIZE(F32, GATE, false);                  \
   } while (0)
   if (a.gate_p_permille != nullptr) {
-    if (a.in_f32) SOL_NQ_BY_SIZE(true, true);
-    else SOL_NQ_BY_SIZE(false, true);
+    if (a.in_f32) SOL_NQ_BY_PART(true, true);
+    else SOL_NQ_BY_PART(false, true);
   } else {
-    if (a.in_f32) SOL_NQ_BY_SIZE(true, false);
-    else SOL_NQ_BY_SIZE(false, false);
+    if (a.in_f32) SOL_NQ_BY_PART(true, false);
+    else SOL_NQ_BY_PART(false, false);
   }
+#undef SOL_NQ_BY_PART
 #undef SOL_NQ_BY_SIZE
 #undef SOL_NQ_LAUNCH
 }
