@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(SC_WARPS * 32) attn_score_kernel(const ScoreDe
 // ============================================================================
 // Exact top-k of a (sequence, kv-head) row of scores.
 //
-//   token_select one CTA per 8192 tokens: histogram of its scores over 4096 value bins in shared memory,
+//   token_select one CTA per 16384 tokens: histogram of its scores over 4096 value bins in shared memory,
 //                flushed (non-empty bins) to the row's histogram in global memory, and the largest |score|.
 //                The CTA that finishes last (rows of one segment go straight on) finds the bin of the k-th
 //                largest score and two values: everything above `edge` (the bin's upper end plus a small
@@ -857,7 +857,7 @@ __device__ __forceinline__ void settle_row(const SelectDev& p, SelectSmemOverlay
 
 constexpr int TS_REHEARSAL = 1024;  // scores of a rehearsal
 
-// One (sequence, kv-head, 8192-token segment) of a row that needs a selection; the phase of hs.bar is the caller's.
+// One (sequence, kv-head, 16384-token segment) of a row that needs a selection; the phase of hs.bar is the caller's.
 // live == false: a rehearsal on made-up scores, 1/64 apart, which reads and writes shared memory only.  scores_read: called
 // by all threads when hs.score is no longer needed (the caller then lets the next unit's scores come).
 template <typename ScoresRead>
