@@ -1,5 +1,8 @@
 """Kernels at the sizes where their tiling can go wrong: remainders, single tiles, the smallest and largest of a range;
 values that a wrong step shows in (zeros, infinities, NaNs); inputs that are written late."""
+import os
+import zlib
+
 import numpy as np
 import pytest
 import torch
@@ -53,6 +56,29 @@ def test_attention_of_a_full_batch():
     cfg = dict(TINY, n_q_heads=8, n_kv_heads=8, d_model=512)
     rng = np.random.default_rng(5)
     _attention_case(cfg, rng.integers(1, 1300, 128), rng.choice([60, 125, 500, 999, 1000], 128), seed=5)
+
+
+# The last bits of rows that are merged from 2 to 32 partial results, and from more: the order of the sums is fixed, so that a
+# program gets the same results from every build.  The file has a checksum for every query head, of results that were compared
+# with the oracle like all others; a change that is meant to round otherwise records them anew.
+def merged_row_checksums(hd, hq, hkv):
+    cfg = dict(TINY, head_dim=hd, n_q_heads=hq, n_kv_heads=hkv, d_model=256)
+    shape, _ = H.make_shapes(cfg)
+    lens = np.asarray([300, 2049, 4096, 8192, 12000, 9000], np.int32)
+    k_pool, v_pool, table = H.make_case_kv(cfg, lens, 9)
+    dw = H.device_weights(synth.make_layer_weights(cfg, 9), shape)
+    B = len(lens)
+    _, taps, st = H.gpu_layer(shape, dw, H.device_kv(k_pool, v_pool, table, lens), synth.make_hidden(cfg, 9, B),
+                              [1000, 1000, 500, 1000, 1000, 250], [0] * B, [16] * B)
+    assert st[0] == 0
+    return [[hd, hq, hkv, b, h, zlib.crc32(taps["attn_out"][b, h].tobytes())] for b in range(B) for h in range(hq)]
+
+
+@pytest.mark.parametrize("hd,hq,hkv", [(64, 4, 1), (64, 8, 1), (128, 4, 2)])
+def test_merged_rows_bit_for_bit(hd, hq, hkv):
+    golden = np.loadtxt(os.path.join(os.path.dirname(__file__), "golden", "merged_rows.txt"), dtype=np.int64)
+    want = golden[(golden[:, :3] == [hd, hq, hkv]).all(1)]
+    assert len(want) == 6 * hq and np.array_equal(merged_row_checksums(hd, hq, hkv), want)
 
 
 # The exact re-scoring of the channel selection: rows shorter than, equal to and longer than what a CTA takes at once (2048
