@@ -159,6 +159,12 @@ __device__ __forceinline__ int plan_find(const int* cum, int n, int u) {
 // ============================================================================
 // attn_prep
 // ============================================================================
+// Rotation of an element pair.  The multiply-adds are spelled out: left to the compiler, which of the two products is rounded
+// by itself differed between the queries and the keys, and between builds.
+__device__ __forceinline__ float2 rotate(float x0, float x1, float c, float s) {
+  return make_float2(__fmaf_rn(x0, c, -__fmul_rn(x1, s)), __fmaf_rn(x1, c, __fmul_rn(x0, s)));
+}
+
 struct PrepDev {
   sol_shape_t sh;
   sol_kv_t kv;
@@ -273,9 +279,9 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
       const int gi = i / half, f = i % half, h = kvh * G + gi;
       float q0, q1;
       if (layer) {
-        const float x0 = rowbuf[gi * hd + f], x1 = rowbuf[gi * hd + f + half];
-        q0 = x0 * cs[f] + (-x1) * sn[f];
-        q1 = x1 * cs[f] + x0 * sn[f];
+        const float2 v = rotate(rowbuf[gi * hd + f], rowbuf[gi * hd + f + half], cs[f], sn[f]);
+        q0 = v.x;
+        q1 = v.y;
       } else {
         const uint16_t* src = p.q_bf16 + ((size_t)b * Hq + h) * hd;
         q0 = bf2f(src[f]);
@@ -316,8 +322,8 @@ __global__ void __launch_bounds__(PREP_THREADS) attn_prep_kernel(const PrepDev p
       const float* vr = rowbuf + (G + 1) * hd;
       const size_t dst = (((size_t)page * Hkv + kvh) * PAGE + slot) * hd;
       for (int f = tid; f < half; f += PREP_THREADS) {
-        const float x0 = kr[f], x1 = kr[f + half];
-        const uint16_t k0 = f2bf(x0 * cs[f] + (-x1) * sn[f]), k1 = f2bf(x1 * cs[f] + x0 * sn[f]);
+        const float2 k = rotate(kr[f], kr[f + half], cs[f], sn[f]);
+        const uint16_t k0 = f2bf(k.x), k1 = f2bf(k.y);
         const uint16_t v0 = f2bf(vr[f]), v1 = f2bf(vr[f + half]);
         if (good && live) {
           kp[dst + f] = k0;

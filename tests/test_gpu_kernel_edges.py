@@ -81,6 +81,27 @@ def test_merged_rows_bit_for_bit(hd, hq, hkv):
     assert len(want) == 6 * hq and np.array_equal(merged_row_checksums(hd, hq, hkv), want)
 
 
+# Queries and keys are rotated alike, to the last bit: the key's rows of the projection are those of its group's first query
+# head, both halves of a pair have the same sums, and at these positions their products nearly cancel, so that what is rounded
+# where shows in many of the 16-bit results.
+def test_queries_and_keys_rotate_alike():
+    cfg = dict(TINY, d_model=512, n_q_heads=8, n_kv_heads=4, rope_theta=10000.0)
+    B, hd, d = 64, 64, 512
+    shape, _ = H.make_shapes(cfg)
+    at = np.arange(64, 2048)
+    pos = np.resize([at[np.argmin(np.abs(np.cos(at) + np.sin(at)))], at[np.argmin(np.abs(np.cos(at) - np.sin(at)))]], B)
+    lens = (pos + 1).astype(np.int32)
+    k_pool, v_pool, table = H.make_case_kv(cfg, lens, 2)
+    w = synth.make_layer_weights(cfg, 2)
+    rows = w.w_qkv.reshape(16, 2, hd // 2, d)  # 8 query heads, 4 keys, 4 values
+    rows[:, 1] = rows[:, 0]
+    rows[8:12] = rows[0:8:2]
+    kv = H.device_kv(k_pool, v_pool, table, lens)
+    _, taps, st = H.gpu_layer(shape, H.device_weights(w, shape), kv, synth.make_hidden(cfg, 2, B), [500] * B, [0] * B, [16] * B)
+    new = H.host_u16(kv.k_pool)[table[np.arange(B), pos // 64], :, pos % 64]  # [B][kv-head][hd]
+    assert st[0] == 0 and np.array_equal(new, synth.to_bf16(taps["q_rot"][:, ::2]))
+
+
 # The exact re-scoring of the channel selection: rows shorter than, equal to and longer than what a CTA takes at once (2048
 # elements), and more open candidates than one pass takes (groups of identical channels around the threshold).
 @pytest.mark.parametrize("d,ff", [(256, 1056), (2048, 512), (2304, 512), (4096, 1024), (8192, 256)])
