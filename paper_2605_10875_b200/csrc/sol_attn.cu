@@ -107,6 +107,7 @@ constexpr int ITEM_C0 = 64, ITEM_NC = 5;
 struct PlanSmem {
   int cum[PLAN_STRIDE];
   int n_items[ITEM_NC], longest[ITEM_NC];  // per option: items of a kv-head, kept tokens of the longest
+  int sel_units;  // units of token_select of a kv-head
   int wsum[4], per_item;
 };
 // By the first 128 threads of the CTA.  The options are tried in a rolled loop: this runs once per CTA, at the pace at which
@@ -115,10 +116,13 @@ __device__ __forceinline__ int plan_items(const sol_shape_t& sh, const sol_kv_t&
                                           int target_items, PlanSmem& ps) {
   const int tid = threadIdx.x, lane = tid & 31;
   if (tid < ITEM_NC) ps.n_items[tid] = ps.longest[tid] = 0;
+  if (tid == 0) ps.sel_units = 0;
   plan_sync();
   RowPlan rp;
-  rp.T = rp.k = 0;
+  rp.T = rp.k = rp.mode = 0;
   if (tid < B) rp = row_plan(sh, kv, r_permille, tid);
+  const int units = __reduce_add_sync(0xffffffffu, rp.mode == 2 ? (rp.T + TH_SEG - 1) / TH_SEG : 0);
+  if (lane == 0 && units) atomicAdd(&ps.sel_units, units);
   auto items_of = [&](int c) {  // one item at least, so that the output is always written
     const int len = gather_item_tokens(rp, c, min_len);
     return max(1, (rp.T + len - 1) / len);
@@ -710,6 +714,7 @@ struct SelectDev {
   uint32_t* row_ctl;     // [B*Hkv][RC_WORDS], zero on entry
   int32_t* kept_cnt;
   int32_t* work_ctr;
+  int few;               // the grid is a quarter of the SMs at most
   int* status;
 };
 
@@ -1104,12 +1109,18 @@ __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(con
     mbar_init(&hs.bar, 1);
     fence_mbar_init();
   }
+  int len = 0;
+  if (tid < p.B) {
+    const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
+    if (rp.mode == 2) len = rp.T;
+  }
+  // Nothing to select: pass 2 is not kept waiting for the order of the units, and has the SMs at once.  The first CTA waits for
+  // the kernels before, on which the ones after rely.
+  if (p.few && __syncthreads_or(len) == 0) {
+    if (blockIdx.x == 0) pdl_wait();
+    return;
+  }
   if (tid < 128) {
-    int len = 0;
-    if (tid < p.B) {
-      const RowPlan rp = row_plan(p.sh, p.kv, p.r_permille, tid);
-      if (rp.mode == 2) len = rp.T;
-    }
     hs.len[tid] = len;
     plan_sync();
     int rank = 0;
@@ -1125,6 +1136,7 @@ __global__ void __launch_bounds__(TS_THREADS, TS_PER_SM) token_select_kernel(con
   }
   __syncthreads();
   const int n_units = hs.cum[128] * Hkv;
+  if (p.few && (int)blockIdx.x >= n_units) return;  // makes room for pass 2
   uint32_t phase = 0;
   int live = rehearse && (int)blockIdx.x < n_units ? 0 : 1;
   int unit = blockIdx.x, next = blockIdx.x;
@@ -1232,7 +1244,7 @@ struct GatherDev {
   float scale_log2;
   AttnOut out;
   int* status;
-  int rehearse;
+  int sure_ctas;  // CTAs that are there before the selection ends, whatever it has to do; 0: no rule on that
 };
 
 constexpr int GA_BATCH = 32;   // kept tokens per warp step: one per lane in the softmax part
@@ -1303,20 +1315,34 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
   float* ml = reinterpret_cast<float*>(my_q);  // at the end of an item: [GMAX] maxima, [GMAX] sums
   pdl_trigger();
   // The first four warps make the list of items; the others wait for it at a barrier that the first four only arrive at.
-  // Where CTAs are there early (`rehearse`), the last quarter of the warps rehearse meanwhile: they run the code of an item
-  // on absent tokens (even warps that of a selected row, odd ones that of a row that keeps every token), write nothing and
-  // leave the code in the instruction caches.  The first pass through code that comes from L2 was half of the time of a
-  // launch with one item per warp (a single sequence of 2000 tokens: 19.5 us in the chain, 11.8 with the rehearsal).
-  int live = 1, per_item = 0, n_items = 0, item = warp * gridDim.x + blockIdx.x;
+  // Where CTAs are there early (the first `sure_ctas`), the last quarter of the warps rehearse meanwhile: they run the code of
+  // an item on absent tokens (even warps that of a selected row, odd ones that of a row that keeps every token; the merge
+  // loads whatever the first slot of the partial results holds and drops it), write nothing and leave the code in the
+  // instruction caches.  The first pass through code that comes from L2 was half of the time of a launch with one item per
+  // warp (a single sequence of 2000 tokens: 19.5 us in the chain, 11.8 with the rehearsal).
+  // The selection's CTAs hold SMs until it ends, and the CTAs of this kernel that wait for those are there late: where the
+  // others have a warp for every item, they take all of them (attention of four sequences of 8000 tokens, a quarter kept, 64-wide
+  // heads: 38.4 us, dealt to every CTA 40.6); else every CTA has its share (128-wide heads, more items than the others have
+  // warps: 52.7 us, with the rest left to whoever is free first 62.8).  Up to three items per CTA go to the CTAs that are
+  // there whatever the selection does (2000 tokens, all kept: 20.2, dealt to every CTA 21.6).
+  int live = 1, per_item = 0, n_items = 0, item = 0;
   bool planned = false, waited = false;
   const int total_warps = gridDim.x * WARPS;
-  if (warp < 4) {
-    per_item = plan_items(p.sh, p.kv, p.r_permille, p.B, p.min_len, p.sms * WARPS, ps);
-    if (threadIdx.x == 0) ps.per_item = per_item;
+  auto read_plan = [&] {
+    per_item = ps.per_item;
     n_items = cum[p.B] * Hkv;
+    const int grid = gridDim.x, early = min(grid, max(p.sure_ctas, p.sms - ps.sel_units * Hkv));
+    const int deal = p.sure_ctas == 0 ? grid : n_items <= 3 * p.sure_ctas ? min(grid, p.sure_ctas) : n_items <= early * WARPS ? early : grid;
+    item = (int)blockIdx.x < deal ? warp * deal + blockIdx.x : n_items;
     planned = true;
+  };
+  if (warp < 4) {
+    const int c = plan_items(p.sh, p.kv, p.r_permille, p.B, p.min_len, p.sms * WARPS, ps);
+    if (threadIdx.x == 0) ps.per_item = c;
+    plan_sync();
+    read_plan();
     asm volatile("bar.arrive 2, %0;" ::"n"(C::THREADS) : "memory");  // the list is there
-  } else if (p.rehearse && warp >= C::REHEARSE) {
+  } else if ((int)blockIdx.x < p.sure_ctas && warp >= C::REHEARSE) {
     live = 0;
   }
 #pragma unroll 1
@@ -1325,9 +1351,7 @@ __global__ void __launch_bounds__(GatherCfg<HD, GMAX>::THREADS, 1) attn_gather_k
     if (live) {
       if (!planned) {
         asm volatile("bar.sync 2, %0;" ::"n"(C::THREADS) : "memory");
-        planned = true;
-        per_item = ps.per_item;
-        n_items = cum[p.B] * Hkv;
+        read_plan();
       }
       if (item >= n_items) break;
     }
@@ -1746,10 +1770,10 @@ static void launch_score(const ScoreDev& d, int groups_per_row, cudaStream_t st)
 
 // Persistent: at most one CTA per SM.
 template <int HD, int GMAX>
-static void launch_gather(const GatherDev& d, long long items, int ctas, cudaStream_t st) {
+static void launch_gather(const GatherDev& d, long long items, cudaStream_t st) {
   using C = GatherCfg<HD, GMAX>;
   ensure_dynamic_smem(reinterpret_cast<const void*>(&attn_gather_kernel<HD, GMAX>), C::SMEM);
-  const int grid = (int)(items < ctas ? items : ctas);
+  const int grid = (int)(items < d.sms ? items : d.sms);
   SOL_LAUNCH("attn_gather_v", (attn_gather_kernel<HD, GMAX>), dim3(grid), dim3(C::THREADS), C::SMEM, st, d);
 }
 
@@ -1806,6 +1830,10 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   const long long sel_units = (long long)a.B * Hkv * ((Tmax + TH_SEG - 1) / TH_SEG), sel_res = (long long)sm_count() * TS_PER_SM;
   ensure_dynamic_smem(reinterpret_cast<const void*>(&token_select_kernel), (int)sizeof(SelSmem));
   const int sel_ctas = (int)(sel_units < sel_res ? sel_units : sel_res);
+  // Few CTAs: those without a unit leave ahead of the kernels before, so that pass 2 has their SMs (four sequences of 8000 tokens,
+  // every token kept: 30 us with it, 33 with those SMs left out).  Of many this does not pay throughout: steps of 48, 64 and 96
+  // sequences of 500 tokens, every token kept, 3 to 5 % slower, of 24 and 128 as much faster.
+  se.few = sel_ctas <= sm_count() / 4;
   const long long score_ctas = (long long)a.B * Hkv * groups_per_row;
   // A rehearsal (about 3 us) pays where a CTA is there well before pass 1 ends: where the CTAs of both leave room for each
   // other on every SM.  Elsewhere a CTA starts when one of pass 1 ends, and a rehearsal is in its way (16 sequences of 4096
@@ -1826,17 +1854,15 @@ void launch_attention(const AttnArgs& a, cudaStream_t st) {
   gd.logits = a.logits; gd.sigma = a.sigma; gd.row_ctl = a.row_ctl; gd.work_ctr = a.work_ctr; gd.sms = sm_count();
   gd.part = a.part; gd.scale_log2 = (float)(1.4426950408889634 / sqrt((double)hd)); gd.out = out; gd.status = a.status;
   const long long items = (long long)a.B * Hkv * a.splits;
-  // The selection's CTAs hold their SMs until it ends.  Where they are few, pass 2 leaves those SMs alone: its CTAs are then
-  // there early and have the time for a rehearsal.  Where they are many, a rehearsal delays the items (24 sequences of about
-  // 2000 tokens: 22.8 us without, 25.2 with it).
-  const int gather_ctas = sel_ctas <= sm_count() / 4 ? sm_count() - sel_ctas : sm_count();
-  gd.rehearse = gather_ctas < sm_count();
+  // Where the selection's CTAs are few, the CTAs of pass 2 that are surely there before it ends have the time for a rehearsal.
+  // Where they are many, a rehearsal delays the items (24 sequences of about 2000 tokens: 22.8 us without, 25.2 with it).
+  gd.sure_ctas = se.few ? sm_count() - sel_ctas : 0;
   if (hd == 64) {
-    if (G <= 4) launch_gather<64, 4>(gd, items, gather_ctas, st);
-    else launch_gather<64, 8>(gd, items, gather_ctas, st);
+    if (G <= 4) launch_gather<64, 4>(gd, items, st);
+    else launch_gather<64, 8>(gd, items, st);
   } else {
-    if (G <= 4) launch_gather<128, 4>(gd, items, gather_ctas, st);
-    else launch_gather<128, 8>(gd, items, gather_ctas, st);
+    if (G <= 4) launch_gather<128, 4>(gd, items, st);
+    else launch_gather<128, 8>(gd, items, st);
   }
 }
 

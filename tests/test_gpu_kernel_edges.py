@@ -51,6 +51,16 @@ def test_token_selection_segments(lens, r):
     _attention_case(TINY, lens, r, seed=len(lens), n_sink=3, n_window=2)
 
 
+# Few sequences of long context: the selection holds some SMs, and pass 2 has fewer items than the warps of the others, about as
+# many, and more; rows that keep every token among them, and rows of several segments.
+@pytest.mark.parametrize("hd", [64, 128])
+@pytest.mark.parametrize("lens,r", [([2000] * 4, [250] * 4), ([8000, 7000, 8100, 5], [250, 1000, 500, 1000]), ([8000] * 4, [250] * 4),
+                                    ([16000, 15000, 16384], [500, 500, 1000]), ([20000, 33000], [500, 250])])
+def test_attention_of_few_long_sequences(hd, lens, r):
+    cfg = dict(TINY, head_dim=hd, n_q_heads=8, n_kv_heads=8, d_model=1024)
+    _attention_case(cfg, lens, r, seed=hd + len(lens))
+
+
 def test_attention_of_a_full_batch():
     """More units of the selection and more items of pass 2 than are worked on at once, rows of every length and rate."""
     cfg = dict(TINY, n_q_heads=8, n_kv_heads=8, d_model=512)
