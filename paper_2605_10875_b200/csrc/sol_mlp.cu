@@ -173,8 +173,10 @@ __device__ __forceinline__ void settle_open(const ChanDev& p, SelectSmem& sm, in
 
 // A token whose candidates did not fit the list (long runs of equal scores), from the beginning and for any input, by one
 // CTA: the m-th largest |t| by a radix select, the channels within the error bound of it by their exact scores, or, where
-// those do not fit the list either, in float32 order with ties to the lower index.  Rare, so its loops over the row
-// are short and read it from L2 each time.
+// those do not fit the list either, in float32 order with ties to the lower index.  Its loops over the row are short and read it
+// from L2 each time, so the loads are 16 bytes wide and several in flight; a padding row's scores are all equal and need no radix
+// select (128 rows of a Llama-8B MLP, half of them zeros: 222 us with single floats and the select, this 188; with the row in the
+// registers of 1024 threads, a kernel of 124 registers in every layer's way, 202).
 __device__ __noinline__ void redo_token(const ChanDev& p, SelectSmem& sm, int b) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   constexpr int WARPS = CR_THREADS / 32;
@@ -183,19 +185,38 @@ __device__ __noinline__ void redo_token(const ChanDev& p, SelectSmem& sm, int b)
   const int m = (int)(((long long)(1000 - p.p_permille[b]) * ff + 999) / 1000);
   if (tid < 4) sm.counts[tid] = 0;
   float gmax = 0.f, umax = 0.f;  // for the error window
-#pragma unroll 1
-  for (int j = tid; j < ff; j += CR_THREADS) {
-    gmax = fmaxf(gmax, fabsf(p.g[(size_t)b * ff + j]));
-    umax = fmaxf(umax, fabsf(p.u[(size_t)b * ff + j]));
+  uint32_t key_max = 0u, key_min = 0xffffffffu;
+#pragma unroll 4
+  for (int j = tid * 4; j < ff; j += CR_THREADS * 4) {  // ff is a multiple of 4
+    const float4 g4 = *reinterpret_cast<const float4*>(p.g + (size_t)b * ff + j), u4 = *reinterpret_cast<const float4*>(p.u + (size_t)b * ff + j),
+                 t4 = *reinterpret_cast<const float4*>(tt + j);
+    gmax = fmaxf(fmaxf(gmax, fmaxf(fabsf(g4.x), fabsf(g4.y))), fmaxf(fabsf(g4.z), fabsf(g4.w)));
+    umax = fmaxf(fmaxf(umax, fmaxf(fabsf(u4.x), fabsf(u4.y))), fmaxf(fabsf(u4.z), fabsf(u4.w)));
+    const uint32_t k0 = float_key(fabsf(t4.x)), k1 = float_key(fabsf(t4.y)), k2 = float_key(fabsf(t4.z)), k3 = float_key(fabsf(t4.w));
+    key_max = max(max(key_max, max(k0, k1)), max(k2, k3));
+    key_min = min(min(key_min, min(k0, k1)), min(k2, k3));
   }
   gmax = block_max<CR_THREADS>(gmax, 0, sm);
   umax = block_max<CR_THREADS>(umax, 1, sm);
-  int tie_need = 0;
-  auto key = [&](int i) -> uint32_t {
-    const int j = i * CR_THREADS + tid;
-    return j < ff ? float_key(fabsf(tt[j])) : 0u;
-  };
-  const uint32_t key_thr = select_kth<CR_THREADS, 0>(key, m, tie_need, sm, (ff + CR_THREADS - 1) / CR_THREADS);
+  key_max = __reduce_max_sync(0xffffffffu, key_max);
+  key_min = __reduce_min_sync(0xffffffffu, key_min);
+  if (lane == 0) {
+    sm.rank_key[warp] = key_max;
+    sm.rank_key[WARPS + warp] = key_min;
+  }
+  __syncthreads();
+  key_max = __reduce_max_sync(0xffffffffu, sm.rank_key[lane % WARPS]);
+  key_min = __reduce_min_sync(0xffffffffu, sm.rank_key[WARPS + lane % WARPS]);
+  __syncthreads();  // the scratch is taken by the selection
+  uint32_t key_thr = key_max;
+  int tie_need = m;
+  if (key_min != key_max) {  // not all equal, as the scores of a padding row are
+    auto key = [&](int i) -> uint32_t {
+      const int j = i * CR_THREADS + tid;
+      return j < ff ? float_key(fabsf(tt[j])) : 0u;
+    };
+    key_thr = select_kth<CR_THREADS, 0>(key, m, tie_need, sm, (ff + CR_THREADS - 1) / CR_THREADS);
+  }
   const float thr32 = key_to_float(key_thr);
   // error taken for g_j, u_j: the tensor cores add each 16-long slice of the dot product to the running
   // float32 sum with truncation, so the error grows with the d/16 steps: (d/16) * 2^-24 of the largest
@@ -204,15 +225,35 @@ __device__ __noinline__ void redo_token(const ChanDev& p, SelectSmem& sm, int b)
   const float delta = 2.0f * eps * (1.1f * umax + gmax) + 1e-6f * thr32;  // |silu'| <= 1.1, |silu(g)| <= |g|
   const float hi = thr32 + delta, lo = thr32 - delta;
   int n_in = 0;
-#pragma unroll 1
-  for (int j = tid; j < ff; j += CR_THREADS) {
-    const float sv = key_to_float(float_key(fabsf(tt[j])));
-    if (sv > hi) {
-      ++n_in;
-    } else if (sv >= lo) {
-      const int slot = atomicAdd(&sm.counts[0], 1);
-      if (slot < SEL_CAND_CAP) sm.cand_idx[slot] = j;
+#pragma unroll 2
+  for (int j0 = 0; j0 < ff; j0 += CR_THREADS * 4) {
+    const int j = j0 + tid * 4;
+    float4 t4 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (j < ff) t4 = *reinterpret_cast<const float4*>(tt + j);
+    const float vv[4] = {t4.x, t4.y, t4.z, t4.w};
+    uint32_t in = 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float sv = fabsf(vv[e]);
+      if (j >= ff) continue;
+      if (sv > hi) ++n_in;
+      else if (sv >= lo) in |= 1u << e;
     }
+    int incl = __popc(in);  // the candidates' places: one request per warp
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
+    }
+    int slot = 0;
+    if (lane == 31 && incl) slot = atomicAdd(&sm.counts[0], incl);
+    slot = __shfl_sync(0xffffffffu, slot, 31) + incl - __popc(in);
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      if ((in >> e) & 1u) {
+        if (slot < SEL_CAND_CAP) sm.cand_idx[slot] = j + e;
+        ++slot;
+      }
   }
   n_in = block_count<CR_THREADS>(n_in, 0, sm);
   int n_cand = sm.counts[0];
@@ -374,7 +415,7 @@ struct ChanMultiSmem {
   float thr_hi, thr_lo;
   int idx[CH_CAND_CAP];
   float2 av[CH_CAND_CAP];          // a candidate's float32 |t| and the bound of its error
-  int open[CH_CAND_CAP];           // the candidates to recompute
+  int open[CH_CAND_CAP];           // the channels to recompute
   double val[CH_CAND_CAP];         // their exact |t|
   size_t row_off[CM_EXACT];        // of up to CM_EXACT of them: where their weight rows start, the rows' swizzle,
   int row_swz[CM_EXACT];
@@ -390,7 +431,7 @@ __device__ __forceinline__ void exact_candidates(const ChanDev& p, ChanMultiSmem
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = p.d;
   const uint32_t chunk_bytes = (uint32_t)p.R * 128;
   if (tid < n) {  // where the candidate's gate row starts (its up row follows 128 bytes later)
-    const int row = 2 * sm.idx[sm.open[i0 + tid]], tile = row / p.R, r = row - tile * p.R;
+    const int row = 2 * sm.open[i0 + tid], tile = row / p.R, r = row - tile * p.R;
     sm.row_off[tid] = ((size_t)tile * p.chunks * p.R + r) * 128;
     sm.row_swz[tid] = r & 7;
   }
@@ -679,26 +720,32 @@ __global__ void __launch_bounds__(CM_THREADS, 3) channel_select_multi_kernel(con
       atomicAdd(&sm.n_sure, 1);
       keep_channel(p, b, sm.idx[c]);
     } else {
-      sm.open[atomicAdd(&sm.n_open, 1)] = c;
+      sm.open[atomicAdd(&sm.n_open, 1)] = sm.idx[c];
     }
   }
   __syncthreads();
   const int n_open = sm.n_open, need_open = min(max(need - sm.n_sure, 0), n_open);
   if (tid == 0) p.kept_cnt[b] = m;
   if (p.hand_over > 0 && n_open * d > p.hand_over) {
-    for (int i = tid; i < n_open; i += CM_THREADS) p.cand_idx[(size_t)b * CH_CAND_CAP + i] = sm.idx[sm.open[i]];
+    for (int i = tid; i < n_open; i += CM_THREADS) p.cand_idx[(size_t)b * CH_CAND_CAP + i] = sm.open[i];
     if (tid == 0) sel[CH_OPEN] = ((uint32_t)n_open << 16) | (uint32_t)need_open;
     return;
   }
   if (n_open == 0) return;
 #pragma unroll 1
   for (int i0 = 0; i0 < n_open; i0 += CM_EXACT) exact_candidates(p, sm, b, i0, min(CM_EXACT, n_open - i0));
-  for (int c = tid; c < n_open; c += CM_THREADS) {
-    const double mine = sm.val[c];
-    const int j = sm.idx[sm.open[c]];
+  for (int c0 = 0; c0 < n_open; c0 += CM_THREADS / 4) {  // four threads per channel
+    const int c = c0 + (tid >> 2);
+    const double mine = c < n_open ? sm.val[c] : 0.0;
+    const int j = c < n_open ? sm.open[c] : 0;
     int rank = 0;
-    for (int o = 0; o < n_open; ++o) rank += sm.val[o] > mine || (sm.val[o] == mine && sm.idx[sm.open[o]] < j);
-    if (rank < need_open) keep_channel(p, b, j);
+    for (int o = tid & 3; o < n_open; o += 4) {
+      const double vo = sm.val[o];
+      rank += (vo > mine) || (vo == mine && sm.open[o] < j);
+    }
+    rank += __shfl_xor_sync(0xffffffffu, rank, 1);
+    rank += __shfl_xor_sync(0xffffffffu, rank, 2);
+    if (c < n_open && rank < need_open && (tid & 3) == 0) keep_channel(p, b, j);
   }
   if (tid == 0) atomicAdd(p.status + ST_CH_REFINED, n_open);
 }

@@ -172,7 +172,9 @@ def test_attention_selection_with_nan_keys(T):
 # Exactly equal scores: a row of zeros (a padding row) ranks every channel equal, and so do channels whose up rows are
 # zeros of either sign beside gate rows that are not; denormal weights are smaller than everything but those.  The exact
 # sums have to say so: ties go to the lower index.
-def test_channel_selection_of_scores_that_are_zero():
+# (24 rows: the CTA that lists a token's candidates settles them itself.)
+@pytest.mark.parametrize("copies", [1, 6])
+def test_channel_selection_of_scores_that_are_zero(copies):
     cfg = dict(TINY, d_ff=1024)
     shape, _ = H.make_shapes(cfg)
     ff, d = cfg["d_ff"], cfg["d_model"]
@@ -188,12 +190,13 @@ def test_channel_selection_of_scores_that_are_zero():
     x[2] = x[1]
     x[3] = np.where(np.arange(d) % 2, 0x8000, 0).astype(np.uint16)  # zeros of either sign
     m = [-(-ff * (1000 - p) // 1000) for p in (500, 500, 650, 250)]
-    _, kept, st = H.gpu_mlp(shape, x, H.device_weights(w, shape), [500, 500, 650, 250])
+    _, kept, st = H.gpu_mlp(shape, np.tile(x, (copies, 1)), H.device_weights(w, shape), [500, 500, 650, 250] * copies)
     assert st[0] == 0
     zero = np.sort(zero)
-    assert np.array_equal(kept[0], np.arange(m[0])) and np.array_equal(kept[3], np.arange(m[3]))
-    assert np.array_equal(kept[1], np.sort(np.concatenate([normal, tiny, zero[:m[1] - 400]])))
-    assert len(kept[2]) == m[2] and np.isin(normal, kept[2]).all() and np.isin(kept[2], np.concatenate([normal, tiny])).all()
+    for k in np.arange(4 * copies).reshape(copies, 4):
+        assert np.array_equal(kept[k[0]], np.arange(m[0])) and np.array_equal(kept[k[3]], np.arange(m[3]))
+        assert np.array_equal(kept[k[1]], np.sort(np.concatenate([normal, tiny, zero[:m[1] - 400]])))
+        assert len(kept[k[2]]) == m[2] and np.isin(normal, kept[k[2]]).all() and np.isin(kept[k[2]], np.concatenate([normal, tiny])).all()
 
 
 # Scores of +inf are all kept, more of them than the budget included; the count says what the list holds (rows of one
