@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
     int live = EPI == EPI_SWIGLU ? 0 : 1;
 #pragma unroll 1
     for (;; live = 1) {
-      asm volatile("" : "+r"(live));  // one code for both
+      if constexpr (EPI == EPI_SWIGLU) asm volatile("" : "+r"(live));  // one code for both
       if (live) {
         pdl_wait_hold(p.hold);  // the epilogue reads scales and overwrites buffers earlier kernels used
         if (EPI == EPI_SWIGLU) {
@@ -284,12 +284,10 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
         } else {
           const int n = tile * p.R + r;
           const bool valid = r < p.R && n < p.N;
-          for (int c0 = half * 16; c0 < (live ? p.Mpad : half * 16 + 1) && ok; c0 += 16 * UM_EPI_SETS) {
+          for (int c0 = half * 16; c0 < p.Mpad && ok; c0 += 16 * UM_EPI_SETS) {
             float v[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) v[i] = 0.f;
-            if (live) tmem_ld16(tl + c0, v);
-            if (p.n_b == 2 && live) {  // high-part and low-part products
+            tmem_ld16(tl + c0, v);
+            if (p.n_b == 2) {  // high-part and low-part products
               float w2[16];
               tmem_ld16(tl + p.Mpad + c0, w2);
 #pragma unroll
@@ -298,7 +296,7 @@ __global__ void __launch_bounds__(UM_THREADS, 1) umma_nk_kernel(const NKDev p) {
 #pragma unroll
             for (int i = 0; i < 16; ++i) {
               const int m = c0 + i;
-              if (live && m < p.M && valid) p.out0[((size_t)blockIdx.y * p.M + m) * p.N + n] = v[i];
+              if (m < p.M && valid) p.out0[((size_t)blockIdx.y * p.M + m) * p.N + n] = v[i];
             }
           }
         }
