@@ -28,8 +28,7 @@ def test_down_rows_tiles(B, ff):
 
 
 # The attention's passes at the edges of their tiles: 16-token steps and 64-token pages of the rows that keep every token,
-# 256-token chunks of the scores, rows around one selection segment (8192), runs of several items, forced sets wider than a
-# chunk, in every register layout (head_dim, heads per kv-head).
+# 256-token chunks of the scores, runs of several items, forced sets wider than a chunk, in every register layout (head_dim, heads per kv-head).
 @pytest.mark.parametrize("hd,hq,hkv", [(64, 4, 2), (64, 12, 4), (64, 8, 1), (128, 4, 2), (128, 8, 1), (128, 6, 2)])
 @pytest.mark.parametrize("sink,window", [(0, 1), (5, 300)])
 def test_attention_pass_edges(hd, hq, hkv, sink, window):
@@ -39,10 +38,37 @@ def test_attention_pass_edges(hd, hq, hkv, sink, window):
         _attention_case(cfg, lens, np.resize(rates, len(lens)), seed=seed, n_sink=sink, n_window=window)
 
 
+# Rows around one and two segments of the selection (16384 tokens).
 @pytest.mark.parametrize("hd", [64, 128])
 def test_attention_rows_around_a_selection_segment(hd):
     cfg = dict(TINY, head_dim=hd, n_q_heads=4, n_kv_heads=1, d_model=256)
     _attention_case(cfg, [8191, 8192, 8193, 16385, 40], [125, 500, 250, 1000, 300], seed=hd)
+    _attention_case(cfg, [16383, 16384, 16385, 32768, 32769], [125, 500, 250, 999, 300], seed=hd + 1)
+
+
+# Crowded scores in rows of several segments: keys that are all equal or of three neighbouring values (a bin is split, and there are
+# more between the edges than the list of candidates holds: float32 order, ties to the lower index), and of 128 (the bin is
+# split, its part fits the list).
+@pytest.mark.parametrize("T,r", [(17000, 250), (33000, 500)])
+@pytest.mark.parametrize("values", [1, 3, 128])
+def test_token_selection_of_crowded_scores_over_segments(T, r, values):
+    cfg = dict(TINY, n_q_heads=4, n_kv_heads=1)
+    shape, _ = H.make_shapes(cfg, 0, 1)
+    lens = np.asarray([T], np.int32)
+    k_pool, v_pool, table = H.make_case_kv(cfg, lens, 5)
+    q = synth.make_queries(cfg, 5, 1)
+    group = np.arange(T) % values
+    keys = np.tile(np.sign(synth.bf16_to_f32(k_pool[0, 0, 0])), (values, 1))
+    keys[:, 0] = 1 + np.arange(values) / 128
+    for j in range(values):
+        at = np.flatnonzero(group == j)
+        k_pool[table[0, at // 64], :, at % 64] = synth.to_bf16(keys[j])
+    _, kept, st = H.gpu_attention(shape, q, H.device_kv(k_pool, v_pool, table, lens), [r])
+    score = keys @ synth.bf16_to_f32(q[0]).astype(np.float64).sum(0)
+    k = -(-T * r // 1000)
+    order = np.lexsort((np.arange(T), -score[group]))
+    want = np.sort(np.append(order[order != T - 1][:k - 1], T - 1))  # the newest token is always kept
+    assert st[0] == 0 and np.array_equal(np.asarray(kept[0][0]), want)
 
 
 # The token selection around one segment (16384 tokens) and over several, and more units than CTAs are resident.
@@ -151,14 +177,15 @@ def test_channel_selection_of_crowded_scores(ff, spread):
     H.assert_outputs(out_o, out, "mlp output")
 
 
-# Keys that are not numbers: never kept, and the count says what the list holds (rows of one selection segment and of two).
-@pytest.mark.parametrize("T", [700, 9000])
-def test_attention_selection_with_nan_keys(T):
+# Keys that are not numbers: never kept, and the count says what the list holds (rows of one segment of the selection, of two and
+# of three; the keys in every segment, in the first or the last one, and in all but the first).
+@pytest.mark.parametrize("T,bad", [(700, [3, 64, 200, 650]), (9000, [3, 64, 200, 8950]), (17000, [3, 16383, 16384, 16950]),
+                                   (17000, [5, 200]), (17000, [16500]), (33000, [40, 20000, 32990]), (33000, [16384, 32768])])
+def test_attention_selection_with_nan_keys(T, bad):
     cfg = dict(TINY, n_q_heads=4, n_kv_heads=1)
     shape, _ = H.make_shapes(cfg, 0, 1)
     lens = np.asarray([T], np.int32)
     k_pool, v_pool, table = H.make_case_kv(cfg, lens, 5)
-    bad = [3, 64, 200, T - 50]
     for j in bad:
         k_pool[table[0, j // 64], :, j % 64, :] = 0x7FC0
     kv = H.device_kv(k_pool, v_pool, table, lens)
@@ -199,17 +226,19 @@ def test_channel_selection_of_scores_that_are_zero(copies):
         assert len(kept[k[2]]) == m[2] and np.isin(normal, kept[k[2]]).all() and np.isin(kept[k[2]], np.concatenate([normal, tiny])).all()
 
 
-# Scores of +inf are all kept, more of them than the budget included; the count says what the list holds (rows of one
-# selection segment and of two).
-@pytest.mark.parametrize("T,r,n_inf", [(60, 50, 5), (700, 4, 9), (9000, 1, 20), (700, 10, 4), (700, 1000, 4)])
-def test_attention_selection_with_infinite_scores(T, r, n_inf):
+# Scores of +inf are all kept, more of them than the budget included; the count says what the list holds (rows of one segment of
+# the selection, of two and of three; `first`: the token from which they may lie).
+@pytest.mark.parametrize("T,r,n_inf,first", [(60, 50, 5, 0), (700, 4, 9, 0), (9000, 1, 20, 0), (700, 10, 4, 0), (700, 1000, 4, 0),
+                                             (17000, 1, 30, 0), (17000, 1, 30, 16384), (17000, 250, 5, 16384), (33000, 1, 50, 0),
+                                             (33000, 1, 50, 32768), (33000, 500, 9, 0)])
+def test_attention_selection_with_infinite_scores(T, r, n_inf, first):
     cfg = dict(TINY, n_q_heads=4, n_kv_heads=4)
     shape, _ = H.make_shapes(cfg, 0, 1)
     lens = np.asarray([T], np.int32)
     k_pool, v_pool, table = H.make_case_kv(cfg, lens, 5)
     q = synth.make_queries(cfg, 5, 1)
     huge = np.where(q[0] & 0x8000, 0xFF61, 0x7F61).astype(np.uint16)  # +-2.99e38 with the query's signs
-    inf = np.sort(np.random.default_rng(T).permutation(T - 1)[:n_inf])
+    inf = np.sort(first + np.random.default_rng(T).permutation(T - 1 - first)[:n_inf])
     for j in inf:
         k_pool[table[0, j // 64], :, j % 64, :] = huge
     kv = H.device_kv(k_pool, v_pool, table, lens)
