@@ -761,6 +761,10 @@ int down_chunks(int ff, int d) {
 }
 
 void launch_gemm_down(const GemmDown& g, cudaStream_t st) {
+  if (g.p_permille == nullptr) {
+    record_cuda_error(cudaErrorInvalidValue, "down projection without prune rates");
+    return;
+  }
   if (g.M <= DR_MAXB && g.t_f32 != nullptr && g.keep != nullptr) {  // small batch: channel by channel, only kept rows
     DownRowsDev r;
     r.M = g.M; r.Mpad = pad_rows(g.M); r.ff = g.ff; r.d = g.d; r.chunks = g.chunks;

@@ -181,7 +181,8 @@ struct GemmDown {
   const void* t;     // packed masked activations: 2 Mpad rows (high parts, then low parts), K = ff
   const float* t_f32;         // [M][ff] unmasked t and
   const unsigned char* keep;  // [M][ff] keep mask: the small-batch kernel reads these instead of the packed operand
-  const int32_t* p_permille;  // [M] prune rates (small-batch kernel)
+  const int32_t* p_permille;  // [M] prune rates, required; both kernels read them ahead of their wait for the kernels before, so they
+                              // are complete when the call's second kernel starts (an input, or written by a plain launch ahead)
   const void* w;     // packed W_down_t
   const int32_t* live;  // [ff/32] non-zero if any token keeps a channel of the granule
   int M, ff, d;
