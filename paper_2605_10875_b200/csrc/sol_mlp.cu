@@ -761,8 +761,7 @@ __global__ void __launch_bounds__(THREADS) channel_list_kernel(const unsigned ch
   pdl_wait();
   const int b = blockIdx.x, j0 = threadIdx.x * KPT;
   const unsigned char* k = keep + (size_t)b * ff;
-  auto klass = [&](int i) -> int { return (j0 + i < ff && k[j0 + i]) ? 2 : 0; };
-  compact_indices<THREADS, KPT>(klass, [](int, bool, int) {}, 0, kept_ch + (size_t)b * ff, sm, KPT);
+  compact_indices<THREADS, KPT>([&](int i) { return j0 + i < ff && k[j0 + i] != 0; }, kept_ch + (size_t)b * ff, sm);
 }
 
 void launch_channel_select(const ChannelSelectArgs& a, cudaStream_t st) {

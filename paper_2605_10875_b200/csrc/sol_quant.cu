@@ -71,7 +71,7 @@ norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, i
   }
   const int width = bits ? __ldcg(bits + row) : 16;
   // a bf16 row without partial sums is an input of the call: that kernel is the first one, or the stand-alone quantizer
-  constexpr bool REHEARSE = PART || GATE || IN_F32;
+  constexpr bool REHEARSE = PART || IN_F32;
   int live = !REHEARSE || first ? 1 : 0;
 #pragma unroll 1
   for (;; live = 1) {
@@ -328,9 +328,9 @@ void launch_norm_quant(const NormQuantArgs& a, cudaStream_t st) {
     if (a.part != nullptr) SOL_NQ_BY_SIZE(F32, GATE, true); \
     else SOL_NQ_BY_SIZE(F32, GATE, false);                  \
   } while (0)
-  if (a.gate_p_permille != nullptr) {
-    if (a.in_f32) SOL_NQ_BY_PART(true, true);
-    else SOL_NQ_BY_PART(false, true);
+  if (a.gate_p_permille != nullptr) {  // the second RMSNorm of a layer: always with the partial sums of the output projection
+    if (a.in_f32) SOL_NQ_BY_SIZE(true, true, true);
+    else SOL_NQ_BY_SIZE(false, true, true);
   } else {
     if (a.in_f32) SOL_NQ_BY_PART(true, false);
     else SOL_NQ_BY_PART(false, false);

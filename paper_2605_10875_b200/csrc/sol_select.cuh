@@ -272,76 +272,27 @@ __device__ __forceinline__ void rank_candidates(int n_cand, int need, Smem& sm) 
   }
 }
 
-// klass(i) in {0 dropped, 1 tie, 2 kept} for element j = first + tid*per_thread + i, i < per_thread (called
-// twice per element).  Ties
-// are kept in ascending index order until tie_need runs out.  Kept indices go to out[] ascending;
-// emit(i, keep, pos) reports the final decision of every element and, for a kept one, its place in out[].  Returns the kept total to every thread.
-// All threads call; uses sm.scan.
-template <int THREADS, int KPT, typename ClassFn, typename EmitFn, typename Smem>
-__device__ __forceinline__ int compact_counted(int c2, int c1, ClassFn klass, EmitFn emit, int tie_need, int32_t* out,
-                                               Smem& sm, int per_thread, int first = 0);
-
-template <int THREADS, int KPT, typename ClassFn, typename EmitFn, typename Smem>
-__device__ __forceinline__ int compact_indices(ClassFn klass, EmitFn emit, int tie_need, int32_t* out, Smem& sm,
-                                               int per_thread, int first = 0) {
-  int c2 = 0, c1 = 0;
-  for_keys<KPT>(per_thread, [&](int i) {
-    const int c = klass(i);
-    c2 += c == 2;
-    c1 += c == 1;
-  });
-  return compact_counted<THREADS, KPT>(c2, c1, klass, emit, tie_need, out, sm, per_thread, first);
-}
-
-// The same when the caller already knows how many of its elements are of class 2 (c2) and 1 (c1).
-template <int THREADS, int KPT, typename ClassFn, typename EmitFn, typename Smem>
-__device__ __forceinline__ int compact_counted(int c2, int c1, ClassFn klass, EmitFn emit, int tie_need, int32_t* out,
-                                               Smem& sm, int per_thread, int first) {
-  constexpr int WARPS = THREADS / 32;
+// Writes the elements j = tid * KPT + i (i < KPT) with keep(i) to out[], ascending (keep is called twice per element).  All
+// threads call; uses sm.scan.
+template <int THREADS, int KPT, typename KeepFn, typename Smem>
+__device__ __forceinline__ void compact_indices(KeepFn keep, int32_t* out, Smem& sm) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // exclusive prefix of ties over the block (threads in index order), then of kept elements
-  int t_incl = c1;
+  int mine = 0;
+#pragma unroll
+  for (int i = 0; i < KPT; ++i) mine += keep(i) ? 1 : 0;
+  int incl = mine;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, t_incl, o);
-    if (lane >= o) t_incl += v;
+    const int v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
   }
-  __syncthreads();  // earlier readers of sm.scan are done
-  if (lane == 31) sm.scan[0][warp] = t_incl;
+  if (lane == 31) sm.scan[0][warp] = incl;
   __syncthreads();
-  int t_before = t_incl - c1;
-  for (int w = 0; w < warp; ++w) t_before += sm.scan[0][w];
-  const int my_ties = min(max(tie_need - t_before, 0), c1);
-  const int mine = c2 + my_ties;
-  int k_incl = mine;
+  int pos = incl - mine;
+  for (int w = 0; w < warp; ++w) pos += sm.scan[0][w];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int v = __shfl_up_sync(0xffffffffu, k_incl, o);
-    if (lane >= o) k_incl += v;
-  }
-  if (lane == 31) sm.scan[1][warp] = k_incl;
-  __syncthreads();
-  int pos = k_incl - mine, total = 0;
-  for (int w = 0; w < WARPS; ++w) {
-    const int v = sm.scan[1][w];
-    if (w < warp) pos += v;
-    total += v;
-  }
-  int ties_left = my_ties;
-  const int j0 = first + threadIdx.x * per_thread;
-  for_keys<KPT>(per_thread, [&](int i) {
-    const int c = klass(i);
-    bool kp = c == 2;
-    if (c == 1 && ties_left > 0) {
-      kp = true;
-      --ties_left;
-    }
-    if (kp) out[pos] = j0 + i;
-    emit(i, kp, pos);
-    if (kp) ++pos;
-  });
-  __syncthreads();  // sm.scan may be reused by the caller
-  return total;
+  for (int i = 0; i < KPT; ++i)
+    if (keep(i)) out[pos++] = (int)threadIdx.x * KPT + i;
 }
 
 }  // namespace sol
