@@ -43,9 +43,10 @@ struct NoSmem {
 // reads nothing that an earlier kernel writes and writes nothing), so that it is in the instruction caches.
 // In the chain, per launch: a single sequence 4.9 us, this 3.3; 24 to 32 sequences 7.3 and 5.5; with the input gating 16.5
 // and 12.1.
-// PART: the row comes with the partial sums of a projection.  Their loads in flight take up to 200 registers, one CTA per SM,
-// which a layer's 128 rows fit; the stand-alone quantizer takes any number of rows and has none (26 to 64 registers; a call
-// of thousands of rows took 29 us with the registers of the partial sums, 9 without).
+// PART: the row comes with the partial sums of a projection.  Their loads in flight take 110 to 199 registers (219 to 255 with the
+// gating), one CTA per SM, which a layer's 128 rows fit; on an SM that holds a row the projections around it find no room.  The
+// stand-alone quantizer takes any number of rows and has none of that (26 to 64 registers; 4096 rows of 2048 elements 14 us, of
+// 4096 elements 25.5; with the partial sums' registers a call of thousands of rows took three times as long).
 template <bool IN_F32, bool GATE, int NV, bool PART>
 __global__ void __launch_bounds__(NQ_THREADS)
 norm_quant_kernel(const void* __restrict__ in, const float* __restrict__ part, int ksplit, size_t part_stride,
